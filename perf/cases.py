@@ -160,7 +160,7 @@ class _Stream:
         rng = np.random.default_rng(9)  # the sessions' sizes belong to the case, their problems to the seed
         self.server = N.Server(slots=SLOTS, cluster=CLUSTER, threads=THREADS, max_nodes=case["n_max"] + 1,
                                max_boxes=30)
-        self.sids, self.ticks, self.rows, total = [], [[], []], [], 0
+        self.sids, self.ticks, rows, total = [], [[], []], [], 0
         for k in range(case["sessions"]):
             n = int(rng.integers(case["n_min"], case["n_max"] + 1))
             pb = serving.session_problem(seed * 1000 + k, n)
@@ -170,19 +170,22 @@ class _Stream:
             for tick in self.ticks:
                 tick.append(mover.step())
             self.sids.append(sid)
-            self.rows.append((total, total + pb.N))
+            rows.append(total)
             total += pb.N
         self.parent = torch.zeros(2, total, dtype=torch.int32, device="cuda")
         self.cost = torch.zeros(2, total, dtype=torch.float32, device="cuda")
+        # each request as the loop sends it: session, request id, boxes, where its tree goes
+        s = case["sessions"]
+        self.requests = [[(self.sids[k], t * s + k, *self.ticks[t][k], self.parent[t].data_ptr() + 4 * rows[k],
+                           self.cost[t].data_ptr() + 4 * rows[k]) for k in range(s)] for t in range(2)]
 
     def run(self):
         s = len(self.sids)
         goal, path_cost, checks = np.zeros(2 * s, np.int32), np.zeros(2 * s, np.float32), np.zeros(2 * s, np.int64)
         edges, status = np.zeros(2 * s, np.int64), np.zeros(2 * s, np.int32)
-        for t, boxes in enumerate(self.ticks):
-            for k, (sid, (lo, hi), (a, _)) in enumerate(zip(self.sids, boxes, self.rows)):
-                self.server.submit(sid, t * s + k, lo, hi, self.parent[t].data_ptr() + 4 * a,
-                                   self.cost[t].data_ptr() + 4 * a)
+        for requests in self.requests:
+            for request in requests:
+                self.server.submit(*request)
             done = 0
             while done < s:
                 for r in self.server.poll(s, 100):
