@@ -125,6 +125,7 @@ struct gmt_graph {
     int* grid_start = nullptr;     size_t cap_grid_start = 0;
     int* grid_list = nullptr;      size_t cap_grid_list = 0;
     int* grid_big = nullptr;       size_t cap_grid_big = 0;
+    float4* grid_packed = nullptr; size_t cap_grid_packed = 0;
     int* halton = nullptr;         size_t cap_halton = 0;    // multi-block Halton sampler scratch (ints)
     // plan workspace
     float* ocost = nullptr;        size_t cap_ocost = 0;
@@ -176,7 +177,7 @@ struct gmt_graph {
         void* dev[] = {X, is_goal, out_row, in_row_own, counts, out_col, out_cost, in_col_own,
                        in_cost_own, out_tau, in_tau, in_path, mask, maskT, tile_cnt, elist, epath, wpre, wpreT,
                        cell_of, cell_sorted, cell_cnt,
-                       cell_start, grid_cnt, grid_start, grid_list, grid_big, halton, ocost, stamp,
+                       cell_start, grid_cnt, grid_start, grid_list, grid_big, grid_packed, halton, ocost, stamp,
                        lists, ctl};
         for (void* p : dev)
             if (p) cudaFree(p);
@@ -271,6 +272,10 @@ cudaError_t build_box_grid(gmt_graph* g, const BoxArgs& boxes, BoxGridArgs* gr, 
     if ((e = grow(&g->grid_start, &g->cap_grid_start, cells + 1)) != cudaSuccess) return e;
     if ((e = grow(&g->grid_list, &g->cap_grid_list, B * kBoxGridMaxCells)) != cudaSuccess) return e;
     if ((e = grow(&g->grid_big, &g->cap_grid_big, B)) != cudaSuccess) return e;
+    const bool packed = g->dp <= 3 && boxes.count <= kBoxGridPackMax;
+    if (packed && (e = grow(&g->grid_packed, &g->cap_grid_packed, B * kBoxGridMaxCells * (g->dp == 2 ? 1 : 2))) !=
+                      cudaSuccess)
+        return e;
     gr->use = 1;
     gr->g = G;
     for (int k = 0; k < 2; ++k) {
@@ -279,11 +284,11 @@ cudaError_t build_box_grid(gmt_graph* g, const BoxArgs& boxes, BoxGridArgs* gr, 
     }
     gr->start = g->grid_start;
     gr->list = g->grid_list;
+    gr->packed = packed ? g->grid_packed : nullptr;
     gr->big = g->grid_big;
     gr->nbig = g->grid_cnt + cells;
-    if ((e = cudaMemsetAsync(g->grid_cnt, 0, (cells + 1) * sizeof(int), st)) != cudaSuccess) return e;
-    return launch_box_grid(g->dp, boxes, *gr, g->grid_cnt, g->grid_start, g->grid_list, g->grid_big,
-                           g->grid_cnt + cells, st);
+    return launch_box_grid(g->dp, boxes, *gr, g->grid_cnt, g->grid_start, g->grid_list,
+                           packed ? g->grid_packed : nullptr, g->grid_big, g->grid_cnt + cells, st);
 }
 }  // namespace
 
@@ -664,18 +669,12 @@ gmt_status gmt_plan(gmt_graph* g, const gmt_boxes* boxes, const gmt_params* para
     }
 
     int blocks = g->plan_blocks, threads = g->plan_threads, cluster = g->plan_cluster;
-    if (blocks <= 0 && cluster <= 0 && threads <= 0 && g->kind == GMT_COST_EUCLID && g->dp == 2 && N <= 2049) {
-        // small 2D graphs: one CTA with the wavefront state in shared memory
-        // (measured 10-15% faster than a cluster up to about 2k nodes; slower
-        // beyond, and for 3D, double-integrator and Dubins graphs, whose
-        // iterations carry more work than one SM issues quickly)
-        blocks = 1;
-        threads = 1024;
-    }
     if (blocks <= 0 && cluster <= 0) {
-        // automatic: the largest resident thread-block cluster (hardware
-        // barriers; measured fastest on GB300 for N from 1e3 to 4e3), else a
-        // cooperative grid of one CTA per SM
+        // automatic: the largest resident thread-block cluster (measured
+        // fastest on GB300 at every size; CTAs of 512 threads up to 2048 nodes,
+        // where idle warps cost more than they carry: 2D n = 1024 0.107 ms
+        // against 0.116 with 1024 threads and 0.142 on one CTA, equal at 4096),
+        // else a cooperative grid of one CTA per SM
         if (g->auto_cluster < 0) g->auto_cluster = plan_max_cluster(g->kind, g->dp, N <= 2048 ? 512 : 1024);
         cluster = g->auto_cluster;
         if (threads <= 0) threads = N <= 2048 ? 512 : 1024;

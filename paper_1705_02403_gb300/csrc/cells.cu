@@ -59,11 +59,19 @@ __global__ void __launch_bounds__(256) box_grid_count_kernel(BoxArgs boxes, int 
         for (int cx = c0[0]; cx <= c1[0]; ++cx) atomicAdd(&cnt[cy * grid.g + cx], 1);
 }
 
+// Entry t of the grid's list is box b (and its packed copy, in 2D and 3D).
+__device__ __forceinline__ void box_grid_put(const BoxArgs& boxes, int dp, int b, int t, int* list, float4* packed) {
+    list[t] = b;
+    if (!packed) return;
+    if (dp == 2) pack_box<2>(packed, boxes.lo, boxes.hi, b, t);
+    else pack_box<3>(packed, boxes.lo, boxes.hi, b, t);
+}
+
 // One thread per box: writes it into each of its cells' lists (cnt counts
 // back down to 0).
 __global__ void __launch_bounds__(256) box_grid_scatter_kernel(BoxArgs boxes, int dp, BoxGridArgs grid,
                                                                const int* __restrict__ start, int* __restrict__ cnt,
-                                                               int* __restrict__ list) {
+                                                               int* __restrict__ list, float4* __restrict__ packed) {
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= boxes.count) return;
     int c0[2], c1[2];
@@ -73,18 +81,101 @@ __global__ void __launch_bounds__(256) box_grid_scatter_kernel(BoxArgs boxes, in
     for (int cy = c0[1]; cy <= c1[1]; ++cy)
         for (int cx = c0[0]; cx <= c1[0]; ++cx) {
             const int c = cy * grid.g + cx;
-            list[start[c] + atomicSub(&cnt[c], 1) - 1] = b;
+            box_grid_put(boxes, dp, b, start[c] + atomicSub(&cnt[c], 1) - 1, list, packed);
         }
 }
 
+// The whole grid by one block, its cell counts in shared memory: a plan with
+// many boxes builds it before the wavefront (and a build before sampling), so
+// three dependent launches and a memset cost more than the work (1500 boxes:
+// 18.5 us of kernels in a row before).
+__global__ void __launch_bounds__(1024) box_grid_block_kernel(BoxArgs boxes, int dp, BoxGridArgs grid,
+                                                              int* __restrict__ start, int* __restrict__ list,
+                                                              float4* __restrict__ packed, int* __restrict__ big,
+                                                              int* __restrict__ nbig) {
+    __shared__ int cnt[64 * 64];
+    __shared__ int warp_sum[32];
+    __shared__ int s_big;
+    const int cells = grid.g * grid.g, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    for (int c = tid; c < 64 * 64; c += 1024) cnt[c] = 0;
+    if (tid == 0) s_big = 0;
+    __syncthreads();
+    for (int b = tid; b < boxes.count; b += 1024) {
+        int c0[2], c1[2];
+        box_grid_range(grid, boxes.lo + (size_t)b * dp, boxes.hi + (size_t)b * dp, c0, c1);
+        if (c0[0] > c1[0] || c0[1] > c1[1]) continue;  // lo > hi: the box holds no point
+        if ((c1[0] - c0[0] + 1) * (c1[1] - c0[1] + 1) > kBoxGridMaxCells) {
+            big[atomicAdd(&s_big, 1)] = b;
+            continue;
+        }
+        for (int cy = c0[1]; cy <= c1[1]; ++cy)
+            for (int cx = c0[0]; cx <= c1[0]; ++cx) atomicAdd(&cnt[cy * grid.g + cx], 1);
+    }
+    __syncthreads();
+    // exclusive prefix of the counts, four consecutive cells per thread
+    int v[4], sum = 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        v[k] = cnt[4 * tid + k];
+        sum += v[k];
+    }
+    int incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+    }
+    if (lane == 31) warp_sum[warp] = incl;
+    __syncthreads();
+    if (warp == 0) {
+        int w = warp_sum[lane];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, w, o);
+            if (lane >= o) w += y;
+        }
+        warp_sum[lane] = w;
+    }
+    __syncthreads();
+    int at = (warp > 0 ? warp_sum[warp - 1] : 0) + incl - sum;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int c = 4 * tid + k;
+        cnt[c] = at;  // from here on the cell's next free entry
+        if (c < cells) start[c] = at;
+        at += v[k];
+    }
+    if (tid == 1023) {
+        start[cells] = at;  // the cells past the grid's are empty
+        *nbig = s_big;
+    }
+    __syncthreads();
+    for (int b = tid; b < boxes.count; b += 1024) {
+        int c0[2], c1[2];
+        box_grid_range(grid, boxes.lo + (size_t)b * dp, boxes.hi + (size_t)b * dp, c0, c1);
+        if (c0[0] > c1[0] || c0[1] > c1[1]) continue;
+        if ((c1[0] - c0[0] + 1) * (c1[1] - c0[1] + 1) > kBoxGridMaxCells) continue;
+        for (int cy = c0[1]; cy <= c1[1]; ++cy)
+            for (int cx = c0[0]; cx <= c1[0]; ++cx)
+                box_grid_put(boxes, dp, b, atomicAdd(&cnt[cy * grid.g + cx], 1), list, packed);
+    }
+}
+
 cudaError_t launch_box_grid(int dp, BoxArgs boxes, const BoxGridArgs& grid, int* cnt, int* start, int* list,
-                            int* big, int* nbig, cudaStream_t st) {
-    if (dp < 2 || boxes.count < 1) return cudaErrorInvalidValue;
+                            float4* packed, int* big, int* nbig, cudaStream_t st) {
+    if (dp < 2 || boxes.count < 1 || grid.g > 64) return cudaErrorInvalidValue;
+    if (boxes.count <= kBoxGridBlockMax) {
+        box_grid_block_kernel<<<1, 1024, 0, st>>>(boxes, dp, grid, start, list, packed, big, nbig);
+        return cudaGetLastError();
+    }
+    cudaError_t me = cudaMemsetAsync(cnt, 0, (size_t)grid.g * grid.g * sizeof(int), st);
+    if (me == cudaSuccess) me = cudaMemsetAsync(nbig, 0, sizeof(int), st);
+    if (me != cudaSuccess) return me;
     const unsigned blocks = (unsigned)((boxes.count + 255) / 256);
     box_grid_count_kernel<<<blocks, 256, 0, st>>>(boxes, dp, grid, cnt, big, nbig);
     cudaError_t e = launch_scan(cnt, start, grid.g * grid.g, st);
     if (e != cudaSuccess) return e;
-    box_grid_scatter_kernel<<<blocks, 256, 0, st>>>(boxes, dp, grid, start, cnt, list);
+    box_grid_scatter_kernel<<<blocks, 256, 0, st>>>(boxes, dp, grid, start, cnt, list, packed);
     return cudaGetLastError();
 }
 

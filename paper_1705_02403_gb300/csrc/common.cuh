@@ -56,6 +56,16 @@ __device__ __forceinline__ Ctr4 philox4x32_10(Ctr4 c, uint32_t k0, uint32_t k1) 
     return c;
 }
 
+// Position of the m-th (from 0) set bit of x (x has more than m set bits):
+// the largest p with fewer than m + 1 set bits below it, by binary search.
+__device__ __forceinline__ int select_bit(uint32_t x, int m) {
+    int p = 0;
+#pragma unroll
+    for (int step = 16; step > 0; step >>= 1)
+        if (__popc(x & ((1u << (p + step)) - 1u)) <= m) p += step;
+    return p;
+}
+
 // Top 24 bits of a word scaled by 2^-24: exact, in [0, 1).
 __device__ __forceinline__ float unit_float(uint32_t w) { return (float)(w >> 8) * 0x1p-24f; }
 
@@ -70,25 +80,77 @@ __device__ __forceinline__ bool in_box(const float* p, const float* lo, const fl
     return inside;
 }
 
-// Does p lie in one of the boxes b0 + i, i a set bit of `near`?  Four boxes per
-// step with every comparison evaluated (no short circuit), so their loads
-// issue together; the answer is that of testing them one by one.
+// The obstacles of a plan's checks: `packed` (boxes staged in shared memory,
+// lo then hi in kQ float4s each, so a box takes two 16-byte loads in 3D
+// instead of six scalar ones) or, when NULL, the caller's arrays.
 template <int DP>
-__device__ __forceinline__ bool in_near_boxes(const float* p, const float* lo, const float* hi, int b0,
-                                              unsigned near) {
+struct BoxSet {
+    static constexpr int kQ = (2 * DP + 3) / 4;
+    const float4* packed;
+    const float* lo;
+    const float* hi;
+    int count;
+    __device__ __forceinline__ void load(int b, float* l, float* h) const {
+        if (packed) {
+            float v[4 * kQ];
+#pragma unroll
+            for (int k = 0; k < kQ; ++k) {
+                const float4 f = packed[b * kQ + k];
+                v[4 * k] = f.x; v[4 * k + 1] = f.y; v[4 * k + 2] = f.z; v[4 * k + 3] = f.w;
+            }
+#pragma unroll
+            for (int a = 0; a < DP; ++a) { l[a] = v[a]; h[a] = v[DP + a]; }
+        } else {
+#pragma unroll
+            for (int a = 0; a < DP; ++a) { l[a] = lo[b * DP + a]; h[a] = hi[b * DP + a]; }
+        }
+    }
+    // Does p lie in box b?  Every comparison evaluated, no short circuit.
+    __device__ __forceinline__ bool holds(int b, const float* p) const {
+        float l[DP], h[DP];
+        load(b, l, h);
+        bool in = true;
+#pragma unroll
+        for (int a = 0; a < DP; ++a) in = in & (l[a] <= p[a]) & (p[a] <= h[a]);
+        return in;
+    }
+    // Does box b meet [plo, phi] (closed intervals on all axes)?
+    __device__ __forceinline__ bool meets(int b, const float* plo, const float* phi) const {
+        float l[DP], h[DP];
+        load(b, l, h);
+        bool m = true;
+#pragma unroll
+        for (int a = 0; a < DP; ++a) m = m & (l[a] <= phi[a]) & (plo[a] <= h[a]);
+        return m;
+    }
+};
+
+// Packs boxes lo[], hi[] ([count][DP]) as BoxSet reads them, one thread per
+// box entry.
+template <int DP>
+__device__ __forceinline__ void pack_box(float4* packed, const float* lo, const float* hi, int from, int to) {
+    constexpr int kQ = BoxSet<DP>::kQ;
+    float v[4 * kQ] = {};
+#pragma unroll
+    for (int a = 0; a < DP; ++a) { v[a] = lo[(size_t)from * DP + a]; v[DP + a] = hi[(size_t)from * DP + a]; }
+#pragma unroll
+    for (int k = 0; k < kQ; ++k) packed[(size_t)to * kQ + k] = make_float4(v[4 * k], v[4 * k + 1], v[4 * k + 2], v[4 * k + 3]);
+}
+
+// Does p lie in one of the boxes b0 + i, i a set bit of `near`?  Four boxes per
+// step, so their loads issue together; the answer is that of testing them one
+// by one.
+template <int DP>
+__device__ __forceinline__ bool in_near_boxes(const float* p, const BoxSet<DP>& B, int b0, unsigned near) {
     bool hit = false;
     for (unsigned w = near; w;) {
         const int first = b0 + __ffs(w) - 1;
         bool h = false;
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            const bool valid = w != 0u;
-            const int b = valid ? b0 + __ffs(w) - 1 : first;
+            const int b = w != 0u ? b0 + __ffs(w) - 1 : first;  // past the last: the first again
             w &= w - 1u;
-            bool inside = valid;
-#pragma unroll
-            for (int a = 0; a < DP; ++a) inside = inside & (lo[b * DP + a] <= p[a]) & (p[a] <= hi[b * DP + a]);
-            h = h | inside;
+            h = h | B.holds(b, p);
         }
         hit = hit | h;
     }
@@ -108,15 +170,42 @@ __device__ __forceinline__ int box_grid_cell(const BoxGridArgs& g, float x, int 
     return min(max(k, 0), g.g - 1);
 }
 
+// Box t of the grid's list holds p: through the packed copies in list order
+// when the grid has them (one or two 16-byte loads, no index to follow).
+template <int DP>
+__device__ __forceinline__ bool grid_entry_holds(const float* p, const float* blo, const float* bhi,
+                                                 const BoxGridArgs& grid, int t) {
+    if ((DP == 2 || DP == 3) && grid.packed) {
+        constexpr int kQ = BoxSet<DP>::kQ;
+        float v[4 * kQ];
+#pragma unroll
+        for (int k = 0; k < kQ; ++k) {
+            const float4 f = __ldg(&grid.packed[(size_t)t * kQ + k]);
+            v[4 * k] = f.x; v[4 * k + 1] = f.y; v[4 * k + 2] = f.z; v[4 * k + 3] = f.w;
+        }
+        bool in = true;
+#pragma unroll
+        for (int a = 0; a < DP; ++a) in = in & (v[a] <= p[a]) & (p[a] <= v[DP + a]);
+        return in;
+    }
+    return in_box<DP>(p, blo, bhi, __ldg(&grid.list[t]));
+}
+
 // Does point p lie in a box?  With the grid, only the boxes listed in p's
-// cell and the big boxes can hold it; each is tested exactly.  One thread.
+// cell and the big boxes can hold it; each is tested exactly, four per step
+// (their loads issue together: a cell of a finely sliced obstacle lists tens
+// of boxes, and one box per step is a chain of load latencies).  One thread.
 template <int DP>
 __device__ __forceinline__ bool in_any_box_grid(const float* p, const float* blo, const float* bhi,
                                                 const BoxGridArgs& grid) {
     const int c = box_grid_cell(grid, p[1], 1) * grid.g + box_grid_cell(grid, p[0], 0);
     const int e = __ldg(&grid.start[c + 1]);
-    for (int t = __ldg(&grid.start[c]); t < e; ++t)
-        if (in_box<DP>(p, blo, bhi, __ldg(&grid.list[t]))) return true;
+    for (int t = __ldg(&grid.start[c]); t < e; t += 4) {
+        bool h = false;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) h = h | grid_entry_holds<DP>(p, blo, bhi, grid, min(t + u, e - 1));
+        if (h) return true;
+    }
     const int nb = __ldg(grid.nbig);
     for (int t = 0; t < nb; ++t)
         if (in_box<DP>(p, blo, bhi, __ldg(&grid.big[t]))) return true;
@@ -328,16 +417,20 @@ __device__ __forceinline__ bool di_bern_may_connect(const float* s0, const float
 //   p = ((h00 p0 + (h10 tau) v0) + h01 p1) + (h11 tau) v1,
 //   h00 = (2 s^3 - 3 s^2) + 1, h10 = (s^3 - 2 s^2) + s, h01 = 3 s^2 - 2 s^3,
 //   h11 = s^3 - s^2, s^2 = s s, s^3 = s^2 s.
-__device__ __forceinline__ void hermite_point(const float* s0, const float* s1, float tau, float s, float* p) {
+// The basis (h00, h10, h01, h11) depends on s alone: the same for point k of
+// every edge, so a kernel may keep it in a table.
+__device__ __forceinline__ float4 hermite_basis(float s) {
     const float s2 = s * s;
     const float s3 = s2 * s;
-    const float h00 = (2.0f * s3 - 3.0f * s2) + 1.0f;
-    const float h10 = (s3 - 2.0f * s2) + s;
-    const float h01 = 3.0f * s2 - 2.0f * s3;
-    const float h11 = s3 - s2;
-    const float h10t = h10 * tau, h11t = h11 * tau;
+    return make_float4((2.0f * s3 - 3.0f * s2) + 1.0f, (s3 - 2.0f * s2) + s, 3.0f * s2 - 2.0f * s3, s3 - s2);
+}
+__device__ __forceinline__ void hermite_point(const float* s0, const float* s1, float tau, const float4& h, float* p) {
+    const float h10t = h.y * tau, h11t = h.w * tau;
 #pragma unroll
-    for (int a = 0; a < 3; ++a) p[a] = ((h00 * s0[a] + h10t * s0[3 + a]) + h01 * s1[a]) + h11t * s1[3 + a];
+    for (int a = 0; a < 3; ++a) p[a] = ((h.x * s0[a] + h10t * s0[3 + a]) + h.z * s1[a]) + h11t * s1[3 + a];
+}
+__device__ __forceinline__ void hermite_point(const float* s0, const float* s1, float tau, float s, float* p) {
+    hermite_point(s0, s1, tau, hermite_basis(s), p);
 }
 
 // ---------------------------------------------------------------------------

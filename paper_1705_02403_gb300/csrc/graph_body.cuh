@@ -119,7 +119,7 @@ __device__ __forceinline__ bool point_in_boxes_group(const float* p, const BoxAr
     if (grid.use) {
         const int c = box_grid_cell(grid, p[1], 1) * grid.g + box_grid_cell(grid, p[0], 0);
         const int e = __ldg(&grid.start[c + 1]);
-        for (int t = __ldg(&grid.start[c]) + sub; t < e; t += G) hit |= in_box<DP>(p, boxes.lo, boxes.hi, __ldg(&grid.list[t]));
+        for (int t = __ldg(&grid.start[c]) + sub; t < e; t += G) hit |= grid_entry_holds<DP>(p, boxes.lo, boxes.hi, grid, t);
         const int nb = __ldg(grid.nbig);
         for (int t = sub; t < nb; t += G) hit |= in_box<DP>(p, boxes.lo, boxes.hi, __ldg(&grid.big[t]));
     } else {
@@ -537,16 +537,6 @@ __device__ __forceinline__ void tile_prefix_row(int* __restrict__ tile_cnt, int 
             acc += c[u];
         }
     }
-}
-
-// Position of the m-th (from 0) set bit of x (x has more than m set bits):
-// the largest p with fewer than m + 1 set bits below it, by binary search.
-__device__ __forceinline__ int select_bit(uint32_t x, int m) {
-    int p = 0;
-#pragma unroll
-    for (int step = 16; step > 0; step >>= 1)
-        if (__popc(x & ((1u << (p + step)) - 1u)) <= m) p += step;
-    return p;
 }
 
 template <int D>

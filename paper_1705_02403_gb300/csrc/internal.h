@@ -51,6 +51,7 @@ struct BoxGridArgs {
     float lo[2], inv_h[2];
     const int* start;   // [g * g + 1] first list entry of each cell
     const int* list;    // box indices, grouped by cell
+    const float4* packed;  // 2D/3D: the boxes of `list` in its order (lo then hi, one or two float4s), or NULL
     const int* big;     // indices of the boxes over more than kBoxGridMaxCells cells
     const int* nbig;    // [1] their count
 };
@@ -64,10 +65,18 @@ inline int box_grid_cells(int count) {
     while (g < 64 && g * g < count) g *= 2;
     return g;
 }
-// Builds the grid: cnt [g*g] and nbig [1] must be zeroed; start [g*g + 1],
-// list [count * kBoxGridMaxCells], big [count].
+// Boxes up to which one block builds the grid in one launch (each of its
+// threads then takes at most eight); more boxes take count, scan and scatter
+// launches over the whole chip.
+constexpr int kBoxGridBlockMax = 8192;
+// Boxes up to which the list also keeps packed copies (2D and 3D; at most
+// kBoxGridMaxCells copies of 32 bytes per box).
+constexpr int kBoxGridPackMax = 65536;
+// Builds the grid: cnt [g*g], nbig [1], start [g*g + 1],
+// list [count * kBoxGridMaxCells], packed [as many entries of 1 (2D) or 2 (3D)
+// float4s] or NULL, big [count].
 cudaError_t launch_box_grid(int dp, BoxArgs boxes, const BoxGridArgs& grid, int* cnt, int* start, int* list,
-                            int* big, int* nbig, cudaStream_t st);
+                            float4* packed, int* big, int* nbig, cudaStream_t st);
 
 // Flags written by the sampling kernel.
 enum { kSampleBadInit = 1, kSampleExhausted = 2, kSampleBadAppend = 4, kSampleTimeout = 8 };

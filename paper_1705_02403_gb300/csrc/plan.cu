@@ -34,8 +34,11 @@
 // are appended with one atomic per warp (ballot + popc prefix), the prefix-sum
 // compaction of Section IV.  Counters are double-buffered by parity so that
 // resets need no extra barrier.
+#include <algorithm>
+
 #include "plan_core.cuh"
 #include "plan_fused.cuh"
+#include "plan_local.cuh"
 
 namespace gmtk {
 
@@ -51,9 +54,7 @@ __device__ __forceinline__ void plan_body(const PlanArgs& A, const Team& team, f
         sbox[nbs * DP + t] = A.boxes.hi[t];
     }
     __syncthreads();
-    const float* blo = nbs ? sbox : A.boxes.lo;
-    const float* bhi = nbs ? sbox + nbs * DP : A.boxes.hi;
-    const int nbox = A.boxes.count;
+    const BoxSet<DP> B{nullptr, nbs ? sbox : A.boxes.lo, nbs ? sbox + nbs * DP : A.boxes.hi, A.boxes.count};
 
     PlanCtl* ctl = A.ctl;
     const int rank = team.rank(), size = team.size();
@@ -241,40 +242,9 @@ __device__ __forceinline__ void plan_body(const PlanArgs& A, const Team& team, f
                     if (lane == 0) { ++n_checks; ++n_failed; atomicCAS(&ctl->error, 0, (int)GMT_ERR_CUDA); }
                     continue;
                 }
-                float sy[D];
-#pragma unroll
-                for (int a = 0; a < D; ++a) sy[a] = __ldg(&A.X[(size_t)a * A.pitch + by]);
-                bool free_edge;
-                const int cached = A.verdict ? (int)__ldcg(&A.verdict[be]) : 0;
-                if (cached != 0) {
-                    free_edge = cached == 1;
-                } else {
-                    if (KIND == GMT_COST_EUCLID)
-                        free_edge = segment_free_warp<DP>(sy, sx, __ldg(&A.in_cost[be]), A.seg_spacing, blo, bhi,
-                                                          nbox, A.grid);
-                    else if (KIND == GMT_COST_DUBINS) {
-                        // the edge's shortest word: stored by the graph build, or recomputed
-                        DubPath P;
-                        if (A.in_path) {
-                            const float4 w = __ldg(reinterpret_cast<const float4*>(A.in_path) + be);
-                            P = DubPath{__float_as_int(w.w), w.x, w.y, w.z, ((w.x + w.y) + w.z) * A.rho};
-                        } else {
-                            P = dubins_path(sy, sx, A.rho);
-                        }
-                        free_edge = dubins_free_warp(sy, sx, P, __ldg(&A.in_cost[be]), A.seg_spacing, A.rho,
-                                                     A.pos_lo, A.pos_hi, blo, bhi, nbox, A.grid);
-                    }
-                    else {
-                        // arrival time of the edge: stored by the graph build, or recomputed
-                        const float tau = A.in_tau ? __ldg(&A.in_tau[be]) : di_tau(di_coef(sy, sx), A.r);
-                        free_edge = trajectory_free_warp(sy, sx, tau, A.traj_points, A.pos_lo, A.pos_hi, blo, bhi, nbox,
-                                                         A.grid);
-                    }
-                    if (lane == 0) {
-                        ++n_computed;
-                        if (A.verdict) A.verdict[be] = free_edge ? 1 : 2;
-                    }
-                }
+                bool computed;
+                const bool free_edge = lazy_check<KIND, DP, 32>(A, by, be, sx, B, nullptr, computed);
+                if (lane == 0 && computed) ++n_computed;
                 if (lane == 0) {
                     n_pull += (unsigned long long)(r1 - r0);
                     ++n_checks;
@@ -411,35 +381,12 @@ __global__ void __launch_bounds__(1024, 1) plan_kernel(PlanArgs A, Team team) {
     }
 }
 
-// One CTA whose wavefront state lives in its shared memory: after the region
-// of staged boxes / parent copy (region0 bytes) come the control block, the
-// snapshot (ocost), the stamps and the lists (plan_smem_state_bytes).  Every
-// step of the body then touches L2 only for the read-only CSR, the samples and
-// the outputs.  The control block is copied out for the host at the end.
-template <int KIND, int DP>
-__global__ void __launch_bounds__(1024, 1) plan_kernel_smem(PlanArgs A, unsigned region0) {
-    extern __shared__ __align__(16) float smem[];
-    unsigned char* base = reinterpret_cast<unsigned char*>(smem);
-    PlanCtl* gctl = A.ctl;
-    PlanCtl* sctl = reinterpret_cast<PlanCtl*>(base + region0);
-    const size_t N = (size_t)A.N;
-    float* socost = reinterpret_cast<float*>(base + region0 + kSmemCtlBytes);
-    int* sstamp = reinterpret_cast<int*>(socost + N);
-    int* slists = reinterpret_cast<int*>(base + region0 + kSmemCtlBytes + smem_round16(8 * N));
-    for (int t = threadIdx.x; t < (int)(sizeof(PlanCtl) / sizeof(int)); t += blockDim.x)
-        reinterpret_cast<int*>(sctl)[t] = 0;
-    __syncthreads();
-    A.ctl = sctl;
-    A.ocost = socost;
-    A.stamp = sstamp;
-    assign_plan_lists(A, slists, N);
-    plan_body<BlockTeam, KIND, DP, true>(A, BlockTeam{}, smem, region0);
-    __syncthreads();
-    for (int t = threadIdx.x; t < (int)(sizeof(PlanCtl) / sizeof(int)); t += blockDim.x) {
-        const int v = reinterpret_cast<const int*>(sctl)[t];
-        reinterpret_cast<int*>(gctl)[t] = v;
-        if (A.host_ctl) reinterpret_cast<int*>(A.host_ctl)[t] = v;
-    }
+// One plan on a team that keeps the wavefront's state in its shared memory.
+template <class Team, int KIND, int DP>
+__global__ void __launch_bounds__(1024, 1) plan_local_kernel(PlanArgs A, Team team, bool cache) {
+    extern __shared__ __align__(16) unsigned char plan_smem[];
+    if (plan_body_local<Team, KIND, DP, kPlanPullLanes>(A, team, plan_smem, cache) && A.host_ctl && threadIdx.x < 32)
+        publish_ctl(A.host_ctl, A.ctl, threadIdx.x);
 }
 
 // Persistent batched wavefront: every team (a CTA, or a cluster) takes the next
@@ -526,10 +473,60 @@ __global__ void __launch_bounds__(1024, 1) plan_batch_smem_kernel(const PlanArgs
 
 // ----------------------------------------------------------------- launcher
 namespace {
+// Does the wavefront's state of an N-node plan fit the shared memory of n
+// CTAs, and with the own nodes' rows and states beside it?  CTAs of at most
+// 512 threads are kept small enough for two of them to share an SM where the
+// row cache is what would prevent it.
+bool plan_local_fits(int N, int n, int D, bool directed, size_t box_bytes, int threads, size_t* bytes, bool* cache) {
+    int dev = 0, optin = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (N < 1 || N > (1 << 20) || (N + n - 1) / n > 65535) return false;
+    const size_t room = (size_t)optin - kPlanStaticSmem - sizeof(LocalCtl);
+    const size_t with = local_layout((unsigned)box_bytes, N, n, D, directed, true).total;
+    const size_t without = local_layout((unsigned)box_bytes, N, n, D, directed, false).total;
+    *cache = with <= (threads <= 512 ? std::min(room, (size_t)110 * 1024) : room);
+    *bytes = *cache ? with : without;
+    return *bytes <= room;
+}
+
+template <class Kern, class Team>
+cudaError_t launch_local(Kern kern, const PlanArgs& a, const Team& team, bool cache, int n, int threads, size_t smem,
+                         cudaStream_t st) {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess && n > 8) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(n);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = n;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, a, team, cache);
+}
+
 template <int KIND, int DP>
 cudaError_t plan_t(const PlanArgs& a, int blocks, int threads, int cluster, cudaStream_t st) {
     const int nbs = a.boxes.count <= smem_box_cap(DP) ? a.boxes.count : 0;
     const size_t smem = plan_smem_bytes(nbs, DP, a.N);
+    // one cluster or one CTA: the wavefront's state in its shared memory, when
+    // it fits (and the rows can be read four entries at a time)
+    const bool aligned = (((uintptr_t)a.out_col | (uintptr_t)a.in_col | (uintptr_t)a.in_cost) & 15) == 0;
+    const int n = cluster > 1 ? cluster : 1;
+    size_t local = 0;
+    bool cache = false;
+    if ((cluster > 1 || blocks <= 1) && aligned &&
+        plan_local_fits(a.N, n, a.d, KIND != GMT_COST_EUCLID,
+                        (size_t)local_staged_boxes(a, DP) * BoxSet<DP>::kQ * 16, threads, &local, &cache))
+        return n == 1 ? launch_local(plan_local_kernel<BlockTeam, KIND, DP>, a, BlockTeam{}, cache, 1, threads, local, st)
+                      : launch_local(plan_local_kernel<ClusterTeam, KIND, DP>, a, ClusterTeam{}, cache, n, threads,
+                                     local, st);
     if (cluster > 1) {
         auto kern = plan_kernel<ClusterTeam, KIND, DP>;
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
@@ -549,19 +546,6 @@ cudaError_t plan_t(const PlanArgs& a, int blocks, int threads, int cluster, cuda
         return cudaLaunchKernelEx(&cfg, kern, a, ClusterTeam{});
     }
     if (blocks <= 1) {
-        // one CTA: the wavefront state goes to shared memory when it fits
-        int dev = 0, optin = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-        const size_t region0 = smem_round16(smem);
-        const size_t total = plan_smem_state_bytes(region0, a.N);
-        if (total <= (size_t)optin) {
-            auto kern = plan_kernel_smem<KIND, DP>;
-            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)total);
-            if (e != cudaSuccess) return e;
-            kern<<<1, threads, total, st>>>(a, (unsigned)region0);
-            return cudaGetLastError();
-        }
         plan_kernel<BlockTeam, KIND, DP><<<1, threads, smem, st>>>(a, BlockTeam{});
         return cudaGetLastError();
     }

@@ -12,6 +12,8 @@ namespace gmtk {
 
 constexpr int kDefaultSpinLimit = 1 << 22;
 
+__host__ __device__ constexpr size_t smem_round16(size_t b) { return (b + 15) / 16 * 16; }
+
 __device__ __forceinline__ int ldcg_i(const int* p) { return __ldcg(p); }
 __device__ __forceinline__ unsigned ldcg_u(const unsigned* p) { return __ldcg(p); }
 __device__ __forceinline__ float ldcg_f(const float* p) { return __ldcg(p); }
@@ -19,6 +21,7 @@ __device__ __forceinline__ float ldcg_f(const float* p) { return __ldcg(p); }
 // Every team also names its CTAs (cta() in [0, ctas())), so that work can be
 // dealt to CTAs round-robin.
 struct BlockTeam {
+    static constexpr bool kSingle = true;
     static constexpr bool kSharedCtl = true;  // the team's counters can live in shared memory
     __device__ __forceinline__ int id() const { return blockIdx.x; }
     __device__ __forceinline__ int cta() const { return 0; }
@@ -75,6 +78,7 @@ struct GridTeam {
 // scope); it cannot wait forever because every thread of the cluster reaches
 // every barrier (all exits from the iteration loop are uniform).
 struct ClusterTeam {
+    static constexpr bool kSingle = false;
     static constexpr bool kSharedCtl = true;
     __device__ __forceinline__ static unsigned cta_rank() {
         unsigned r;
@@ -238,23 +242,13 @@ __device__ __forceinline__ unsigned cluster_map(const void* p, unsigned rank) {
 // the computed points is never dropped: the verdict equals testing every
 // point against every box.
 
-// Does box b meet [lo, hi] (closed intervals on all DP axes)?
-template <int DP>
-__device__ __forceinline__ bool box_meets(const float* blo, const float* bhi, int b, const float* lo,
-                                          const float* hi) {
-    bool m = true;
-#pragma unroll
-    for (int a = 0; a < DP; ++a) m = m && blo[b * DP + a] <= hi[a] && lo[a] <= bhi[b * DP + a];
-    return m;
-}
-
 // Geometric edge y -> x of length L: m = max(2, ceil(L/spacing) + 1) points
 // p_k = y + t_k (x - y), t_k = k/(m-1); collision if one lies in a closed box.
 // Without the grid, boxes that do not meet the segment's bounding box (every
 // computed p_k lies within a few ulps of it) are set aside W at a time first.
 template <int DP, int W = 32>
-__device__ __forceinline__ bool segment_free_warp(const float* y, const float* x, float L, float spacing, const float* blo,
-                                  const float* bhi, int nbox, const BoxGridArgs& grid) {
+__device__ __forceinline__ bool segment_free_warp(const float* y, const float* x, float L, float spacing,
+                                                  const BoxSet<DP>& B, const BoxGridArgs& grid) {
     using LG = LaneGroup<W>;
     const int lane = LG::lane();
     int m = (int)ceilf(L / spacing) + 1;
@@ -269,7 +263,7 @@ __device__ __forceinline__ bool segment_free_warp(const float* y, const float* x
                 float p[DP];
 #pragma unroll
                 for (int a = 0; a < DP; ++a) p[a] = y[a] + t * (x[a] - y[a]);
-                hit = in_any_box_grid<DP>(p, blo, bhi, grid);
+                hit = in_any_box_grid<DP>(p, B.lo, B.hi, grid);
             }
             if (LG::any(hit)) return false;
         }
@@ -282,9 +276,9 @@ __device__ __forceinline__ bool segment_free_warp(const float* y, const float* x
         lo[a] = fminf(x[a], y[a]) - e;
         hi[a] = fmaxf(x[a], y[a]) + e;
     }
-    for (int b0 = 0; b0 < nbox; b0 += W) {
+    for (int b0 = 0; b0 < B.count; b0 += W) {
         const int b = b0 + lane;
-        const unsigned near = LG::ballot(b < nbox && box_meets<DP>(blo, bhi, b, lo, hi));
+        const unsigned near = LG::ballot(b < B.count && B.meets(b, lo, hi));
         if (!near) continue;
         for (int k0 = 0; k0 < m; k0 += W) {
             const int k = k0 + lane;
@@ -294,7 +288,7 @@ __device__ __forceinline__ bool segment_free_warp(const float* y, const float* x
                 float p[DP];
 #pragma unroll
                 for (int a = 0; a < DP; ++a) p[a] = y[a] + t * (x[a] - y[a]);
-                for (unsigned w = near; w; w &= w - 1) hit = hit || in_box<DP>(p, blo, bhi, b0 + __ffs(w) - 1);
+                for (unsigned w = near; w; w &= w - 1) hit = hit | B.holds(b0 + __ffs(w) - 1, p);
             }
             if (LG::any(hit)) return false;
         }
@@ -302,52 +296,65 @@ __device__ __forceinline__ bool segment_free_warp(const float* y, const float* x
     return true;
 }
 
+// Least and greatest value over a lane group, one instruction each (a NaN is
+// passed over).
+__device__ __forceinline__ float group_min(unsigned mask, float v) {
+    float r;
+    asm volatile("redux.sync.min.f32 %0, %1, %2;" : "=f"(r) : "f"(v), "r"(mask));
+    return r;
+}
+__device__ __forceinline__ float group_max(unsigned mask, float v) {
+    float r;
+    asm volatile("redux.sync.max.f32 %0, %1, %2;" : "=f"(r) : "f"(v), "r"(mask));
+    return r;
+}
+
+// Does one of the lane group's points (has: the lane holds one) lie in a box?
+// Only the boxes that meet the bounding box of the group's computed points can
+// hold one (no rounding is in between, so nothing is inflated); one box per
+// lane, W at a time.
+template <int W>
+__device__ __forceinline__ bool points_hit(const float* p, bool has, const BoxSet<3>& B) {
+    using LG = LaneGroup<W>;
+    float lo[3], hi[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        lo[a] = group_min(LG::mask(), has ? p[a] : f_inf());
+        hi[a] = group_max(LG::mask(), has ? p[a] : -f_inf());
+    }
+    bool hit = false;
+    for (int b0 = 0; b0 < B.count; b0 += W) {
+        const int b = b0 + LG::lane();
+        const unsigned near = LG::ballot(b < B.count && B.meets(b, lo, hi));
+        if (near && has && !hit) hit = in_near_boxes<3>(p, B, b0, near);
+    }
+    return hit;
+}
+
 // Double-integrator edge: `points` samples of the Hermite trajectory at
 // s_k = k/(points-1); collision if one lies in a box or outside the position
-// bounds.  Without the grid, the boxes are first filtered against the
-// bounding box of the cubic's Bezier control points p0, p0 + tau v0 / 3,
-// p1 - tau v1 / 3, p1 (the curve lies in their convex hull), inflated.
+// bounds.  basis: the points' Hermite basis (points entries), or NULL to
+// compute it.  (The boxes used to be filtered against the hull of the cubic's
+// Bezier control points, which a chunk's own points fill only in part.)
 template <int W = 32>
-__device__ __forceinline__ bool trajectory_free_warp(const float* y, const float* x, float tau, int points, const float* plo,
-                                            const float* phi, const float* blo, const float* bhi, int nbox,
-                                            const BoxGridArgs& grid) {
+__device__ __forceinline__ bool trajectory_free_warp(const float* y, const float* x, float tau, int points,
+                                                     const float* plo, const float* phi, const BoxSet<3>& B,
+                                                     const BoxGridArgs& grid, const float4* basis = nullptr) {
     using LG = LaneGroup<W>;
     const int lane = LG::lane();
     const float denom = (float)(points - 1);
-    float lo[3], hi[3];
-    unsigned near_first = 0;  // boxes 0..W-1, reused by the first chunk of points
-    if (!grid.use) {
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            const float c1 = y[a] + tau * y[3 + a] / 3.0f, c2 = x[a] - tau * x[3 + a] / 3.0f;
-            const float e =
-                1e-5f * (fabsf(y[a]) + fabsf(x[a]) + tau * (fabsf(y[3 + a]) + fabsf(x[3 + a]))) + 1e-30f;
-            lo[a] = fminf(fminf(y[a], x[a]), fminf(c1, c2)) - e;
-            hi[a] = fmaxf(fmaxf(y[a], x[a]), fmaxf(c1, c2)) + e;
-        }
-        if (nbox > 0) near_first = LG::ballot(lane < nbox && box_meets<3>(blo, bhi, lane, lo, hi));
-    }
     for (int k0 = 0; k0 < points; k0 += W) {
         const int k = k0 + lane;
         bool hit = false;
-        float p[3];
+        float p[3] = {0.0f, 0.0f, 0.0f};
         if (k < points) {
-            const float s = (float)k / denom;
-            hermite_point(y, x, tau, s, p);
+            hermite_point(y, x, tau, basis ? basis[k] : hermite_basis((float)k / denom), p);
 #pragma unroll
-            for (int a = 0; a < 3; ++a) hit = hit || p[a] < plo[a] || p[a] > phi[a];
-            if (grid.use && !hit) hit = in_any_box_grid<3>(p, blo, bhi, grid);
-        }
-        if (!grid.use) {
-            for (int b0 = 0; b0 < nbox; b0 += W) {
-                const unsigned near =
-                    b0 == 0 ? near_first
-                            : LG::ballot(b0 + lane < nbox && box_meets<3>(blo, bhi, b0 + lane, lo, hi));
-                if (k < points)
-                    if (!hit && near) hit = in_near_boxes<3>(p, blo, bhi, b0, near);
-            }
+            for (int a = 0; a < 3; ++a) hit = hit | (p[a] < plo[a]) | (p[a] > phi[a]);
+            if (grid.use && !hit) hit = in_any_box_grid<3>(p, B.lo, B.hi, grid);
         }
         if (LG::any(hit)) return false;
+        if (!grid.use && B.count > 0 && LG::any(points_hit<W>(p, k < points, B))) return false;
     }
     return true;
 }
@@ -355,16 +362,11 @@ __device__ __forceinline__ bool trajectory_free_warp(const float* y, const float
 // Dubins airplane edge y -> x of cost c along its shortest word P:
 // m = max(2, ceil(c / spacing) + 1) trajectory points at fractions k / (m - 1);
 // a point in a box or outside the position bounds collides.  Every lane walks
-// the segment start poses once, then its own points.  Without the box grid,
-// boxes are first tested against a bound of the whole trajectory: its planar
-// part stays within c/2 of the midpoint of y and x (a point at arc length l is
-// within l of y and L - l of x, L <= c), its altitude between the two end
-// altitudes.
+// the segment start poses once, then its own points.
 template <int W = 32>
 __device__ __forceinline__ bool dubins_free_warp(const float* y, const float* x, const DubPath& P, float c,
                                                  float spacing, float rho, const float* plo, const float* phi,
-                                                 const float* blo, const float* bhi, int nbox,
-                                                 const BoxGridArgs& grid) {
+                                                 const BoxSet<3>& B, const BoxGridArgs& grid) {
     using LG = LaneGroup<W>;
     const int lane = LG::lane();
     if (P.word >= kDubNone) return false;  // no word: never an edge (its cost would be +inf)
@@ -372,42 +374,56 @@ __device__ __forceinline__ bool dubins_free_warp(const float* y, const float* x,
     int m = (int)ceilf(c / spacing) + 1;
     if (m < 2) m = 2;
     const float denom = (float)(m - 1);
-    float lo[3], hi[3];
-    unsigned near_first = 0;
-    if (!grid.use) {
-        const float e = 1e-3f * c + 1e-5f * (fabsf(y[0]) + fabsf(y[1]) + fabsf(y[2]) + rho) + 1e-30f;
-#pragma unroll
-        for (int a = 0; a < 2; ++a) {
-            const float mid = 0.5f * (y[a] + x[a]);
-            lo[a] = mid - 0.5f * c - e;
-            hi[a] = mid + 0.5f * c + e;
-        }
-        lo[2] = fminf(y[2], x[2]) - e;
-        hi[2] = fmaxf(y[2], x[2]) + e;
-        if (nbox > 0) near_first = LG::ballot(lane < nbox && box_meets<3>(blo, bhi, lane, lo, hi));
-    }
     for (int k0 = 0; k0 < m; k0 += W) {
         const int k = k0 + lane;
         bool hit = false;
-        float p[3];
+        float p[3] = {0.0f, 0.0f, 0.0f};
         if (k < m) {
             dubins_point(y, x, G, (float)k / denom, p);
 #pragma unroll
-            for (int a = 0; a < 3; ++a) hit = hit || p[a] < plo[a] || p[a] > phi[a];
-            if (grid.use && !hit) hit = in_any_box_grid<3>(p, blo, bhi, grid);
-        }
-        if (!grid.use) {
-            for (int b0 = 0; b0 < nbox; b0 += W) {
-                const unsigned near =
-                    b0 == 0 ? near_first
-                            : LG::ballot(b0 + lane < nbox && box_meets<3>(blo, bhi, b0 + lane, lo, hi));
-                if (k < m)
-                    if (!hit && near) hit = in_near_boxes<3>(p, blo, bhi, b0, near);
-            }
+            for (int a = 0; a < 3; ++a) hit = hit | (p[a] < plo[a]) | (p[a] > phi[a]);
+            if (grid.use && !hit) hit = in_any_box_grid<3>(p, B.lo, B.hi, grid);
         }
         if (LG::any(hit)) return false;
+        if (!grid.use && B.count > 0 && LG::any(points_hit<W>(p, k < m, B))) return false;
     }
     return true;
+}
+
+// The lazy collision check (Alg. 1) of in-edge be of the node with state sx,
+// whose chosen parent is node by: the cached verdict if there is one, else
+// the check of that edge, kept in the cache.  Run by a group of W lanes.
+template <int KIND, int DP, int W>
+__device__ __forceinline__ bool lazy_check(const PlanArgs& A, int by, int be, const float* sx, const BoxSet<DP>& B,
+                                           const float4* basis, bool& computed) {
+    constexpr int D = KIND == GMT_COST_DI ? 6 : (KIND == GMT_COST_DUBINS ? 4 : DP);
+    float sy[D];
+#pragma unroll
+    for (int a = 0; a < D; ++a) sy[a] = __ldg(&A.X[(size_t)a * A.pitch + by]);
+    const int cached = A.verdict ? (int)__ldcg(&A.verdict[be]) : 0;
+    computed = cached == 0;
+    if (cached != 0) return cached == 1;
+    bool free_edge;
+    if constexpr (KIND == GMT_COST_EUCLID) {
+        free_edge = segment_free_warp<DP, W>(sy, sx, __ldg(&A.in_cost[be]), A.seg_spacing, B, A.grid);
+    } else if constexpr (KIND == GMT_COST_DUBINS) {
+        // the edge's shortest word: stored by the graph build, or recomputed
+        DubPath P;
+        if (A.in_path) {
+            const float4 w = __ldg(reinterpret_cast<const float4*>(A.in_path) + be);
+            P = DubPath{__float_as_int(w.w), w.x, w.y, w.z, ((w.x + w.y) + w.z) * A.rho};
+        } else {
+            P = dubins_path(sy, sx, A.rho);
+        }
+        free_edge = dubins_free_warp<W>(sy, sx, P, __ldg(&A.in_cost[be]), A.seg_spacing, A.rho, A.pos_lo, A.pos_hi,
+                                        B, A.grid);
+    } else {
+        // arrival time of the edge: stored by the graph build, or recomputed
+        const float tau = A.in_tau ? __ldg(&A.in_tau[be]) : di_tau(di_coef(sy, sx), A.r);
+        free_edge = trajectory_free_warp<W>(sy, sx, tau, A.traj_points, A.pos_lo, A.pos_hi, B, A.grid, basis);
+    }
+    if (A.verdict && LaneGroup<W>::lane() == 0) A.verdict[be] = free_edge ? 1 : 2;
+    return free_edge;
 }
 
 // Loads of the wavefront's mutable state (snapshot, lists, control block):
@@ -463,7 +479,6 @@ __device__ __forceinline__ void lane_parent_min(const int* __restrict__ in_col, 
 // Shared-memory layout of the single-CTA kernel that keeps the wavefront state
 // on chip (plan_kernel_smem): region0 (boxes / parent copy), the control
 // block, ocost and stamp (N each), the lists.
-__host__ __device__ constexpr size_t smem_round16(size_t b) { return (b + 15) / 16 * 16; }
 constexpr size_t kSmemCtlBytes = smem_round16(sizeof(PlanCtl));
 inline size_t plan_smem_state_bytes(size_t region0, int N) {
     return smem_round16(region0) + kSmemCtlBytes + smem_round16((size_t)8 * N) +

@@ -45,8 +45,8 @@ struct FusedCounts {
 // candidates side by side).
 template <int KIND, int DP, int W, bool SH>
 __device__ __forceinline__ void fused_pull(const PlanArgs& A, const TeamCtl<SH>& tc, int x, const float* ocur,
-                                           float* onext, int2* nxt, int set, int p, const float* blo,
-                                           const float* bhi, int nbox, FusedCounts& cnt) {
+                                           float* onext, int2* nxt, int set, int p, const BoxSet<DP>& B,
+                                           FusedCounts& cnt) {
     constexpr int D = KIND == GMT_COST_DI ? 6 : (KIND == GMT_COST_DUBINS ? 4 : DP);
     using LG = LaneGroup<W>;
     const int lane = LG::lane();
@@ -74,37 +74,9 @@ __device__ __forceinline__ void fused_pull(const PlanArgs& A, const TeamCtl<SH>&
         if (lane == 0) { ++cnt.checks; ++cnt.failed; tc.cas(&ctl->error, 0, (int)GMT_ERR_CUDA); }
         return;
     }
-    float sy[D];
-#pragma unroll
-    for (int a = 0; a < D; ++a) sy[a] = __ldg(&A.X[(size_t)a * A.pitch + by]);
-    bool free_edge;
-    const int cached = A.verdict ? (int)__ldcg(&A.verdict[be]) : 0;
-    if (cached != 0) {
-        free_edge = cached == 1;
-    } else {
-        if (KIND == GMT_COST_EUCLID) {
-            free_edge =
-                segment_free_warp<DP, W>(sy, sx, __ldg(&A.in_cost[be]), A.seg_spacing, blo, bhi, nbox, A.grid);
-        } else if (KIND == GMT_COST_DUBINS) {
-            DubPath P;
-            if (A.in_path) {
-                const float4 w = __ldg(reinterpret_cast<const float4*>(A.in_path) + be);
-                P = DubPath{__float_as_int(w.w), w.x, w.y, w.z, ((w.x + w.y) + w.z) * A.rho};
-            } else {
-                P = dubins_path(sy, sx, A.rho);
-            }
-            free_edge = dubins_free_warp<W>(sy, sx, P, __ldg(&A.in_cost[be]), A.seg_spacing, A.rho, A.pos_lo,
-                                            A.pos_hi, blo, bhi, nbox, A.grid);
-        } else {
-            const float tau = A.in_tau ? __ldg(&A.in_tau[be]) : di_tau(di_coef(sy, sx), A.r);
-            free_edge =
-                trajectory_free_warp<W>(sy, sx, tau, A.traj_points, A.pos_lo, A.pos_hi, blo, bhi, nbox, A.grid);
-        }
-        if (lane == 0) {
-            ++cnt.computed;
-            if (A.verdict) A.verdict[be] = free_edge ? 1 : 2;
-        }
-    }
+    bool computed;
+    const bool free_edge = lazy_check<KIND, DP, W>(A, by, be, sx, B, nullptr, computed);
+    if (lane == 0 && computed) ++cnt.computed;
     if (lane == 0) {
         cnt.pull += (unsigned long long)(r1 - r0);
         ++cnt.checks;
@@ -139,9 +111,7 @@ __device__ __forceinline__ void plan_body_fused(const PlanArgs& A, const Team& t
         sbox[nbs * DP + t] = A.boxes.hi[t];
     }
     __syncthreads();
-    const float* blo = nbs ? sbox : A.boxes.lo;
-    const float* bhi = nbs ? sbox + nbs * DP : A.boxes.hi;
-    const int nbox = A.boxes.count;
+    const BoxSet<DP> B{nullptr, nbs ? sbox : A.boxes.lo, nbs ? sbox + nbs * DP : A.boxes.hi, A.boxes.count};
 
     PlanCtl* ctl = A.ctl;
     // the team's counters: a copy in CTA 0's shared memory for a CTA or a
@@ -335,7 +305,7 @@ __device__ __forceinline__ void plan_body_fused(const PlanArgs& A, const Team& t
             }
             x = __shfl_sync(LaneGroup<W>::mask(), x, 0, W);
             if (x < 0) break;
-            fused_pull<KIND, DP, W, SH>(A, tc, x, ocur, onext, nxt, set, p, blo, bhi, nbox, cnt);
+            fused_pull<KIND, DP, W, SH>(A, tc, x, ocur, onext, nxt, set, p, B, cnt);
         }
         __syncwarp();  // the lane groups leave the queue apart; the barrier wants whole warps
         if (!(ok = team.sync(ctl))) break;

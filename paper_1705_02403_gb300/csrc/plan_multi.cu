@@ -108,41 +108,10 @@ __device__ bool pull_candidate(const PlanArgs* __restrict__ Ap, LockSmem& sm, in
         }
         return false;
     }
-    float sy[D];
-#pragma unroll
-    for (int a = 0; a < D; ++a) sy[a] = __ldg(&X[(size_t)a * pitch + by]);
-    const int nbox = Ap->boxes.count;
-    const float* blo = Ap->boxes.lo;
-    const float* bhi = Ap->boxes.hi;
-    uint8_t* verdict = Ap->verdict;
-    bool free_edge;
-    const int cached = verdict ? (int)__ldcg(&verdict[be]) : 0;
-    if (cached != 0) {
-        free_edge = cached == 1;
-    } else {
-        if (KIND == GMT_COST_EUCLID) {
-            free_edge =
-                segment_free_warp<DP>(sy, sx, __ldg(&in_cost[be]), Ap->seg_spacing, blo, bhi, nbox, Ap->grid);
-        } else if (KIND == GMT_COST_DUBINS) {
-            DubPath P;
-            if (Ap->in_path) {
-                const float4 w = __ldg(reinterpret_cast<const float4*>(Ap->in_path) + be);
-                P = DubPath{__float_as_int(w.w), w.x, w.y, w.z, ((w.x + w.y) + w.z) * Ap->rho};
-            } else {
-                P = dubins_path(sy, sx, Ap->rho);
-            }
-            free_edge = dubins_free_warp(sy, sx, P, __ldg(&in_cost[be]), Ap->seg_spacing, Ap->rho, Ap->pos_lo,
-                                         Ap->pos_hi, blo, bhi, nbox, Ap->grid);
-        } else {
-            const float tau = Ap->in_tau ? __ldg(&Ap->in_tau[be]) : di_tau(di_coef(sy, sx), Ap->r);
-            free_edge = trajectory_free_warp(sy, sx, tau, Ap->traj_points, Ap->pos_lo, Ap->pos_hi, blo, bhi, nbox,
-                                             Ap->grid);
-        }
-        if (lane == 0) {
-            atomicAdd(&sm.acc_computed[q], 1u);
-            if (verdict) verdict[be] = free_edge ? 1 : 2;
-        }
-    }
+    const BoxSet<DP> B{nullptr, Ap->boxes.lo, Ap->boxes.hi, Ap->boxes.count};
+    bool computed;
+    const bool free_edge = lazy_check<KIND, DP, 32>(*Ap, by, be, sx, B, nullptr, computed);
+    if (lane == 0 && computed) atomicAdd(&sm.acc_computed[q], 1u);
     if (lane == 0) {
         atomicAdd(&sm.acc_pull[q], (unsigned)(r1 - r0));
         atomicAdd(&sm.acc_checks[q], 1u);

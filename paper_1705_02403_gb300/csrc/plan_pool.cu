@@ -236,39 +236,10 @@ __device__ void pull_item(const PlanArgs& A, int j, const PoolIter& I, TaskCount
             continue;
         }
         if (lane == 0) cnt.pull += (unsigned long long)(r1 - r0);
-        float sy[D];
-#pragma unroll
-        for (int a = 0; a < D; ++a) sy[a] = __ldg(&A.X[(size_t)a * A.pitch + by]);
-        bool free_edge;
-        const int cached = A.verdict ? (int)__ldcg(&A.verdict[be]) : 0;
-        const float* blo = A.boxes.lo;
-        const float* bhi = A.boxes.hi;
-        if (cached != 0) {
-            free_edge = cached == 1;
-        } else {
-            if (KIND == GMT_COST_EUCLID) {
-                free_edge = segment_free_warp<DP>(sy, sx, __ldg(&A.in_cost[be]), A.seg_spacing, blo, bhi,
-                                                  A.boxes.count, A.grid);
-            } else if (KIND == GMT_COST_DUBINS) {
-                DubPath P;
-                if (A.in_path) {
-                    const float4 w = __ldg(reinterpret_cast<const float4*>(A.in_path) + be);
-                    P = DubPath{__float_as_int(w.w), w.x, w.y, w.z, ((w.x + w.y) + w.z) * A.rho};
-                } else {
-                    P = dubins_path(sy, sx, A.rho);
-                }
-                free_edge = dubins_free_warp(sy, sx, P, __ldg(&A.in_cost[be]), A.seg_spacing, A.rho, A.pos_lo,
-                                             A.pos_hi, blo, bhi, A.boxes.count, A.grid);
-            } else {
-                const float tau = A.in_tau ? __ldg(&A.in_tau[be]) : di_tau(di_coef(sy, sx), A.r);
-                free_edge = trajectory_free_warp(sy, sx, tau, A.traj_points, A.pos_lo, A.pos_hi, blo, bhi,
-                                                 A.boxes.count, A.grid);
-            }
-            if (lane == 0) {
-                ++cnt.computed;
-                if (A.verdict) A.verdict[be] = free_edge ? 1 : 2;
-            }
-        }
+        const BoxSet<DP> B{nullptr, A.boxes.lo, A.boxes.hi, A.boxes.count};
+        bool computed;
+        const bool free_edge = lazy_check<KIND, DP, 32>(A, by, be, sx, B, nullptr, computed);
+        if (lane == 0 && computed) ++cnt.computed;
         if (lane == 0) {
             ++cnt.checks;
             if (free_edge) {

@@ -16,9 +16,8 @@
 //    (cudaGetSymbolAddress, with that device current) and caches it, together
 //    with the largest resident cluster of the plan kernel; make that first
 //    call before any stream capture begins.
-//  - Launch: the same automatic shape as gmt_plan (one CTA with its state in
-//    shared memory for small 2D graphs, else the largest resident thread-block
-//    cluster, else a cooperative grid).  Obstacles are scanned linearly by
+//  - Launch: the same automatic shape as gmt_plan (the largest resident
+//    thread-block cluster, else a cooperative grid).  Obstacles are scanned linearly by
 //    every check: the box grid that gmt_plan builds for 128 or more boxes needs
 //    allocated scratch, so many boxes cost more here than in gmt_plan.
 //  - Sharing: every call on a device uses the same array and the array keeps
@@ -164,23 +163,18 @@ extern "C" gmt_status gmt_plan_static(const gmt_space* space, const gmt_graph_vi
 
     // launch shape: as gmt_plan chooses it automatically
     int blocks = 0, cluster = 0, threads = 0;
-    if (g->kind == GMT_COST_EUCLID && g->pos_dim == 2 && g->N <= 2049) {
-        blocks = 1;  // one CTA, wavefront state in shared memory
-        threads = 1024;
-    } else {
-        threads = g->N <= 2048 ? 512 : 1024;
-        s = max_cluster(g->kind, g->pos_dim, threads, &cluster);
-        if (s != GMT_OK) return s;
-        if (cluster <= 1) {
-            cluster = 0;
-            int dev = 0, sms = 0;
-            cudaError_t e = cudaGetDevice(&dev);
-            if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-            if (e != cudaSuccess) return cuda_fail(e, "device attribute");
-            const int maxb = plan_max_coresident_blocks(g->kind, g->pos_dim, threads);
-            if (maxb <= 0) return fail(GMT_ERR_CUDA, "plan kernel cannot be resident");
-            blocks = sms < maxb ? sms : maxb;
-        }
+    threads = g->N <= 2048 ? 512 : 1024;
+    s = max_cluster(g->kind, g->pos_dim, threads, &cluster);
+    if (s != GMT_OK) return s;
+    if (cluster <= 1) {
+        cluster = 0;
+        int dev = 0, sms = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (e != cudaSuccess) return cuda_fail(e, "device attribute");
+        const int maxb = plan_max_coresident_blocks(g->kind, g->pos_dim, threads);
+        if (maxb <= 0) return fail(GMT_ERR_CUDA, "plan kernel cannot be resident");
+        blocks = sms < maxb ? sms : maxb;
     }
     // a cooperative grid's barrier counts live in the control block and must
     // start at zero; the other launches clear their result fields themselves
