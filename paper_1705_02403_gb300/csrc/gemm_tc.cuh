@@ -1,6 +1,8 @@
 // BF16 x BF16 -> FP32 GEMM on the 5th-generation tensor cores (tcgen05) for
 // sm_103a, written with inline PTX:
 //   C[M, N] = A[M, K] . B[N, K]^T   (both operands K-major, row-major in memory)
+// For M <= 128 (fewer rows than half of a CTA pair's tile); more rows take the
+// CTA-pair kernel at the end of this file.
 //
 // One CTA of 128 threads computes a 128 x 128 tile of C (optionally a K-slice
 // of it, for split-K):
@@ -260,6 +262,249 @@ __global__ void __launch_bounds__(128, 1) gemm_tn_bf16_kernel(const __grid_const
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 128;" ::"r"(tmem) : "memory");
+}
+
+// ---------------------------------------------------------------- CTA pairs
+// The same product on pairs of CTAs (cta_group::2), for M > 128: a pair of SMs
+// computes a 256 x tile_n tile of C with one tcgen05.mma of M = 256, each CTA
+// holding 128 rows of A and half of B's rows, so a K-block costs 128 +
+// tile_n / 2 rows of shared-memory fill and reads per SM instead of 256 (the
+// single-CTA kernel is bound by them: 4096^3 took 194 us, 0.71 PFLOP/s).  The
+// grid is persistent, one pair per two SMs, over (K-slice, tile) items; the
+// accumulator is double-buffered in TMEM (2 x 256 columns), so the epilogue
+// of one item runs beside the loads and MMAs of the next.
+//   warp 0: TMA producer of its CTA; both CTAs' copies complete on the leader's
+//           "full" barriers
+//   warp 1 (leader): MMA issuer; tcgen05.commit returns each stage to both
+//           CTAs' producers and each finished accumulator to both epilogues
+//   warp 2: TMEM allocation
+//   warps 4-7: epilogue of the CTA's 128 rows
+// An operand may be stored with its rows (M or N) contiguous instead of K
+// (MN-major): boxes of 64 rows x 64 K then land as 64 lines of 128 bytes, which
+// the descriptor addresses 8 K at a time (stride 1024) and 64 rows at a time
+// (stride 8192); the backward products read activations and weights this way
+// without a transposed copy.
+constexpr int kPairStages = 6;
+constexpr int kPairThreads = 256;
+constexpr int kPairStageBytes = 2 * kGemmTileBytes;  // A 16 KB, B at most 16 KB
+constexpr int kPairStagePitch = 33;
+constexpr int kPairSmem = kPairStages * kPairStageBytes + 4 * 32 * kPairStagePitch * 4 + 1024 + 256;
+
+struct PairArgs {
+    GemmArgs g;
+    int tile_n, tiles_m, tiles_n, splits;
+    int a_mn, b_mn;  // operand stored [K][rows]
+};
+
+__device__ __forceinline__ uint64_t mn_desc(uint32_t saddr) {
+    uint64_t d = 0;
+    d |= (uint64_t)((saddr & 0x3FFFF) >> 4);
+    d |= (uint64_t)(8192 >> 4) << 16;
+    d |= (uint64_t)(1024 >> 4) << 32;
+    d |= (uint64_t)1 << 46;
+    d |= (uint64_t)2 << 61;
+    return d;
+}
+
+__device__ __forceinline__ uint32_t cta_map(const void* p, uint32_t rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_u32(p)), "r"(rank));
+    return r;
+}
+
+// TMA load into this CTA's shared memory that completes on the barrier at
+// shared::cluster address `bar` (the leader's).
+__device__ __forceinline__ void tma_load_pair(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, "
+        "%3}], [%4];" ::"r"(dst),
+        "l"((uint64_t)map), "r"(x), "r"(y), "r"(bar)
+        : "memory");
+}
+
+__device__ __forceinline__ void mma_bf16_pair(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                              uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+        ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+
+// Arrives on the barrier at this offset in both CTAs once the MMAs issued so
+// far are done.
+__device__ __forceinline__ void mma_commit_pair(uint64_t* bar) {
+    asm volatile(
+        "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
+            smem_u32(bar)),
+        "h"((uint16_t)3)
+        : "memory");
+}
+
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar) {
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
+    gemm_pair_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+                          PairArgs a) {
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* base = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    float* staging = (float*)(base + kPairStages * kPairStageBytes);
+    uint64_t* full = (uint64_t*)(staging + 4 * 32 * kPairStagePitch);
+    uint64_t* empty = full + kPairStages;
+    uint64_t* acc_full = empty + kPairStages;
+    uint64_t* acc_empty = acc_full + 2;
+    uint32_t* tmem_slot = (uint32_t*)(acc_empty + 2);
+
+    const GemmArgs& g = a.g;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    uint32_t crank;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(crank));
+    const int pair = blockIdx.x >> 1, pairs = gridDim.x >> 1;
+    const int kb_total = (g.K + kGemmBK - 1) / kGemmBK;
+    const int tiles = a.tiles_m * a.tiles_n, items = tiles * a.splits;
+    const int half_n = a.tile_n / 2;
+
+    if (warp == 2) {
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(tmem_slot))
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    }
+    if (threadIdx.x == 32) {
+        for (int s = 0; s < kPairStages; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], 1);
+        }
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(&acc_full[b], 1);
+            mbar_init(&acc_empty[b], 8);  // four epilogue warps of each CTA
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem = *tmem_slot;
+
+    // item -> (split, tile): the tiles of a K-slice one after another, rows first
+    if (warp == 0) {
+        if (lane == 0) {
+            const uint32_t bytes = 2u * (uint32_t)(kGemmTileBytes + half_n * kGemmBK * 2);  // both CTAs'
+            int n_issued = 0;
+            bool ok = true;
+            for (int item = pair; item < items && ok; item += pairs) {
+                const int split = item / tiles, tile = item % tiles;
+                const int m0 = (tile % a.tiles_m) * 256 + (int)crank * 128;
+                const int n0 = (tile / a.tiles_m) * a.tile_n + (int)crank * half_n;
+                const int kb0 = split * g.k_blocks_per_split, kb1 = min(kb_total, kb0 + g.k_blocks_per_split);
+                for (int kb = kb0; kb < kb1; ++kb, ++n_issued) {
+                    const int s = n_issued % kPairStages, round = n_issued / kPairStages;
+                    if (round > 0 && !mbar_wait(&empty[s], (round - 1) & 1, g.error)) { ok = false; break; }
+                    if (crank == 0) mbar_expect_tx(&full[s], bytes);
+                    const uint32_t bar = cta_map(&full[s], 0);
+                    const uint32_t sA = smem_u32(base + s * kPairStageBytes), sB = sA + kGemmTileBytes;
+                    const int kx = kb * kGemmBK;
+                    if (a.a_mn) {
+                        tma_load_pair(sA, &tmA, m0, kx, bar);
+                        tma_load_pair(sA + 8192, &tmA, m0 + 64, kx, bar);
+                    } else {
+                        tma_load_pair(sA, &tmA, kx, m0, bar);
+                    }
+                    if (a.b_mn) {
+                        for (int c = 0; c < half_n; c += 64) tma_load_pair(sB + c * 128, &tmB, n0 + c, kx, bar);
+                    } else {
+                        tma_load_pair(sB, &tmB, kx, n0, bar);
+                    }
+                }
+            }
+            if (!ok && crank == 0)  // stopped early: the copies already issued land before the pair leaves
+                for (int i = max(0, n_issued - kPairStages); i < n_issued; ++i)
+                    mbar_wait(&full[i % kPairStages], (i / kPairStages) & 1, g.error);
+        }
+        __syncwarp();
+    } else if (warp == 1) {
+        if (crank == 0 && lane == 0) {
+            const uint32_t idesc = mma_idesc_bf16(256, a.tile_n) | (a.a_mn ? 1u << 15 : 0u) | (a.b_mn ? 1u << 16 : 0u);
+            const uint32_t stepA = a.a_mn ? 2048u : 32u, stepB = a.b_mn ? 2048u : 32u;  // bytes per 16 K
+            int used = 0, n_item = 0;
+            bool ok = true;
+            for (int item = pair; item < items && ok; item += pairs, ++n_item) {
+                const int split = item / tiles;
+                const int kb0 = split * g.k_blocks_per_split, kb1 = min(kb_total, kb0 + g.k_blocks_per_split);
+                const int b = n_item & 1, use = n_item >> 1;
+                if (use > 0 && !mbar_wait(&acc_empty[b], (use - 1) & 1, g.error)) break;
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                for (int kb = kb0; kb < kb1; ++kb, ++used) {
+                    const int s = used % kPairStages, round = used / kPairStages;
+                    if (!mbar_wait(&full[s], round & 1, g.error)) { ok = false; break; }
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    const uint32_t a0 = smem_u32(base + s * kPairStageBytes), b0 = a0 + kGemmTileBytes;
+#pragma unroll
+                    for (int kk = 0; kk < kGemmBK / 16; ++kk)
+                        mma_bf16_pair(tmem + b * 256, a.a_mn ? mn_desc(a0 + kk * stepA) : sw128_desc(a0 + kk * stepA),
+                                      a.b_mn ? mn_desc(b0 + kk * stepB) : sw128_desc(b0 + kk * stepB), idesc,
+                                      (kb > kb0 || kk > 0) ? 1u : 0u);
+                    mma_commit_pair(&empty[s]);
+                }
+                mma_commit_pair(&acc_full[b]);
+            }
+        }
+        __syncwarp();
+    } else if (warp >= 4) {
+        const int ew = warp & 3;  // the TMEM lanes this warp may read: 32 ew ..
+        float* stage = staging + ew * 32 * kPairStagePitch;
+        int n_item = 0;
+        for (int item = pair; item < items; item += pairs, ++n_item) {
+            const int split = item / tiles, tile = item % tiles;
+            const int m0 = (tile % a.tiles_m) * 256 + (int)crank * 128 + ew * 32, n0 = (tile / a.tiles_m) * a.tile_n;
+            const int b = n_item & 1, use = n_item >> 1;
+            const bool waited = mbar_wait(&acc_full[b], use & 1, g.error);
+            if (!__all_sync(0xffffffffu, waited && *(volatile int*)g.error == 0)) break;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const float* biasp = g.bias;
+            float* const C = g.epilogue == kEpiPartialF32 ? g.C + (size_t)split * g.M * g.ldc : g.C;
+            for (int c = 0; c < a.tile_n; c += 32) {
+                float v[32];
+                tmem_ld32(tmem + ((uint32_t)(ew * 32) << 16) + (uint32_t)(b * 256 + c), v);
+                if (c + 32 >= a.tile_n) {  // the last columns are in registers: the accumulator is free
+                    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive_cluster(cta_map(&acc_empty[b], 0));
+                }
+                __syncwarp();
+#pragma unroll
+                for (int j = 0; j < 32; ++j) stage[lane * kPairStagePitch + j] = v[j];
+                __syncwarp();
+                const int col = n0 + c + lane;
+                if (col < g.N) {
+                    const float bv = biasp && g.epilogue != kEpiStoreF32 && g.epilogue != kEpiPartialF32 ? biasp[col] : 0.0f;
+                    const int rows = min(32, g.M - m0);
+                    if (g.epilogue == kEpiBiasReluBF16) {
+#pragma unroll 8
+                        for (int r = 0; r < rows; ++r)
+                            g.Cb[(size_t)(m0 + r) * g.ldc + col] =
+                                __float2bfloat16_rn(fmaxf(stage[r * kPairStagePitch + lane] + bv, 0.0f));
+                    } else if (g.epilogue == kEpiBiasF32) {
+#pragma unroll 8
+                        for (int r = 0; r < rows; ++r)
+                            C[(size_t)(m0 + r) * g.ldc + col] = stage[r * kPairStagePitch + lane] + bv;
+                    } else {
+#pragma unroll 8
+                        for (int r = 0; r < rows; ++r)
+                            C[(size_t)(m0 + r) * g.ldc + col] = stage[r * kPairStagePitch + lane];
+                    }
+                }
+            }
+        }
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    // neither CTA leaves while the other's copies, MMAs or arrivals may reach it
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    if (warp == 2) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
 }
 
 }  // namespace gmtk

@@ -394,7 +394,7 @@ int plan_pool_max_blocks(int threads, bool all_kinds);
 // epilogue 0 = FP32 store, 1 = BF16 relu(x + bias), 2 = FP32 x + bias.
 cudaError_t gemm_bf16_tn(int M, int N, int K, const __nv_bfloat16* A, const __nv_bfloat16* B, int epilogue,
                          const float* bias, float* C, __nv_bfloat16* Cb, int ldc, int splits, float* partial,
-                         int* error, cudaStream_t st);
+                         int* error, cudaStream_t st, bool a_mn = false, bool b_mn = false);
 
 // graph.cu: copies `count` appended samples (DEVICE [d][src_pitch]) into X
 // columns first.. and computes their goal flags; sets flags kSampleBadAppend

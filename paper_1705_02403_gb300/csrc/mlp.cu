@@ -1,7 +1,9 @@
 // Learned sampling proposal: the BF16 tensor-core GEMM launcher and the C ABI
 // entry point that exposes it (gmt_gemm_bf16).  The network, its training and
 // the proposal sampler build on these (proposal.cu).
+#include <algorithm>
 #include <atomic>
+#include <climits>
 #include <cstring>
 #include <mutex>
 #include <string>
@@ -32,19 +34,49 @@ EncodeTiledFn encode_fn() {
 }
 
 // Tensor map of a row-major BF16 matrix [rows, cols] (cols contiguous) read in
-// boxes of 64 columns x 128 rows, 128-byte swizzle, zero fill out of range.
-cudaError_t make_map(CUtensorMap* map, const void* ptr, int rows, int cols) {
+// boxes of 64 columns x box_rows rows, 128-byte swizzle, zero fill out of range.
+cudaError_t make_map(CUtensorMap* map, const void* ptr, int rows, int cols, int box_rows) {
     EncodeTiledFn fn = encode_fn();
     if (!fn) return cudaErrorNotSupported;
     if (((uintptr_t)ptr & 15) != 0 || (cols * 2) % 16 != 0) return cudaErrorInvalidValue;
     const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
     const cuuint64_t strides[1] = {(cuuint64_t)cols * 2};
-    const cuuint32_t box[2] = {(cuuint32_t)kGemmBK, (cuuint32_t)kGemmBM};
+    const cuuint32_t box[2] = {(cuuint32_t)kGemmBK, (cuuint32_t)box_rows};
     const cuuint32_t estr[2] = {1, 1};
     CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(ptr), dims, strides, box, estr,
                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+
+int device_sms() {
+    static std::atomic<int> cached{0};
+    int sms = cached.load(std::memory_order_relaxed);
+    if (sms <= 0) {
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0)
+            sms = 148;
+        cached.store(sms, std::memory_order_relaxed);
+    }
+    return sms;
+}
+
+// Columns of a CTA pair's tile: the width that finishes soonest, taking a
+// tile's time as its columns (at least 64: below, the loads of A's 256 rows
+// set the pace) plus 24 columns' worth of pipeline fill and epilogue tail,
+// times the waves of items over the pairs.  4096^3 takes 224 (304 items, four
+// full waves of 76) where 256 (256 items) would leave the fourth a third full.
+int pair_tile_n(int M, int N, int splits, int pairs, bool b_mn) {
+    int best = 256;
+    long long best_cost = LLONG_MAX;
+    for (int t = 256; t >= 32; t -= 32) {
+        if (b_mn && t % 128) continue;  // each CTA's half is read in boxes of 64 rows
+        const long long items = (long long)((M + 255) / 256) * ((N + t - 1) / t) * splits;
+        const long long cost = (items + pairs - 1) / pairs * (std::max(t, 64) + 24);
+        if (cost < best_cost) { best_cost = cost; best = t; }
+    }
+    return best;
 }
 
 // Sum of split-K partials [splits][M][N] plus the epilogue.
@@ -66,13 +98,14 @@ __global__ void splitk_reduce_kernel(const float* __restrict__ part, int splits,
 
 }  // namespace
 
-// C = A . B^T with A [M, K], B [N, K] BF16 row-major; epilogue as GemmEpilogue.
-// splits > 1 splits K across gridDim.z into `partial` ([splits][M][N] FP32)
-// and reduces deterministically.
+// C = A . B^T with A [M, K], B [N, K] BF16 row-major (a_mn, b_mn: the operand is
+// stored [K, M] or [K, N] instead; M > 128 only); epilogue as GemmEpilogue.
+// splits > 1 splits K into `partial` ([splits][M][N] FP32) and reduces
+// deterministically.
 cudaError_t gemm_bf16_tn(int M, int N, int K, const __nv_bfloat16* A, const __nv_bfloat16* B, int epilogue,
                          const float* bias, float* C, __nv_bfloat16* Cb, int ldc, int splits, float* partial,
-                         int* error, cudaStream_t st) {
-    if (M <= 0 || N <= 0 || K <= 0 || K % 8 != 0) return cudaErrorInvalidValue;
+                         int* error, cudaStream_t st, bool a_mn, bool b_mn) {
+    if (M <= 0 || N <= 0 || K <= 0 || (K % 8 != 0 && !(a_mn && b_mn))) return cudaErrorInvalidValue;
     static std::atomic<bool> attr_set{false};  // setting it twice is harmless
     if (!attr_set.load(std::memory_order_relaxed)) {
         cudaError_t e = cudaFuncSetAttribute(gemm_tn_bf16_kernel<kGemmStagesDeep>,
@@ -81,40 +114,52 @@ cudaError_t gemm_bf16_tn(int M, int N, int K, const __nv_bfloat16* A, const __nv
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(gemm_tn_bf16_kernel<kGemmStagesShort>,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, gemm_smem_bytes(kGemmStagesShort));
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(gemm_pair_bf16_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kPairSmem);
         if (e != cudaSuccess) return e;
         attr_set.store(true, std::memory_order_relaxed);
     }
-    CUtensorMap ta, tb;
-    cudaError_t e = make_map(&ta, A, M, K);
-    if (e == cudaSuccess) e = make_map(&tb, B, N, K);
-    if (e != cudaSuccess) return e;
     const int kb = (K + kGemmBK - 1) / kGemmBK;
     if (splits < 1) splits = 1;
     if (splits > kb) splits = kb;
     const int per = (kb + splits - 1) / splits;
     splits = (kb + per - 1) / per;  // every split gets at least one K-block
-    GemmArgs g;
-    std::memset(&g, 0, sizeof(g));
+    if (splits > 1 && !partial) return cudaErrorInvalidValue;
+    PairArgs p;
+    std::memset(&p, 0, sizeof(p));
+    GemmArgs& g = p.g;
     g.M = M; g.N = N; g.K = K; g.k_blocks_per_split = per; g.error = error; g.bias = bias; g.ldc = ldc;
-    dim3 grid((M + kGemmBM - 1) / kGemmBM, (N + kGemmBN - 1) / kGemmBN, splits);
-    // short K: a shallow ring, two CTAs per SM
-    const bool shallow = per <= 2 * kGemmStagesShort;
-    auto launch = [&](const GemmArgs& a) {
-        if (shallow)
-            gemm_tn_bf16_kernel<kGemmStagesShort><<<grid, 128, gemm_smem_bytes(kGemmStagesShort), st>>>(ta, tb, a);
+    g.epilogue = epilogue; g.C = C; g.Cb = Cb;
+    if (splits > 1) { g.epilogue = kEpiPartialF32; g.C = partial; g.ldc = N; }
+    CUtensorMap ta, tb;
+    cudaError_t e;
+    // More than half a pair's rows: CTA pairs.  (M <= 128 would leave the
+    // second CTA of every pair without rows: 4096 x 4096 x 128 rows.)
+    if (M > kGemmBM || a_mn || b_mn) {
+        const int pairs = std::max(1, device_sms() / 2);
+        p.splits = splits; p.a_mn = a_mn; p.b_mn = b_mn;
+        p.tile_n = pair_tile_n(M, N, splits, pairs, b_mn);
+        p.tiles_m = (M + 255) / 256;
+        p.tiles_n = (N + p.tile_n - 1) / p.tile_n;
+        e = a_mn ? make_map(&ta, A, K, M, kGemmBK) : make_map(&ta, A, M, K, kGemmBM);
+        if (e == cudaSuccess) e = b_mn ? make_map(&tb, B, K, N, kGemmBK) : make_map(&tb, B, N, K, p.tile_n / 2);
+        if (e != cudaSuccess) return e;
+        const long long items = (long long)p.tiles_m * p.tiles_n * splits;
+        if (items > INT_MAX) return cudaErrorInvalidValue;
+        gemm_pair_bf16_kernel<<<2 * (int)std::min<long long>(items, pairs), kPairThreads, kPairSmem, st>>>(ta, tb, p);
+    } else {
+        e = make_map(&ta, A, M, K, kGemmBM);
+        if (e == cudaSuccess) e = make_map(&tb, B, N, K, kGemmBN);
+        if (e != cudaSuccess) return e;
+        const dim3 grid((M + kGemmBM - 1) / kGemmBM, (N + kGemmBN - 1) / kGemmBN, splits);
+        // short K: a shallow ring, two CTAs per SM
+        if (per <= 2 * kGemmStagesShort)
+            gemm_tn_bf16_kernel<kGemmStagesShort><<<grid, 128, gemm_smem_bytes(kGemmStagesShort), st>>>(ta, tb, g);
         else
-            gemm_tn_bf16_kernel<kGemmStagesDeep><<<grid, 128, gemm_smem_bytes(kGemmStagesDeep), st>>>(ta, tb, a);
-    };
-    if (splits == 1) {
-        g.epilogue = epilogue; g.C = C; g.Cb = Cb;
-        launch(g);
-        return cudaGetLastError();
+            gemm_tn_bf16_kernel<kGemmStagesDeep><<<grid, 128, gemm_smem_bytes(kGemmStagesDeep), st>>>(ta, tb, g);
     }
-    if (!partial) return cudaErrorInvalidValue;
-    g.epilogue = kEpiPartialF32; g.C = partial; g.ldc = N;
-    launch(g);
     e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
+    if (e != cudaSuccess || splits == 1) return e;
     const long long total = (long long)M * N;
     splitk_reduce_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(partial, splits, M, N, epilogue, bias, C, Cb,
                                                                           ldc);
