@@ -278,7 +278,11 @@ __global__ void __launch_bounds__(128, 1) gemm_tn_bf16_kernel(const __grid_const
 //   warp 1 (leader): MMA issuer; tcgen05.commit returns each stage to both
 //           CTAs' producers and each finished accumulator to both epilogues
 //   warp 2: TMEM allocation
-//   warps 4-7: epilogue of the CTA's 128 rows
+//   warps 4-7: epilogue of the CTA's 128 rows: each warp's 32 rows leave 32
+//           columns at a time, from TMEM through a swizzled 4 KB buffer with
+//           a TMA store (FP32 outputs whose rows start on 16 bytes; else, and
+//           for BF16, one row segment per warp store, which took 1.2 us per 32
+//           columns and bound the short products: 512 x 32768 x 256 39 us)
 // An operand may be stored with its rows (M or N) contiguous instead of K
 // (MN-major): boxes of 64 rows x 64 K then land as 64 lines of 128 bytes, which
 // the descriptor addresses 8 K at a time (stride 1024) and 64 rows at a time
@@ -288,12 +292,15 @@ constexpr int kPairStages = 6;
 constexpr int kPairThreads = 256;
 constexpr int kPairStageBytes = 2 * kGemmTileBytes;  // A 16 KB, B at most 16 KB
 constexpr int kPairStagePitch = 33;
-constexpr int kPairSmem = kPairStages * kPairStageBytes + 4 * 32 * kPairStagePitch * 4 + 1024 + 256;
+constexpr int kPairStageBuf = 8192;  // per epilogue warp: two 4 KB store buffers, or one of 32 x 33 floats
+constexpr int kPairSmem = kPairStages * kPairStageBytes + 4 * kPairStageBuf + 1024 + 256;
+static_assert(32 * kPairStagePitch * 4 <= kPairStageBuf, "the row-by-row staging fits");
 
 struct PairArgs {
     GemmArgs g;
     int tile_n, tiles_m, tiles_n, splits;
     int a_mn, b_mn;  // operand stored [K][rows]
+    int tma_store;   // FP32 output through tmC
 };
 
 __device__ __forceinline__ uint64_t mn_desc(uint32_t saddr) {
@@ -342,17 +349,26 @@ __device__ __forceinline__ void mma_commit_pair(uint64_t* bar) {
         : "memory");
 }
 
+// TMA store of a 32 x 32 FP32 box; out-of-range rows and columns are dropped.
+__device__ __forceinline__ void tma_store_3d(const CUtensorMap* map, const void* src, int x, int y, int z) {
+    asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.tile.bulk_group [%0, {%1, %2, %3}], [%4];" ::"l"(
+                     (uint64_t)map),
+                 "r"(x), "r"(y), "r"(z), "r"(smem_u32(src))
+                 : "memory");
+    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+}
+
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar) {
     asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
     gemm_pair_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                          PairArgs a) {
+                          const __grid_constant__ CUtensorMap tmC, PairArgs a) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* base = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    float* staging = (float*)(base + kPairStages * kPairStageBytes);
-    uint64_t* full = (uint64_t*)(staging + 4 * 32 * kPairStagePitch);
+    uint8_t* staging = base + kPairStages * kPairStageBytes;
+    uint64_t* full = (uint64_t*)(staging + 4 * kPairStageBuf);
     uint64_t* empty = full + kPairStages;
     uint64_t* acc_full = empty + kPairStages;
     uint64_t* acc_empty = acc_full + 2;
@@ -455,8 +471,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
         __syncwarp();
     } else if (warp >= 4) {
         const int ew = warp & 3;  // the TMEM lanes this warp may read: 32 ew ..
-        float* stage = staging + ew * 32 * kPairStagePitch;
-        int n_item = 0;
+        float* stage = (float*)(staging + ew * kPairStageBuf);
+        int n_item = 0, n_store = 0;
         for (int item = pair; item < items; item += pairs, ++n_item) {
             const int split = item / tiles, tile = item % tiles;
             const int m0 = (tile % a.tiles_m) * 256 + (int)crank * 128 + ew * 32, n0 = (tile / a.tiles_m) * a.tile_n;
@@ -473,6 +489,27 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
                     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                     __syncwarp();
                     if (lane == 0) mbar_arrive_cluster(cta_map(&acc_empty[b], 0));
+                }
+                if (a.tma_store) {
+                    if (n0 + c >= g.N || m0 >= g.M) continue;  // uniform over the warp
+                    if (biasp && g.epilogue == kEpiBiasF32) {
+#pragma unroll
+                        for (int j = 0; j < 32; ++j) v[j] += n0 + c + j < g.N ? __ldg(&biasp[n0 + c + j]) : 0.0f;
+                    }
+                    float* const buf = stage + (n_store & 1) * 1024;
+                    // the store before last has read this buffer
+                    if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+                    __syncwarp();
+#pragma unroll
+                    for (int j = 0; j < 8; ++j)  // 16-byte chunk j of row `lane`, 128-byte swizzle
+                        *reinterpret_cast<float4*>(buf + lane * 32 + ((j ^ (lane & 7)) * 4)) =
+                            make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                    __syncwarp();
+                    if (lane == 0)
+                        tma_store_3d(&tmC, buf, n0 + c, m0, g.epilogue == kEpiPartialF32 ? split : 0);
+                    ++n_store;
+                    continue;
                 }
                 __syncwarp();
 #pragma unroll
@@ -499,6 +536,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kPairThreads, 1)
                 }
             }
         }
+        if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");  // the last stores are written
+        __syncwarp();
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();

@@ -391,10 +391,15 @@ cudaError_t launch_plan_pool(const PlanArgs* args, const int* order, const long 
 int plan_pool_max_blocks(int threads, bool all_kinds);
 
 // mlp.cu: C = A . B^T on the tensor cores (BF16 in, FP32 accumulate);
-// epilogue 0 = FP32 store, 1 = BF16 relu(x + bias), 2 = FP32 x + bias.
+// epilogue 0 = FP32 store, 1 = BF16 relu(x + bias), 2 = FP32 x + bias.  a_mn,
+// b_mn: the operand is stored [K][M] or [K][N].  partials_left (may be NULL):
+// receives the number of K-slices left unreduced in `partial` ([slices][M][N];
+// the caller applies the epilogue as it sums them in order), or 1 if C or Cb
+// was written.
 cudaError_t gemm_bf16_tn(int M, int N, int K, const __nv_bfloat16* A, const __nv_bfloat16* B, int epilogue,
                          const float* bias, float* C, __nv_bfloat16* Cb, int ldc, int splits, float* partial,
-                         int* error, cudaStream_t st, bool a_mn = false, bool b_mn = false);
+                         int* error, cudaStream_t st, bool a_mn = false, bool b_mn = false,
+                         int* partials_left = nullptr);
 
 // graph.cu: copies `count` appended samples (DEVICE [d][src_pitch]) into X
 // columns first.. and computes their goal flags; sets flags kSampleBadAppend

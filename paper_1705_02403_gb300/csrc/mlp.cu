@@ -49,6 +49,21 @@ cudaError_t make_map(CUtensorMap* map, const void* ptr, int rows, int cols, int 
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
+// Tensor map of an FP32 output [slices][rows][cols] (cols contiguous, row
+// stride ld floats) written in boxes of 32 x 32, 128-byte swizzle.
+cudaError_t make_out_map(CUtensorMap* map, float* ptr, int slices, int rows, int cols, int ld) {
+    EncodeTiledFn fn = encode_fn();
+    if (!fn) return cudaErrorNotSupported;
+    const cuuint64_t dims[3] = {(cuuint64_t)cols, (cuuint64_t)rows, (cuuint64_t)slices};
+    const cuuint64_t strides[2] = {(cuuint64_t)ld * 4, (cuuint64_t)ld * 4 * (cuuint64_t)rows};
+    const cuuint32_t box[3] = {32, 32, 1};
+    const cuuint32_t estr[3] = {1, 1, 1};
+    CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, ptr, dims, strides, box, estr,
+                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+
 int device_sms() {
     static std::atomic<int> cached{0};
     int sms = cached.load(std::memory_order_relaxed);
@@ -104,7 +119,7 @@ __global__ void splitk_reduce_kernel(const float* __restrict__ part, int splits,
 // deterministically.
 cudaError_t gemm_bf16_tn(int M, int N, int K, const __nv_bfloat16* A, const __nv_bfloat16* B, int epilogue,
                          const float* bias, float* C, __nv_bfloat16* Cb, int ldc, int splits, float* partial,
-                         int* error, cudaStream_t st, bool a_mn, bool b_mn) {
+                         int* error, cudaStream_t st, bool a_mn, bool b_mn, int* partials_left) {
     if (M <= 0 || N <= 0 || K <= 0 || (K % 8 != 0 && !(a_mn && b_mn))) return cudaErrorInvalidValue;
     static std::atomic<bool> attr_set{false};  // setting it twice is harmless
     if (!attr_set.load(std::memory_order_relaxed)) {
@@ -146,7 +161,12 @@ cudaError_t gemm_bf16_tn(int M, int N, int K, const __nv_bfloat16* A, const __nv
         if (e != cudaSuccess) return e;
         const long long items = (long long)p.tiles_m * p.tiles_n * splits;
         if (items > INT_MAX) return cudaErrorInvalidValue;
-        gemm_pair_bf16_kernel<<<2 * (int)std::min<long long>(items, pairs), kPairThreads, kPairSmem, st>>>(ta, tb, p);
+        // FP32 outputs leave by TMA where their rows start on 16 bytes
+        CUtensorMap tc;
+        std::memset(&tc, 0, sizeof(tc));
+        p.tma_store = g.epilogue != kEpiBiasReluBF16 && g.ldc % 4 == 0 && ((uintptr_t)g.C & 15) == 0 &&
+                      make_out_map(&tc, g.C, g.epilogue == kEpiPartialF32 ? splits : 1, M, N, g.ldc) == cudaSuccess;
+        gemm_pair_bf16_kernel<<<2 * (int)std::min<long long>(items, pairs), kPairThreads, kPairSmem, st>>>(ta, tb, tc, p);
     } else {
         e = make_map(&ta, A, M, K, kGemmBM);
         if (e == cudaSuccess) e = make_map(&tb, B, N, K, kGemmBN);
@@ -159,7 +179,8 @@ cudaError_t gemm_bf16_tn(int M, int N, int K, const __nv_bfloat16* A, const __nv
             gemm_tn_bf16_kernel<kGemmStagesDeep><<<grid, 128, gemm_smem_bytes(kGemmStagesDeep), st>>>(ta, tb, g);
     }
     e = cudaGetLastError();
-    if (e != cudaSuccess || splits == 1) return e;
+    if (partials_left) *partials_left = splits;
+    if (e != cudaSuccess || splits == 1 || partials_left) return e;
     const long long total = (long long)M * N;
     splitk_reduce_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(partial, splits, M, N, epilogue, bias, C, Cb,
                                                                           ldc);

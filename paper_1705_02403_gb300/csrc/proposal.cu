@@ -10,8 +10,9 @@
 //   logits = Z W3^T + b3                [B, C^3]
 // Training: softmax cross-entropy against a target distribution over cells,
 // backward through the same BF16 tensor-core GEMM with FP32 accumulation
-// (dW = dY^T X computed as GEMMs of transposed BF16 copies), AdamW on FP32
-// master weights, BF16 copies refreshed after every step.
+// (the transposed operands of dW = dY^T X and dX = dY W are read in place,
+// rows contiguous), AdamW on FP32 master weights, BF16 copies refreshed after
+// every step.
 #include <cmath>
 #include <cstdio>
 #include <atomic>
@@ -91,6 +92,42 @@ __global__ void __launch_bounds__(kVoxRows) voxelize_kernel(const EnvBoxes* __re
     }
 }
 
+// Sum of an output element's K-slices, in order: part[k * stride + t].
+__device__ __forceinline__ float slice_sum(const float* __restrict__ part, int splits, size_t stride, size_t t) {
+    float s = 0.0f;
+    for (int k = 0; k < splits; ++k) s += part[(size_t)k * stride + t];
+    return s;
+}
+
+// Layer 2's split-K reduction with its epilogue and the concatenation:
+// H2 = relu(sum + b2), Z = [H2, start/goal (6), zeros], one pass.
+__global__ void reduce_concat_kernel(const float* __restrict__ part, int splits, const float* __restrict__ b2,
+                                     const float* __restrict__ sg, int B, int H, int Dz, bf16* __restrict__ H2,
+                                     bf16* __restrict__ Z) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= B * Dz) return;
+    const int b = t / Dz, c = t % Dz;
+    bf16 v = __float2bfloat16_rn(0.0f);
+    if (c < H) {
+        v = __float2bfloat16_rn(fmaxf(slice_sum(part, splits, (size_t)B * H, (size_t)b * H + c) + b2[c], 0.0f));
+        H2[(size_t)b * H + c] = v;
+    } else if (c < H + 6) {
+        v = __float2bfloat16_rn(sg[b * 6 + (c - H)]);
+    }
+    Z[t] = v;
+}
+
+// Layer 3's split-K reduction with its bias, into the model's logits and the
+// caller's (may be NULL).
+__global__ void reduce_logits_kernel(const float* __restrict__ part, int splits, const float* __restrict__ b3, int B,
+                                     int Nc, float* __restrict__ logits, float* __restrict__ copy) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= B * Nc) return;
+    const float x = slice_sum(part, splits, (size_t)B * Nc, t) + b3[t % Nc];
+    logits[t] = x;
+    if (copy) copy[t] = x;
+}
+
 // Z = [H2, start/goal (6), zeros] in BF16.
 __global__ void concat_kernel(const bf16* __restrict__ H2, const float* __restrict__ sg, int B, int H, int Dz,
                               bf16* __restrict__ Z) {
@@ -103,122 +140,190 @@ __global__ void concat_kernel(const bf16* __restrict__ H2, const float* __restri
     Z[t] = v;
 }
 
-// [R, C] -> [C, R] through 32x32 shared-memory tiles.
-__global__ void transpose_bf16_kernel(const bf16* __restrict__ in, int R, int C, bf16* __restrict__ out) {
-    __shared__ bf16 tile[32][33];
-    const int c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
-    for (int y = threadIdx.y; y < 32; y += blockDim.y) {
-        const int r = r0 + y, c = c0 + threadIdx.x;
-        if (r < R && c < C) tile[y][threadIdx.x] = in[(size_t)r * C + c];
-    }
-    __syncthreads();
-    for (int y = threadIdx.y; y < 32; y += blockDim.y) {
-        const int c = c0 + y, r = r0 + threadIdx.x;
-        if (r < R && c < C) out[(size_t)c * R + r] = tile[threadIdx.x][y];
-    }
-}
-
 __global__ void f32_to_bf16_kernel(const float* __restrict__ in, long long n, bf16* __restrict__ out) {
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (t < n) out[t] = __float2bfloat16_rn(in[t]);
 }
 
-// Row-wise softmax cross-entropy: loss_b = -sum_c T_bc log softmax(l_b)_c and
-// dlogits = (softmax - T) / B (rounded to BF16 for the backward GEMMs).
-__global__ void softmax_xent_kernel(const float* __restrict__ logits, const float* __restrict__ T, int B, int Nc,
-                                    bf16* __restrict__ dlog, float* __restrict__ loss) {
+// Row-wise softmax cross-entropy, one block per row: loss_b =
+// -sum_c T_bc log softmax(l_b)_c and dlogits = (softmax - T) / B (rounded to
+// BF16 for the backward GEMMs).  With part, the row's logits are first summed
+// from layer 3's K-slices (plus b3) and stored.  1024 threads evaluate the
+// exponentials into shared memory; the sums run over 256 threads, thread t
+// taking c = t, t + 256, ... in order, then shuffles, then the eight warps.
+// (One pass over the row by 256 threads, reading the logits three times, took
+// 19.5 us at 256 rows of 4096.)
+// KEEP: the row stays in shared memory beside the terms (cells up to 29); else
+// it is read again from L2.
+constexpr int kXentThreads = 1024, kXentSums = 256;
+constexpr size_t kXentSmem = 200 * 1024;
+template <bool KEEP>
+__global__ void __launch_bounds__(kXentThreads) softmax_xent_kernel(const float* __restrict__ part, int splits,
+                                                                    const float* __restrict__ b3,
+                                                                    float* __restrict__ logits,
+                                                                    const float* __restrict__ T, int B, int Nc,
+                                                                    bf16* __restrict__ dlog, float* __restrict__ loss) {
+    extern __shared__ float term[];  // the terms of the running sum, then the row
+    float* const row = KEEP ? term + Nc : logits + (size_t)blockIdx.x * Nc;
     __shared__ float red[32];
-    const int b = blockIdx.x;
-    const float* l = logits + (size_t)b * Nc;
+    const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    float* l = logits + (size_t)b * Nc;
     const float* t = T + (size_t)b * Nc;
     float mx = -INFINITY;
-    for (int c = threadIdx.x; c < Nc; c += blockDim.x) mx = fmaxf(mx, l[c]);
-    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        float v = threadIdx.x < blockDim.x / 32 ? red[threadIdx.x] : -INFINITY;
-        for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-        red[0] = v;
+    for (int c = tid; c < Nc; c += kXentThreads) {
+        float x;
+        if (part) {
+            x = slice_sum(part, splits, (size_t)B * Nc, (size_t)b * Nc + c) + b3[c];
+            l[c] = x;
+        } else {
+            x = l[c];
+        }
+        if (KEEP) row[c] = x;
+        mx = fmaxf(mx, x);
     }
+    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if (lane == 0) red[warp] = mx;
     __syncthreads();
-    mx = red[0];
+    mx = red[lane];
+    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    for (int c = tid; c < Nc; c += kXentThreads) term[c] = expf(row[c] - mx);
     __syncthreads();
     float se = 0.0f;
-    for (int c = threadIdx.x; c < Nc; c += blockDim.x) se += expf(l[c] - mx);
+    if (tid < kXentSums) {
+        for (int c = tid; c < Nc; c += kXentSums) se += term[c];
+        for (int o = 16; o > 0; o >>= 1) se += __shfl_xor_sync(0xffffffffu, se, o);
+        if (lane == 0) red[warp] = se;
+    }
+    __syncthreads();
+    se = lane < kXentSums / 32 ? red[lane] : 0.0f;
     for (int o = 16; o > 0; o >>= 1) se += __shfl_xor_sync(0xffffffffu, se, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = se;
+    const float lse = mx + logf(se);
     __syncthreads();
-    if (threadIdx.x < 32) {
-        float v = threadIdx.x < blockDim.x / 32 ? red[threadIdx.x] : 0.0f;
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        red[0] = v;
+    for (int c = tid; c < Nc; c += kXentThreads) {
+        const float p = expf(row[c] - lse), tc = t[c];
+        term[c] = tc * (row[c] - lse);
+        dlog[(size_t)b * Nc + c] = __float2bfloat16_rn((p - tc) / (float)B);
     }
     __syncthreads();
-    const float lse = mx + logf(red[0]);
-    __syncthreads();
-    float lo = 0.0f;
-    for (int c = threadIdx.x; c < Nc; c += blockDim.x) {
-        const float p = expf(l[c] - lse);
-        lo -= t[c] * (l[c] - lse);
-        if (dlog) dlog[(size_t)b * Nc + c] = __float2bfloat16_rn((p - t[c]) / (float)B);
+    if (tid < kXentSums) {
+        float lo = 0.0f;
+        for (int c = tid; c < Nc; c += kXentSums) lo -= term[c];
+        for (int o = 16; o > 0; o >>= 1) lo += __shfl_xor_sync(0xffffffffu, lo, o);
+        if (lane == 0) red[warp] = lo;
     }
-    for (int o = 16; o > 0; o >>= 1) lo += __shfl_xor_sync(0xffffffffu, lo, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = lo;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        float s = 0.0f;
-        for (int w = 0; w < (int)(blockDim.x / 32); ++w) s += red[w];
-        loss[b] = s;
+    if (tid == 0) {
+        float sum = 0.0f;
+        for (int w = 0; w < kXentSums / 32; ++w) sum += red[w];
+        loss[b] = sum;
     }
 }
 
-// dpre = d[:, :H] * (act > 0) in BF16 (d has row stride ld).
-__global__ void relu_back_kernel(const float* __restrict__ d, int ld, const bf16* __restrict__ act, int B, int H,
-                                 bf16* __restrict__ dpre) {
+// dpre = d[:, :H] * (act > 0) in BF16, d [B][ld] summed from its K-slices.
+__global__ void reduce_relu_back_kernel(const float* __restrict__ part, int splits, int ld,
+                                        const bf16* __restrict__ act, int B, int H, bf16* __restrict__ dpre) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= B * H) return;
     const int b = t / H, c = t % H;
-    const float a = __bfloat162float(act[t]);
-    dpre[t] = __float2bfloat16_rn(a > 0.0f ? d[(size_t)b * ld + c] : 0.0f);
+    const float d = slice_sum(part, splits, (size_t)B * ld, (size_t)b * ld + c);
+    dpre[t] = __float2bfloat16_rn(__bfloat162float(act[t]) > 0.0f ? d : 0.0f);
 }
 
-// g[c] = sum_b d[b, c] (d BF16 [B, N] or FP32).
-// Column sums of a BF16 matrix [B][N] in FP32: a block of 32 x 8 threads takes
-// 32 columns, each thread a strided eighth of the rows, then the 8 partial
-// sums are added in a fixed order (deterministic).
-__global__ void __launch_bounds__(256) colsum_bf16_kernel(const bf16* __restrict__ d, int B, int N,
-                                                         float* __restrict__ g) {
+// Column sums of BF16 matrices [B][N] in FP32 (the bias gradients), up to
+// three matrices in one launch: a block of 32 x 8 threads takes 32 columns of
+// one, each thread a strided eighth of the rows, then the 8 partial sums are
+// added in a fixed order (deterministic).
+struct ColsumArgs {
+    const bf16* d[3];
+    float* g[3];
+    int N[3], first[4];  // first block of each matrix
+    int B;
+};
+__global__ void __launch_bounds__(256) colsum_bf16_kernel(ColsumArgs a) {
     __shared__ float part[8][33];
+    const int k = (int)blockIdx.x >= a.first[2] ? 2 : (int)blockIdx.x >= a.first[1] ? 1 : 0;
+    const bf16* d = a.d[k];
+    const int N = a.N[k];
     const int cx = threadIdx.x & 31, ry = threadIdx.x >> 5;
-    const int c = blockIdx.x * 32 + cx;
+    const int c = ((int)blockIdx.x - a.first[k]) * 32 + cx;
     float s = 0.0f;
     if (c < N)
-        for (int b = ry; b < B; b += 8) s += __bfloat162float(d[(size_t)b * N + c]);
+        for (int b = ry; b < a.B; b += 8) s += __bfloat162float(d[(size_t)b * N + c]);
     part[ry][cx] = s;
     __syncthreads();
     if (ry == 0 && c < N) {
         float t = part[0][cx];
-        for (int k = 1; k < 8; ++k) t += part[k][cx];
-        g[c] = t;
+        for (int w = 1; w < 8; ++w) t += part[w][cx];
+        a.g[k][c] = t;
     }
 }
 
-// AdamW (decoupled weight decay) on FP32 master weights; refreshes the BF16 copy.
-__global__ void adamw_kernel(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
-                             float* __restrict__ v, long long n, float lr, float b1, float b2, float eps, float wd,
-                             float c1, float c2, bf16* __restrict__ pb) {
-    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= n) return;
-    const float gt = g[t];
-    const float mt = b1 * m[t] + (1.0f - b1) * gt;
-    const float vt = b2 * v[t] + (1.0f - b2) * gt * gt;
-    m[t] = mt;
-    v[t] = vt;
-    float w = p[t] * (1.0f - lr * wd);
-    w -= lr * (mt / c1) / (sqrtf(vt / c2) + eps);
-    p[t] = w;
-    if (pb) pb[t] = __float2bfloat16_rn(w);
+// AdamW (decoupled weight decay) on FP32 master weights; refreshes the BF16
+// copies.  All tensors in one launch, four elements per thread and step (30
+// bytes an element move, so it is bound by HBM: one element per thread and a
+// launch per tensor took 128 us at 19.2 M parameters).  Nothing is updated if
+// a GEMM of the step gave up (err set).
+struct AdamTensor {
+    float *p, *m, *v;
+    const float* g;
+    bf16* pb;        // BF16 copy or NULL
+    long long n;
+    float wd;
+};
+struct AdamArgs {
+    AdamTensor t[6];
+    int first[7];  // first block of each tensor
+    float lr, b1, b2, eps, c1, c2;
+    const int* err;
+};
+constexpr int kAdamPerBlock = 256 * 8;
+
+__device__ __forceinline__ float adam_one(const AdamArgs& a, float wd, float p, float g, float& m, float& v) {
+    const float mt = a.b1 * m + (1.0f - a.b1) * g;
+    const float vt = a.b2 * v + (1.0f - a.b2) * g * g;
+    m = mt;
+    v = vt;
+    float w = p * (1.0f - a.lr * wd);
+    w -= a.lr * (mt / a.c1) / (sqrtf(vt / a.c2) + a.eps);
+    return w;
+}
+
+__global__ void __launch_bounds__(256) adamw_kernel(const __grid_constant__ AdamArgs a) {
+    if (__ldg(a.err) != 0) return;
+    int k = 0;
+    while (k < 5 && (int)blockIdx.x >= a.first[k + 1]) ++k;
+    const AdamTensor& t = a.t[k];
+    const long long base = (long long)((int)blockIdx.x - a.first[k]) * kAdamPerBlock;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const long long e = base + h * 1024 + threadIdx.x * 4;
+        if (e + 4 <= t.n) {  // the tensors are allocated by the library: 16-byte aligned
+            float4 p = *reinterpret_cast<const float4*>(t.p + e), m = *reinterpret_cast<const float4*>(t.m + e),
+                   v = *reinterpret_cast<const float4*>(t.v + e);
+            const float4 g = *reinterpret_cast<const float4*>(t.g + e);
+            p.x = adam_one(a, t.wd, p.x, g.x, m.x, v.x);
+            p.y = adam_one(a, t.wd, p.y, g.y, m.y, v.y);
+            p.z = adam_one(a, t.wd, p.z, g.z, m.z, v.z);
+            p.w = adam_one(a, t.wd, p.w, g.w, m.w, v.w);
+            *reinterpret_cast<float4*>(t.m + e) = m;
+            *reinterpret_cast<float4*>(t.v + e) = v;
+            *reinterpret_cast<float4*>(t.p + e) = p;
+            if (t.pb) {
+                __nv_bfloat162 lo = __floats2bfloat162_rn(p.x, p.y), hi = __floats2bfloat162_rn(p.z, p.w);
+                *reinterpret_cast<uint2*>(t.pb + e) =
+                    make_uint2(*reinterpret_cast<unsigned*>(&lo), *reinterpret_cast<unsigned*>(&hi));
+            }
+        } else {
+            for (long long j = e; j < t.n; ++j) {
+                float m = t.m[j], v = t.v[j];
+                const float w = adam_one(a, t.wd, t.p[j], t.g[j], m, v);
+                t.m[j] = m;
+                t.v[j] = v;
+                t.p[j] = w;
+                if (t.pb) t.pb[j] = __float2bfloat16_rn(w);
+            }
+        }
+    }
 }
 
 // Deterministic N(0, std^2) initial weights from Philox (Box-Muller).
@@ -403,16 +508,17 @@ struct gmt_model {
     uint64_t seed = 0;
     // parameters (FP32 masters), BF16 copies, Adam moments, gradients
     float *W1 = nullptr, *b1 = nullptr, *W2 = nullptr, *b2 = nullptr, *W3 = nullptr, *b3 = nullptr;
-    bf16 *W1b = nullptr, *W2b = nullptr, *W2tb = nullptr, *W3b = nullptr, *W3tb = nullptr;
+    bf16 *W1b = nullptr, *W2b = nullptr, *W3b = nullptr;
     float* mom[6] = {};
     float* vel[6] = {};
     float *gW1 = nullptr, *gb1 = nullptr, *gW2 = nullptr, *gb2 = nullptr, *gW3 = nullptr, *gb3 = nullptr;
     // activations for up to maxB environments
-    bf16 *Xt = nullptr, *H1 = nullptr, *H1t = nullptr, *H2 = nullptr, *Z = nullptr, *Zt = nullptr;
-    bf16 *dlog = nullptr, *dlogt = nullptr, *dH2 = nullptr, *dH2t = nullptr, *dH1p = nullptr, *dH1pt = nullptr;
+    bf16 *H1 = nullptr, *H2 = nullptr, *Z = nullptr;
+    bf16 *dlog = nullptr, *dH2 = nullptr, *dH1p = nullptr;
     float *logits = nullptr, *dZ = nullptr, *dH1 = nullptr, *ws = nullptr, *loss = nullptr;
     size_t ws_floats = 0;
-    int* err = nullptr;
+    int* err = nullptr;             // right behind the losses: one copy brings both back
+    float* h_out = nullptr;         // pinned: the losses and the error flag of a call
     // proposal scratch
     bf16* pvox = nullptr;
     float* psg = nullptr;
@@ -435,6 +541,7 @@ struct gmt_model {
         if (envs) cudaFree(envs);
         if (penv) cudaFree(penv);
         if (pin) cudaFreeHost(pin);
+        if (h_out) cudaFreeHost(h_out);
         if (pin_ev) cudaEventDestroy(pin_ev);
     }
 };
@@ -462,12 +569,6 @@ gmt_status mcuda(cudaError_t e, const char* what) {
         if (e_ != cudaSuccess) return mcuda(e_, what);  \
     } while (0)
 
-cudaError_t transpose(const bf16* in, int R, int C, bf16* out, cudaStream_t st) {
-    dim3 grid((C + 31) / 32, (R + 31) / 32);
-    transpose_bf16_kernel<<<grid, dim3(32, 8), 0, st>>>(in, R, C, out);
-    return cudaGetLastError();
-}
-
 // Split-K factor: enough K-slices that the CTAs cover the SMs once (each
 // slice at least 4 K-blocks deep).
 int splits_for(int M, int N, int K) {
@@ -488,68 +589,134 @@ int splits_for(int M, int N, int K) {
     return s < 1 ? 1 : s;
 }
 
+// left (may be NULL): leaves the K-slices in m->ws, see gemm_bf16_tn.
 cudaError_t gemm(gmt_model* m, int M, int N, int K, const bf16* A, const bf16* B, int epi, const float* bias,
-                 float* C, bf16* Cb, cudaStream_t st) {
+                 float* C, bf16* Cb, cudaStream_t st, bool a_mn = false, bool b_mn = false, int* left = nullptr) {
     int s = splits_for(M, N, K);
     while (s > 1 && (size_t)s * M * N > m->ws_floats) s /= 2;
-    return gemm_bf16_tn(M, N, K, A, B, epi, bias, C, Cb, N, s, m->ws, m->err, st);
+    return gemm_bf16_tn(M, N, K, A, B, epi, bias, C, Cb, N, s, m->ws, m->err, st, a_mn, b_mn, left);
 }
 
-// Refresh the BF16 copies (and transposed copies) of the weights.
+// Refresh the BF16 copies of the weights.
 cudaError_t refresh_copies(gmt_model* m, cudaStream_t st) {
     f32_to_bf16_kernel<<<blocks_for(m->n(0), 256), 256, 0, st>>>(m->W1, m->n(0), m->W1b);
     f32_to_bf16_kernel<<<blocks_for(m->n(2), 256), 256, 0, st>>>(m->W2, m->n(2), m->W2b);
     f32_to_bf16_kernel<<<blocks_for(m->n(4), 256), 256, 0, st>>>(m->W3, m->n(4), m->W3b);
-    cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess) e = transpose(m->W2b, m->H, m->H, m->W2tb, st);
-    if (e == cudaSuccess) e = transpose(m->W3b, m->Nc, m->Dz, m->W3tb, st);
-    return e;
+    return cudaGetLastError();
 }
 
-gmt_status forward(gmt_model* m, int B, const bf16* X, const float* sg, cudaStream_t st) {
+// Layers 1 and 2 and the concatenation (H1, H2, Z), then layer 3's product:
+// *left receives its unreduced K-slices in m->ws, or 1 if the logits are there.
+gmt_status forward_body(gmt_model* m, int B, const bf16* X, const float* sg, int* left, cudaStream_t st) {
     MCUDA(gemm(m, B, m->H, m->Din, X, m->W1b, 1, m->b1, nullptr, m->H1, st), "layer 1 GEMM");
-    MCUDA(gemm(m, B, m->H, m->H, m->H1, m->W2b, 1, m->b2, nullptr, m->H2, st), "layer 2 GEMM");
-    concat_kernel<<<blocks_for((long long)B * m->Dz, 256), 256, 0, st>>>(m->H2, sg, B, m->H, m->Dz, m->Z);
+    int slices = 1;
+    MCUDA(gemm(m, B, m->H, m->H, m->H1, m->W2b, 1, m->b2, nullptr, m->H2, st, false, false, &slices), "layer 2 GEMM");
+    const unsigned blocks = blocks_for((long long)B * m->Dz, 256);
+    if (slices > 1)
+        reduce_concat_kernel<<<blocks, 256, 0, st>>>(m->ws, slices, m->b2, sg, B, m->H, m->Dz, m->H2, m->Z);
+    else
+        concat_kernel<<<blocks, 256, 0, st>>>(m->H2, sg, B, m->H, m->Dz, m->Z);
     MCUDA(cudaGetLastError(), "concat");
-    MCUDA(gemm(m, B, m->Nc, m->Dz, m->Z, m->W3b, 2, m->b3, m->logits, nullptr, st), "layer 3 GEMM");
+    MCUDA(gemm(m, B, m->Nc, m->Dz, m->Z, m->W3b, 2, m->b3, m->logits, nullptr, st, false, false, left),
+          "layer 3 GEMM");
     return GMT_OK;
 }
 
-gmt_status backward(gmt_model* m, int B, const bf16* X, const float* target, cudaStream_t st) {
-    softmax_xent_kernel<<<B, 256, 0, st>>>(m->logits, target, B, m->Nc, m->dlog, m->loss);
+// copy (may be NULL): receives the logits too.
+gmt_status forward(gmt_model* m, int B, const bf16* X, const float* sg, float* copy, cudaStream_t st) {
+    int left = 1;
+    gmt_status s = forward_body(m, B, X, sg, &left, st);
+    if (s != GMT_OK) return s;
+    const long long n = (long long)B * m->Nc;
+    if (left > 1) {
+        reduce_logits_kernel<<<blocks_for(n, 256), 256, 0, st>>>(m->ws, left, m->b3, B, m->Nc, m->logits, copy);
+        MCUDA(cudaGetLastError(), "layer 3 reduction");
+    } else if (copy) {
+        MCUDA(cudaMemcpyAsync(copy, m->logits, (size_t)n * sizeof(float), cudaMemcpyDeviceToDevice, st),
+              "logits copy");
+    }
+    return GMT_OK;
+}
+
+// Forward and backward: logits, losses, gradients.  The gradients' products
+// read dY, the activations and the weights where they are, rows contiguous
+// (MN-major), so nothing is transposed.
+gmt_status forward_backward(gmt_model* m, int B, const bf16* X, const float* sg, const float* target,
+                            cudaStream_t st) {
+    int left = 1;
+    gmt_status s = forward_body(m, B, X, sg, &left, st);
+    if (s != GMT_OK) return s;
+    const size_t row_bytes = (size_t)m->Nc * sizeof(float);
+    const bool keep = 2 * row_bytes <= kXentSmem;
+    static std::atomic<bool> attr_set{false};
+    if (!attr_set.load(std::memory_order_relaxed)) {
+        MCUDA(cudaFuncSetAttribute(softmax_xent_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kXentSmem),
+              "softmax kernel attribute");
+        MCUDA(cudaFuncSetAttribute(softmax_xent_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kXentSmem),
+              "softmax kernel attribute");
+        attr_set.store(true, std::memory_order_relaxed);
+    }
+    const float* const slices = left > 1 ? m->ws : nullptr;
+    if (keep)
+        softmax_xent_kernel<true><<<B, kXentThreads, 2 * row_bytes, st>>>(slices, left, m->b3, m->logits, target, B, m->Nc,
+                                                                          m->dlog, m->loss);
+    else
+        softmax_xent_kernel<false><<<B, kXentThreads, row_bytes, st>>>(slices, left, m->b3, m->logits, target, B, m->Nc,
+                                                                       m->dlog, m->loss);
     MCUDA(cudaGetLastError(), "softmax cross-entropy");
+    // batches are multiples of 8 environments (as when the gradients' operands
+    // were copied to rows of B)
+    if (B % 8) return mcuda(cudaErrorInvalidValue, "dW3 GEMM");
+    const unsigned relu_blocks = blocks_for((long long)B * m->H, 256);
     // layer 3
-    MCUDA(transpose(m->dlog, B, m->Nc, m->dlogt, st), "transpose");
-    MCUDA(transpose(m->Z, B, m->Dz, m->Zt, st), "transpose");
-    MCUDA(gemm(m, m->Nc, m->Dz, B, m->dlogt, m->Zt, 0, nullptr, m->gW3, nullptr, st), "dW3 GEMM");
-    colsum_bf16_kernel<<<blocks_for(m->Nc, 32), 256, 0, st>>>(m->dlog, B, m->Nc, m->gb3);
-    MCUDA(gemm(m, B, m->Dz, m->Nc, m->dlog, m->W3tb, 0, nullptr, m->dZ, nullptr, st), "dZ GEMM");
+    MCUDA(gemm(m, m->Nc, m->Dz, B, m->dlog, m->Z, 0, nullptr, m->gW3, nullptr, st, true, true), "dW3 GEMM");
+    MCUDA(gemm(m, B, m->Dz, m->Nc, m->dlog, m->W3b, 0, nullptr, m->dZ, nullptr, st, false, true, &left), "dZ GEMM");
     // layer 2
-    relu_back_kernel<<<blocks_for((long long)B * m->H, 256), 256, 0, st>>>(m->dZ, m->Dz, m->H2, B, m->H, m->dH2);
+    reduce_relu_back_kernel<<<relu_blocks, 256, 0, st>>>(left > 1 ? m->ws : m->dZ, left, m->Dz, m->H2, B, m->H, m->dH2);
     MCUDA(cudaGetLastError(), "relu backward");
-    MCUDA(transpose(m->dH2, B, m->H, m->dH2t, st), "transpose");
-    MCUDA(transpose(m->H1, B, m->H, m->H1t, st), "transpose");
-    MCUDA(gemm(m, m->H, m->H, B, m->dH2t, m->H1t, 0, nullptr, m->gW2, nullptr, st), "dW2 GEMM");
-    colsum_bf16_kernel<<<blocks_for(m->H, 32), 256, 0, st>>>(m->dH2, B, m->H, m->gb2);
-    MCUDA(gemm(m, B, m->H, m->H, m->dH2, m->W2tb, 0, nullptr, m->dH1, nullptr, st), "dH1 GEMM");
+    MCUDA(gemm(m, m->H, m->H, B, m->dH2, m->H1, 0, nullptr, m->gW2, nullptr, st, true, true), "dW2 GEMM");
+    MCUDA(gemm(m, B, m->H, m->H, m->dH2, m->W2b, 0, nullptr, m->dH1, nullptr, st, false, true, &left), "dH1 GEMM");
     // layer 1
-    relu_back_kernel<<<blocks_for((long long)B * m->H, 256), 256, 0, st>>>(m->dH1, m->H, m->H1, B, m->H, m->dH1p);
+    reduce_relu_back_kernel<<<relu_blocks, 256, 0, st>>>(left > 1 ? m->ws : m->dH1, left, m->H, m->H1, B, m->H,
+                                                         m->dH1p);
     MCUDA(cudaGetLastError(), "relu backward");
-    MCUDA(transpose(m->dH1p, B, m->H, m->dH1pt, st), "transpose");
-    MCUDA(transpose(X, B, m->Din, m->Xt, st), "transpose");
-    MCUDA(gemm(m, m->H, m->Din, B, m->dH1pt, m->Xt, 0, nullptr, m->gW1, nullptr, st), "dW1 GEMM");
-    colsum_bf16_kernel<<<blocks_for(m->H, 32), 256, 0, st>>>(m->dH1p, B, m->H, m->gb1);
+    MCUDA(gemm(m, m->H, m->Din, B, m->dH1p, X, 0, nullptr, m->gW1, nullptr, st, true, true), "dW1 GEMM");
+    ColsumArgs c;
+    c.B = B;
+    const bf16* d[3] = {m->dlog, m->dH2, m->dH1p};
+    float* g[3] = {m->gb3, m->gb2, m->gb1};
+    const int n[3] = {m->Nc, m->H, m->H};
+    c.first[0] = 0;
+    for (int k = 0; k < 3; ++k) {
+        c.d[k] = d[k];
+        c.g[k] = g[k];
+        c.N[k] = n[k];
+        c.first[k + 1] = c.first[k] + (n[k] + 31) / 32;
+    }
+    colsum_bf16_kernel<<<c.first[3], 256, 0, st>>>(c);
     MCUDA(cudaGetLastError(), "bias gradients");
     return GMT_OK;
 }
 
-gmt_status check_err(gmt_model* m, cudaStream_t st) {
-    int h = 0;
-    MCUDA(cudaMemcpyAsync(&h, m->err, sizeof(int), cudaMemcpyDeviceToHost, st), "error flag");
-    MCUDA(cudaStreamSynchronize(st), "model step");
+// Waits for the call's work; the error flag and, with B > 0, the first B
+// losses come back in one copy (they end the loss array: the flag is its last
+// word).  mean_loss may be NULL.
+gmt_status finish(gmt_model* m, int B, float* mean_loss, cudaStream_t st, const char* what) {
+    const int from = B > 0 ? 0 : m->maxB;
+    MCUDA(cudaMemcpyAsync(m->h_out + from, m->loss + from, (size_t)(m->maxB + 1 - from) * sizeof(float),
+                          cudaMemcpyDeviceToHost, st),
+          "result readback");
+    MCUDA(cudaStreamSynchronize(st), what);
+    int h;
+    std::memcpy(&h, m->h_out + m->maxB, sizeof(h));
     if (h) {
         cudaMemsetAsync(m->err, 0, sizeof(int), st);
         return mfail(GMT_ERR_TIMEOUT, "a tensor-core GEMM wait ran out");
+    }
+    if (mean_loss && B > 0) {
+        double a = 0.0;
+        for (int b = 0; b < B; ++b) a += m->h_out[b];
+        *mean_loss = (float)(a / B);
     }
     return GMT_OK;
 }
@@ -622,17 +789,18 @@ gmt_status propose_impl(gmt_model* m, int B, const gmt_space* spaces, const gmt_
         voxelize_kernel<<<dim3(blocks_for((long long)m->G * m->G, kVoxRows), nb), kVoxRows, 0, st>>>(m->envs + b0, m->G,
                                                                                                m->pvox);
         MCUDA(cudaGetLastError(), "voxelize kernel");
-        gmt_status s = forward(m, nb, m->pvox, m->psg, st);
+        gmt_status s = forward(m, nb, m->pvox, m->psg, nullptr, st);
         if (s != GMT_OK) return s;
         proposal_sample_kernel<<<nb, 1024, smem, st>>>(m->logits, m->Nc, m->C, m->penv + b0, count,
                                                                        65536, pitch, m->err);
         MCUDA(cudaGetLastError(), "proposal kernel");
     }
-    int h = 0;
-    MCUDA(cudaMemcpyAsync(&h, m->err, sizeof(int), cudaMemcpyDeviceToHost, st), "flag readback");
+    MCUDA(cudaMemcpyAsync(m->h_out + m->maxB, m->err, sizeof(int), cudaMemcpyDeviceToHost, st), "flag readback");
     MCUDA(cudaStreamSynchronize(st), "proposal");
+    int h;
+    std::memcpy(&h, m->h_out + m->maxB, sizeof(h));
     if (h) {
-        cudaMemset(m->err, 0, sizeof(int));
+        cudaMemsetAsync(m->err, 0, sizeof(int), st);
         return mfail(GMT_ERR_INVALID, "a proposal sample exhausted its attempts (or a GEMM wait ran out)");
     }
     return GMT_OK;
@@ -663,14 +831,18 @@ gmt_status gmt_model_create(const gmt_model_config* cfg, gmt_model** out) {
         if (e == cudaSuccess) e = mk(m, &m->vel[i], m->n(i));
         if (e != cudaSuccess) return fail_delete(mcuda(e, "model allocation"));
     }
-    MK(W1b, m->n(0)); MK(W2b, m->n(2)); MK(W2tb, m->n(2)); MK(W3b, m->n(4)); MK(W3tb, m->n(4));
-    MK(Xt, (size_t)B * m->Din); MK(H1, (size_t)B * m->H); MK(H1t, (size_t)B * m->H); MK(H2, (size_t)B * m->H);
-    MK(Z, (size_t)B * m->Dz); MK(Zt, (size_t)B * m->Dz); MK(dlog, (size_t)B * m->Nc); MK(dlogt, (size_t)B * m->Nc);
-    MK(dH2, (size_t)B * m->H); MK(dH2t, (size_t)B * m->H); MK(dH1p, (size_t)B * m->H); MK(dH1pt, (size_t)B * m->H);
-    MK(logits, (size_t)B * m->Nc); MK(dZ, (size_t)B * m->Dz); MK(dH1, (size_t)B * m->H); MK(loss, B);
+    MK(W1b, m->n(0)); MK(W2b, m->n(2)); MK(W3b, m->n(4));
+    MK(H1, (size_t)B * m->H); MK(H2, (size_t)B * m->H); MK(Z, (size_t)B * m->Dz);
+    MK(dlog, (size_t)B * m->Nc); MK(dH2, (size_t)B * m->H); MK(dH1p, (size_t)B * m->H);
+    MK(logits, (size_t)B * m->Nc); MK(dZ, (size_t)B * m->Dz); MK(dH1, (size_t)B * m->H);
+    MK(loss, (size_t)B + 1);
+    m->err = (int*)(m->loss + B);
     m->ws_floats = (size_t)16 * std::max((size_t)B * m->H, (size_t)B * m->Dz) + (size_t)4 * B * m->Nc;
     MK(ws, m->ws_floats);
-    MK(err, 1);
+    if (cudaMallocHost((void**)&m->h_out, ((size_t)B + 1) * sizeof(float)) != cudaSuccess) {
+        cudaGetLastError();
+        return fail_delete(mfail(GMT_ERR_OOM, "model allocation: pinned memory"));
+    }
     MK(pvox, (size_t)B * m->Din);
     MK(psg, (size_t)B * 6);
 #undef MK
@@ -732,12 +904,8 @@ gmt_status gmt_model_forward(gmt_model* m, int32_t B, const void* voxels, const 
                              gmt_stream stream) {
     if (!m || B < 1 || B > m->maxB || !voxels || !start_goal) return mfail(GMT_ERR_INVALID, "bad forward arguments");
     cudaStream_t st = (cudaStream_t)stream;
-    gmt_status s = forward(m, B, (const bf16*)voxels, start_goal, st);
-    if (s != GMT_OK) return s;
-    if (logits)
-        MCUDA(cudaMemcpyAsync(logits, m->logits, (size_t)B * m->Nc * sizeof(float), cudaMemcpyDeviceToDevice, st),
-              "logits copy");
-    return check_err(m, st);
+    gmt_status s = forward(m, B, (const bf16*)voxels, start_goal, logits, st);
+    return s != GMT_OK ? s : finish(m, 0, nullptr, st, "forward pass");
 }
 
 gmt_status gmt_model_backward(gmt_model* m, int32_t B, const void* voxels, const float* start_goal,
@@ -745,41 +913,37 @@ gmt_status gmt_model_backward(gmt_model* m, int32_t B, const void* voxels, const
     if (!m || B < 1 || B > m->maxB || !voxels || !start_goal || !target)
         return mfail(GMT_ERR_INVALID, "bad backward arguments");
     cudaStream_t st = (cudaStream_t)stream;
-    gmt_status s = forward(m, B, (const bf16*)voxels, start_goal, st);
-    if (s == GMT_OK) s = backward(m, B, (const bf16*)voxels, target, st);
-    if (s != GMT_OK) return s;
-    std::vector<float> l(B);
-    MCUDA(cudaMemcpyAsync(l.data(), m->loss, B * sizeof(float), cudaMemcpyDeviceToHost, st), "loss readback");
-    s = check_err(m, st);
-    if (s != GMT_OK) return s;
-    if (mean_loss) {
-        double a = 0.0;
-        for (float x : l) a += x;
-        *mean_loss = (float)(a / B);
-    }
-    return GMT_OK;
+    gmt_status s = forward_backward(m, B, (const bf16*)voxels, start_goal, target, st);
+    return s != GMT_OK ? s : finish(m, B, mean_loss, st, "model step");
 }
 
 gmt_status gmt_model_train_step(gmt_model* m, int32_t B, const void* voxels, const float* start_goal,
                                 const float* target, float lr, float weight_decay, float* mean_loss,
                                 gmt_stream stream) {
-    gmt_status s = gmt_model_backward(m, B, voxels, start_goal, target, mean_loss, stream);
-    if (s != GMT_OK) return s;
+    if (!m || B < 1 || B > m->maxB || !voxels || !start_goal || !target)
+        return mfail(GMT_ERR_INVALID, "bad backward arguments");
     cudaStream_t st = (cudaStream_t)stream;
-    m->step += 1;
-    const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
-    const float c1 = 1.0f - powf(b1, (float)m->step), c2 = 1.0f - powf(b2, (float)m->step);
+    gmt_status s = forward_backward(m, B, (const bf16*)voxels, start_goal, target, st);
+    if (s != GMT_OK) return s;
+    // queued behind the gradients, without a host wait in between: the kernel
+    // leaves everything as it is if a GEMM gave up
+    const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f, step = (float)(m->step + 1);
+    AdamArgs a;
+    a.lr = lr; a.b1 = b1; a.b2 = b2; a.eps = eps; a.err = m->err;
+    a.c1 = 1.0f - powf(b1, step);
+    a.c2 = 1.0f - powf(b2, step);
     bf16* copies[6] = {m->W1b, nullptr, m->W2b, nullptr, m->W3b, nullptr};
+    a.first[0] = 0;
     for (int i = 0; i < 6; ++i) {
-        const float wd = (i % 2 == 0) ? weight_decay : 0.0f;
-        adamw_kernel<<<blocks_for(m->n(i), 256), 256, 0, st>>>(m->param(i), m->grad(i), m->mom[i], m->vel[i], m->n(i),
-                                                               lr, b1, b2, eps, wd, c1, c2, copies[i]);
+        a.t[i] = AdamTensor{m->param(i), m->mom[i], m->vel[i], m->grad(i), copies[i], m->n(i),
+                            (i % 2 == 0) ? weight_decay : 0.0f};
+        a.first[i + 1] = a.first[i] + (int)blocks_for(m->n(i), kAdamPerBlock);
     }
+    adamw_kernel<<<a.first[6], 256, 0, st>>>(a);
     MCUDA(cudaGetLastError(), "AdamW");
-    MCUDA(transpose(m->W2b, m->H, m->H, m->W2tb, st), "transpose");
-    MCUDA(transpose(m->W3b, m->Nc, m->Dz, m->W3tb, st), "transpose");
-    MCUDA(cudaStreamSynchronize(st), "train step");
-    return GMT_OK;
+    s = finish(m, B, mean_loss, st, "train step");
+    if (s == GMT_OK) m->step += 1;
+    return s;
 }
 
 gmt_status gmt_model_save(const gmt_model* m, const char* path) {
