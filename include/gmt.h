@@ -307,13 +307,11 @@ gmt_status gmt_batch_get_view(const gmt_batch* batch, int32_t k, gmt_graph_view*
 
 /* Plan-stage scheme of a batch.
  *   GMT_BATCH_TEAMS: one persistent launch for every query of the batch; a
- *     team (a CTA or a cluster) runs one query at a time, one team barrier per
- *     Algorithm 1 iteration (double-buffered open-set snapshot; candidates
- *     are pulled from a team-wide queue as soon as they are claimed).  With
- *     one-CTA teams, when the largest query's wavefront state fits in a CTA's
- *     shared memory (about 36 bytes per node), each CTA keeps its query's
- *     whole state there (two barriers per iteration, every step but the CSR
- *     and sample reads on chip).
+ *     team (a CTA or a cluster) runs one query at a time, with the query's
+ *     wavefront state in the team's shared memory (two team barriers per
+ *     Algorithm 1 iteration) when the batch's largest query fits (about 220 KB
+ *     per CTA: 5 bytes per node in every CTA of a cluster, and 12 per node of
+ *     the CTA's share), else in device memory.
  *   GMT_BATCH_LOCKSTEP: one cooperative grid runs up to 512 queries at once,
  *     one Algorithm 1 iteration of every live query per grid step (two
  *     bounded grid barriers per step), so small groups of many queries fill
@@ -323,7 +321,8 @@ gmt_status gmt_batch_get_view(const gmt_batch* batch, int32_t k, gmt_graph_view*
  *     selection over 32 open entries, the push of one group node, the lazy
  *     parent and check of one candidate) that any warp may take, so queries
  *     advance without team barriers and without waiting for one another.
- *   GMT_BATCH_AUTO: the autotuner's choice; before tuning, teams of 4 CTAs. */
+ *   GMT_BATCH_AUTO: the autotuner's choice; before tuning, teams of 2 to 16 CTAs
+ *     by the number of queries and their sizes. */
 typedef enum { GMT_BATCH_AUTO = 0, GMT_BATCH_TEAMS = 1, GMT_BATCH_LOCKSTEP = 2, GMT_BATCH_POOL = 3 } gmt_batch_mode;
 gmt_status gmt_batch_set_mode(gmt_batch* batch, int32_t mode);
 

@@ -426,6 +426,7 @@ struct gmt_batch {
     DevBuf p_args, p_order, p_ecum, p_q, p_ctl, p_scratch;  // pool scheme
     int lock_chunks = 0;
     int max_n = 0;  // largest N of the batch (team scratch slices)
+    int max_scratch = 0;  // teams with a scratch slice
     cudaEvent_t ev_plan[2] = {nullptr, nullptr};  // around the plan stage of every call
     PlanCtl* h_ctl = nullptr;
     int* h_rows = nullptr;  // [q] edge counts, then [q] sampling flags
@@ -521,8 +522,8 @@ cudaError_t record_plan_event(cudaEvent_t e, cudaStream_t st) {
                                                : cudaEventRecord(e, st);
 }
 
-// Untuned choice: teams of 4 CTAs x 512 threads (measured fastest on the
-// 256-query uneven batch; the autotuner compares every scheme and shape).
+// Untuned choice: teams (untuned_shape; the autotuner compares every scheme
+// and shape).
 int plan_mode(const gmt_batch* b) {
     if (b->mode != GMT_BATCH_AUTO) return b->mode;
     if (b->tuned_mode != GMT_BATCH_AUTO) return b->tuned_mode;
@@ -551,27 +552,66 @@ void lock_shape(const gmt_batch* b, const Group& g, int* threads, int* blocks) {
     *blocks = plan_lockstep_max_blocks(g.kind, g.dp, t);
 }
 
-// Dynamic shared memory of the batched team kernel: the most any query asks
-// for (its staged boxes, or the parent copy of its path walk).
-size_t batch_smem(const gmt_batch* b) {
-    size_t smem = 16;
+// Dynamic shared memory of the batched team kernel with `cluster` CTAs per
+// team, the most any query asks for: its wavefront state (*local) when every
+// query's fits, else its staged boxes or the parent copy of its path walk.
+size_t batch_smem(const gmt_batch* b, int cluster, bool* local) {
+    size_t state = 16, scratch = 16;
+    *local = true;
     for (int k = 0; k < b->q; ++k) {
-        const int dp = b->queries[k].space.pos_dim, nb = b->queries[k].boxes.count;
-        smem = std::max(smem, plan_smem_bytes(nb <= smem_box_cap(dp) ? nb : 0, dp, b->N[k]));
+        const gmt_space& sp = b->queries[k].space;
+        const int dp = sp.pos_dim, nb = b->queries[k].boxes.count;
+        scratch = std::max(scratch, plan_smem_bytes(nb <= smem_box_cap(dp) ? nb : 0, dp, b->N[k]));
+        if (!*local) continue;
+        const size_t s = plan_local_bytes(sp.kind, sp.dim, dp, b->N[k], nb, std::max(cluster, 1));
+        if (s == SIZE_MAX) *local = false;
+        state = std::max(state, s);
     }
-    return smem;
+    return *local ? state : scratch;
+}
+
+int batch_max_teams(const gmt_batch* b, int cluster, int threads) {
+    bool local;
+    const size_t smem = batch_smem(b, cluster, &local);
+    return plan_batch_max_teams(threads, cluster, smem, local, pool_all_kinds(b));
+}
+
+// The untuned shape.  Pairs of CTAs with 1024 threads when there are more
+// queries than larger teams, else the largest team that leaves every query one
+// of its own; 256 threads for queries of at most 1025 nodes, whose iterations
+// hold too little work for more warps; more CTAs where the largest query's
+// state needs them, and teams of 4 x 512 when it fits none (the scratch kernel's
+// best).  Plan stage on one GB300, 256 uneven queries up to 16385 nodes: 2 x
+// 1024 1.44 ms, 4 x 1024 1.93, 8 x 512 2.02, 2 x 512 2.45; 200 of 2049: 0.666,
+// 0.944, 0.981, 0.731; 32 of 4097: 4 x 1024 0.268, 8 x 512 0.282, 2 x 1024
+// 0.395; 200 of 513: 2 x 256 0.203, 2 x 1024 0.281.
+void untuned_shape(const gmt_batch* b, int* cluster, int* threads) {
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    int c = 2;
+    while (c < 16 && sms / (2 * c) >= b->q) c *= 2;
+    bool local = false;
+    for (; c <= 16; c *= 2) {
+        batch_smem(b, c, &local);
+        if (local) break;
+    }
+    *cluster = local ? c : 4;
+    *threads = !local ? 512 : b->max_n <= 1025 ? 256 : 1024;
 }
 
 // Plan-stage launch shape of the teams scheme: (cluster, threads, teams).
 void plan_shape(const gmt_batch* b, int* cluster, int* threads, int* teams) {
-    int c = b->cluster > 0 ? b->cluster : (b->tuned_cluster > 0 ? b->tuned_cluster : 4);
-    int t = b->threads > 0 ? b->threads : (b->tuned_threads > 0 ? b->tuned_threads : 512);
-    const size_t smem = batch_smem(b);
-    const bool all = pool_all_kinds(b);
-    int n = plan_batch_max_teams(t, c, smem, b->max_n, true, all);
+    int c, t;
+    untuned_shape(b, &c, &t);
+    if (b->tuned_cluster > 0) c = b->tuned_cluster;
+    if (b->tuned_threads > 0) t = b->tuned_threads;
+    if (b->cluster > 0) c = b->cluster;
+    if (b->threads > 0) t = b->threads;
+    int n = batch_max_teams(b, c, t);
     while (n <= 0 && c > 1) {
         c /= 2;
-        n = plan_batch_max_teams(t, c, smem, b->max_n, true, all);
+        n = batch_max_teams(b, c, t);
     }
     *cluster = c;
     *threads = t;
@@ -676,15 +716,17 @@ gmt_status enqueue_build_back(gmt_batch* b, int32_t* parent, float* cost, cudaSt
         int cluster, threads, teams;
         plan_shape(b, &cluster, &threads, &teams);
         if (teams <= 0) return bfail(GMT_ERR_CUDA, "batched plan kernel cannot be resident");
-        if ((size_t)teams > b->slot.cap / 4) return bfail(GMT_ERR_CUDA, "batched plan scratch is too small");
+        bool local;
+        const size_t smem = batch_smem(b, cluster, &local);
+        if (local) teams = (int)std::min<size_t>(teams, b->slot.cap / 4);  // fewer teams, the same queue
+        else if (teams > b->max_scratch) return bfail(GMT_ERR_CUDA, "batched plan scratch is too small");
         BatchScratch sc;
         sc.ocost = b->s_ocost.as<float>();
         sc.stamp = b->s_stamp.as<int>();
         sc.lists = b->s_lists.as<int>();
         sc.max_nodes = b->max_n;
         BCUDA(launch_plan_batch(b->p_args.as<PlanArgs>(), b->p_order.as<int>(), b->q, b->next.as<int>(),
-                                b->slot.as<int>(), sc, teams, threads, cluster, batch_smem(b), b->max_n,
-                                pool_all_kinds(b), st),
+                                b->slot.as<int>(), sc, teams, threads, cluster, smem, local, pool_all_kinds(b), st),
               "batched plan kernel");
     }
     BCUDA(record_plan_event(b->ev_plan[1], st), "event");
@@ -909,25 +951,25 @@ gmt_status prepare(gmt_batch* b, int q, const gmt_query* queries, int32_t* paren
             return bfail(GMT_ERR_INVALID,
                          "an appended sample is outside X or in X_obs (query " + std::to_string(k) + ")");
     }
-    // edge slices: ints (columns) and floats; a Dubins query's float slice
-    // starts with its in-edge words (4 floats each), kept 16-byte aligned
+    // edge slices: ints (columns) and floats, every array 16-byte aligned; a
+    // Dubins query's float slice starts with its in-edge words (4 floats each)
+    auto up4 = [](size_t n) { return (n + 3) / 4 * 4; };
     size_t ei = 0, ef = 0;
     std::vector<size_t> eo(q), fo(q);
     for (int k = 0; k < q; ++k) {
         b->E[k] = b->h_rows[k];
-        const size_t E = (size_t)b->E[k];
+        const size_t E = up4((size_t)b->E[k]);
         const int kind = queries[k].space.kind;
         eo[k] = ei;
         ei += E * (kind == GMT_COST_EUCLID ? 1 : 2);
         fo[k] = ef;
         ef += (kind == GMT_COST_EUCLID ? E : kind == GMT_COST_DI ? 4 * E : 6 * E);
-        ef = (ef + 3) / 4 * 4;
     }
     BCUDA(b->edges_i.need(ei * 4 + 4), "edge arena");
     BCUDA(b->edges_f.need(ef * 4 + 16), "edge arena");
     for (int k = 0; k < q; ++k) {
         QueryDev& d = b->qd[k];
-        const size_t E = (size_t)b->E[k];
+        const size_t E = up4((size_t)b->E[k]);
         const bool di = d.s.kind == GMT_COST_DI, dub = d.s.kind == GMT_COST_DUBINS, directed = di || dub;
         float* f = b->edges_f.as<float>() + fo[k];
         d.in_path = dub ? f : nullptr;
@@ -938,7 +980,7 @@ gmt_status prepare(gmt_batch* b, int q, const gmt_query* queries, int32_t* paren
         d.in_col = directed ? d.out_col + E : d.out_col;
         d.in_cost = di ? f + 2 * E : dub ? f + E : d.out_cost;
         d.in_tau = di ? f + 3 * E : nullptr;
-        d.edge_cap = (long long)E;
+        d.edge_cap = b->E[k];
     }
     // plan arguments, order (largest edge count first), scratch
     int max_n = 0;
@@ -1066,21 +1108,25 @@ gmt_status prepare(gmt_batch* b, int q, const gmt_query* queries, int32_t* paren
     BCUDA(b->l_stamp.need(lock_nodes * 4), "lockstep scratch");
     BCUDA(b->l_ctl.need((size_t)chunks * sizeof(LockCtl)), "lockstep scratch");
     b->lock_chunks = chunks;
-    // scratch for the most teams any shape can run
-    int max_teams = 0;
+    // scratch for the most teams any shape can run, and state scratch for the
+    // most that any shape without room for its state can
+    int max_teams = 0, max_scratch = 0;
     b->max_n = max_n;
-    {
-        const size_t smem = batch_smem(b);
-        const bool all = pool_all_kinds(b);
-        for (int c : {1, 2, 4, 8, 16})
-            for (int t : {256, 512, 1024})
-                max_teams = std::max(max_teams, plan_batch_max_teams(t, c, smem, max_n, false, all));
+    for (int c : {1, 2, 4, 8, 16}) {
+        bool local;
+        const size_t smem = batch_smem(b, c, &local);
+        for (int t : {256, 512, 1024}) {
+            const int n = plan_batch_max_teams(t, c, smem, local, pool_all_kinds(b));
+            max_teams = std::max(max_teams, n);
+            if (!local) max_scratch = std::max(max_scratch, n);
+        }
     }
     cudaGetLastError();
     if (max_teams <= 0) return bfail(GMT_ERR_CUDA, "batched plan kernel cannot be resident");
-    BCUDA(b->s_ocost.need((size_t)max_teams * 2 * max_n * 4), "scratch");
-    BCUDA(b->s_stamp.need((size_t)max_teams * max_n * 4), "scratch");
-    BCUDA(b->s_lists.need((size_t)max_teams * plan_list_stride(max_n) * 4), "scratch");
+    b->max_scratch = max_scratch;
+    BCUDA(b->s_ocost.need((size_t)max_scratch * 2 * max_n * 4), "scratch");
+    BCUDA(b->s_stamp.need((size_t)max_scratch * max_n * 4), "scratch");
+    BCUDA(b->s_lists.need((size_t)max_scratch * plan_list_stride(max_n) * 4), "scratch");
     BCUDA(b->slot.need((size_t)max_teams * 4), "scratch");
     // scratch slices are indexed by team id, so every group may use all of it
     for (Group& g : b->groups) g.max_n = max_n;

@@ -306,7 +306,7 @@ __host__ __device__ constexpr int smem_box_cap(int dp) { return 4096 / dp; }
 // larger and fits within 48 KB beside the kernel's own static shared memory
 // (at most kPlanStaticSmem bytes), the parent array of N nodes (read for the
 // path walk once the wavefront is over).
-constexpr size_t kPlanStaticSmem = 512;
+constexpr size_t kPlanStaticSmem = 1024;
 inline size_t plan_smem_bytes(int staged_boxes, int dp, int N) {
     const size_t boxes = (size_t)2 * staged_boxes * dp * sizeof(float);
     const size_t parents = (size_t)N * sizeof(int);
@@ -421,19 +421,18 @@ int plan_max_cluster(int kind, int dp, int threads);
 // Persistent batched wavefront (one barrier per iteration) over the `nq`
 // queries queries[order[0 .. nq)] of any kinds, taken in that order from the
 // device counter `next` (zeroed by the caller); `slot` holds one int per team.
-// cluster <= 1: teams are single CTAs, which keep the whole wavefront state
-// in shared memory when the largest query (max_n nodes) fits
-// (batch_state_fits; no scratch used), else use the scratch.  smem: dynamic
-// shared memory per CTA (the largest plan_smem_bytes of the queries).
-// all_kinds = false: every query is geometric (a kernel with fewer
-// registers).  plan_batch_max_teams: resident teams of a shape; with
-// smem_state = false, of the scratch-using kernels only (for sizing the
-// scratch).
+// cluster <= 1: teams are single CTAs.  local: the wavefront's state lives in
+// the team's shared memory (smem: the largest plan_local_bytes of the queries
+// for that cluster; edge arrays 16-byte aligned; the scratch is not used), else
+// in the scratch (smem: the largest plan_smem_bytes).  all_kinds = false: every
+// query is geometric (a kernel with fewer registers).  plan_batch_max_teams:
+// resident teams of a shape.  plan_local_bytes: SIZE_MAX if a query of N nodes
+// does not fit n CTAs.
 cudaError_t launch_plan_batch(const PlanArgs* queries, const int* order, int nq, int* next, int* slot,
                               const BatchScratch& scratch, int teams, int threads, int cluster, size_t smem,
-                              int max_n, bool all_kinds, cudaStream_t st);
-int plan_batch_max_teams(int threads, int cluster, size_t smem, int max_n, bool smem_state, bool all_kinds);
-bool batch_state_fits(size_t smem, int max_n);
+                              bool local, bool all_kinds, cudaStream_t st);
+int plan_batch_max_teams(int threads, int cluster, size_t smem, bool local, bool all_kinds);
+size_t plan_local_bytes(int kind, int d, int dp, int N, int boxes, int n);
 // plan_multi.cu: one cooperative grid of `blocks` CTAs advances all `nq`
 // queries of one (kind, dp) group together (nq <= kLockMaxQueries).  The
 // queries' PlanCtl blocks must be zeroed before the launch.

@@ -426,25 +426,13 @@ __device__ __forceinline__ bool lazy_check(const PlanArgs& A, int by, int be, co
     return free_edge;
 }
 
-// Loads of the wavefront's mutable state (snapshot, lists, control block):
-// from L2 (ld.global.cg) when the team spans several SMs, plain loads when a
-// single CTA keeps that state in its shared memory (SM = true).
-template <bool SM> __device__ __forceinline__ int st_i(const int* p) { if (SM) return *p; return __ldcg(p); }
-template <bool SM> __device__ __forceinline__ unsigned st_u(const unsigned* p) { if (SM) return *p; return __ldcg(p); }
-template <bool SM> __device__ __forceinline__ float st_f(const float* p) { if (SM) return *p; return __ldcg(p); }
-template <bool SM> __device__ __forceinline__ int2 st_i2(const int2* p) { if (SM) return *p; return __ldcg(p); }
-template <bool SM> __device__ __forceinline__ unsigned long long st_ull(const unsigned long long* p) {
-    if (SM) return *p;
-    return __ldcg(p);
-}
-
 // Lazy parent (Alg. 1, Sec. III-A), one lane's share of a group of W lanes:
 // over the in-row entries r0 + lane, r0 + lane + W, ... the minimum (cost, index) of
 // fl(ocost[y] + in_cost[e]) among open y (ocost < +inf); *be = its edge, -1
 // if none.  (cost, index) is a total order, so the order of the entries does
 // not matter: four chunks of W are taken at a time, their column and cost
 // loads issued together, then their snapshot gathers.
-template <bool SM, int W = 32>
+template <int W = 32>
 __device__ __forceinline__ void lane_parent_min(const int* __restrict__ in_col, const float* __restrict__ in_cost,
                                                 const float* ocost, int r0, int r1, int lane, float* bc_out,
                                                 int* by_out, int* be_out) {
@@ -461,7 +449,7 @@ __device__ __forceinline__ void lane_parent_min(const int* __restrict__ in_col, 
             ic[u] = e < r1 ? __ldg(&in_cost[e]) : 0.0f;
         }
 #pragma unroll
-        for (int u = 0; u < 4; ++u) oc[u] = ys[u] >= 0 ? st_f<SM>(&ocost[ys[u]]) : INF;
+        for (int u = 0; u < 4; ++u) oc[u] = ys[u] >= 0 ? ldcg_f(&ocost[ys[u]]) : INF;
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             if (oc[u] < INF) {
@@ -475,14 +463,5 @@ __device__ __forceinline__ void lane_parent_min(const int* __restrict__ in_col, 
     *be_out = be;
 }
 
-
-// Shared-memory layout of the single-CTA kernel that keeps the wavefront state
-// on chip (plan_kernel_smem): region0 (boxes / parent copy), the control
-// block, ocost and stamp (N each), the lists.
-constexpr size_t kSmemCtlBytes = smem_round16(sizeof(PlanCtl));
-inline size_t plan_smem_state_bytes(size_t region0, int N) {
-    return smem_round16(region0) + kSmemCtlBytes + smem_round16((size_t)8 * N) +
-           smem_round16(plan_list_stride((size_t)N) * sizeof(int));
-}
 
 }  // namespace gmtk

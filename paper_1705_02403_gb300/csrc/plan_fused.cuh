@@ -60,7 +60,7 @@ __device__ __forceinline__ void fused_pull(const PlanArgs& A, const TeamCtl<SH>&
     for (int a = 0; a < D; ++a) sx[a] = __ldg(&A.X[(size_t)a * A.pitch + x]);
     float bc;
     int by, be;
-    lane_parent_min<false, W>(A.in_col, A.in_cost, ocur, r0, r1, lane, &bc, &by, &be);
+    lane_parent_min<W>(A.in_col, A.in_cost, ocur, r0, r1, lane, &bc, &by, &be);
 #pragma unroll
     for (int off = W / 2; off > 0; off >>= 1) {
         const float oc = __shfl_xor_sync(gmask, bc, off);

@@ -90,7 +90,7 @@ __device__ bool pull_candidate(const PlanArgs* __restrict__ Ap, LockSmem& sm, in
     for (int a = 0; a < D; ++a) sx[a] = __ldg(&X[(size_t)a * pitch + x]);
     float bc;
     int by, be;
-    lane_parent_min<false>(in_col, in_cost, ocost, r0, r1, lane, &bc, &by, &be);
+    lane_parent_min(in_col, in_cost, ocost, r0, r1, lane, &bc, &by, &be);
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {
         const float oc = __shfl_xor_sync(kFull, bc, off);

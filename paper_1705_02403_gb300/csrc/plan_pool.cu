@@ -221,7 +221,7 @@ __device__ void pull_item(const PlanArgs& A, int j, const PoolIter& I, TaskCount
         for (int a = 0; a < D; ++a) sx[a] = __ldg(&A.X[(size_t)a * A.pitch + x]);
         float bc;
         int by, be;
-        lane_parent_min<false>(A.in_col, A.in_cost, ocur, r0, r1, lane, &bc, &by, &be);
+        lane_parent_min(A.in_col, A.in_cost, ocur, r0, r1, lane, &bc, &by, &be);
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) {
             const float oc = __shfl_xor_sync(0xffffffffu, bc, off);

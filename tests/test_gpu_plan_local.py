@@ -77,3 +77,31 @@ def test_rows_that_are_not_aligned(O, P):
     N.gmt_plan_static(pl.space, raw, pl.boxes, pl.params, pl.parent.data_ptr(), pl.cost.data_ptr())
     assert np.array_equal(pl.parent.cpu().numpy(), parent)
     assert np.array_equal(pl.cost.cpu().numpy().view(np.uint32), cost.view(np.uint32))
+
+
+@pytest.mark.parametrize("q", [1, 9, 10, 38, 39, 100])
+@pytest.mark.parametrize("big", [0, 21000, 120000])
+def test_batches_at_the_untuned_shapes_limits(O, P, q, big):
+    # teams from 16 CTAs (one query) to 2; a largest query whose state needs
+    # more CTAs, and one whose state fits no team (scratch in global memory)
+    if big and q not in (1, 39):
+        pytest.skip("the largest query decides")
+    qs = [envgen.geometric(700 + k, d=2 + k % 2, n=3 + 37 * (k % 11), nbox=5, r=0.35) for k in range(q)]
+    if big:
+        qs.append(envgen.geometric(9, d=2, n=big, nbox=12, r=0.012 if big < 50000 else 0.005))
+    bp = P.BatchPlanner(qs)
+    infos = bp.plan()
+    for k in range(0, len(qs), 5):
+        if qs[k].n > 1000:
+            continue
+        X, goal, g, parent, cost, info = oracle_run(O, qs[k])
+        got_parent, got_cost = bp.result(k)
+        assert np.array_equal(got_parent.cpu().numpy(), parent)
+        assert np.array_equal(got_cost.cpu().numpy().view(np.uint32), cost.view(np.uint32))
+        assert infos[k]["checks"] == info["checks"] and infos[k]["iters"] == info["iters"]
+    if big:  # as planned alone
+        pl = P.Planner(qs[-1]).build()
+        info = pl.plan()
+        got_parent, got_cost = bp.result(len(qs) - 1)
+        assert torch.equal(got_parent, pl.parent) and torch.equal(got_cost.view(torch.int32), pl.cost.view(torch.int32))
+        assert all(infos[-1][f] == info[f] for f in ("iters", "checks", "push_edges", "pull_edges", "goal_node"))
