@@ -187,7 +187,7 @@ template <int D, bool FILL>
 __global__ void __launch_bounds__(kCellWarps * 32) batch_cells_tile_kernel(const QueryDev* __restrict__ Q,
                                                                            const long long* __restrict__ off, int nq,
                                                                            int words) {
-    extern __shared__ int cell_buf[];
+    extern __shared__ __align__(16) int cell_buf[];
     const long long c = blockIdx.x;
     if (c >= off[nq]) return;
     const int k = find_query(off, nq, c);
@@ -195,7 +195,8 @@ __global__ void __launch_bounds__(kCellWarps * 32) batch_cells_tile_kernel(const
     if (!q.use_cells) return;
     if (FILL && (long long)q.out_row[q.s.N] > q.edge_cap) return;
     cell_tile<D, FILL>(q.s, q.X, q.cg, q.cell_start, q.cell_sorted, q.out_count, q.cell_info, q.out_row, q.out_col,
-                       q.out_cost, q.cell_info + 1, cell_buf, words, (int)(c - off[k]));
+                       q.out_cost, q.cell_info + 1, cell_buf, words, FILL ? cell_rank_words(q.cg, q.s.N) : 0,
+                       (int)(c - off[k]));
     if (FILL && threadIdx.x == 0 && __ldcg(&q.cell_info[1]) != 0) q.out_row[q.s.N] = INT_MAX;
 }
 
@@ -301,21 +302,27 @@ cudaError_t batch_cells_front(int d, const QueryDev* Q, const long long* off, co
     batch_cells_scan_kernel<<<nq, 1024, 0, st>>>(Q);
     batch_cells_scatter_kernel<<<tb, 256, 0, st>>>(Q, off, nq);
     if (cells > 0) {
-        const size_t smem = cell_tile_smem(d, 0);
+        const size_t smem = cell_tile_smem(d, false, 0, 0);
         if (d == 2) batch_cells_tile_kernel<2, false><<<(unsigned)cells, kCellWarps * 32, smem, st>>>(Q, off_cells, nq, 0);
         else batch_cells_tile_kernel<3, false><<<(unsigned)cells, kCellWarps * 32, smem, st>>>(Q, off_cells, nq, 0);
     }
     return cudaGetLastError();
 }
-// words: the largest cell_fill_words of the group's cell-list queries
+// words, rank_words: the largest cell_fill_words and cell_rank_words of the
+// group's cell-list queries
 cudaError_t batch_cells_fill(int d, const QueryDev* Q, const long long* off_cells, int nq, long long cells, int words,
-                             cudaStream_t st) {
+                             int rank_words, cudaStream_t st) {
     if (cells <= 0) return cudaSuccess;
-    const size_t smem = cell_tile_smem(d, words);
-    if (d == 2) batch_cells_tile_kernel<2, true><<<(unsigned)cells, kCellWarps * 32, smem, st>>>(Q, off_cells, nq, words);
-    else if (d == 3) batch_cells_tile_kernel<3, true><<<(unsigned)cells, kCellWarps * 32, smem, st>>>(Q, off_cells, nq, words);
-    else return cudaErrorInvalidValue;
-    return cudaGetLastError();
+    const size_t smem = cell_tile_smem(d, true, words, rank_words);
+    auto launch = [&](auto kern) {
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        kern<<<(unsigned)cells, kCellWarps * 32, smem, st>>>(Q, off_cells, nq, words);
+        return cudaGetLastError();
+    };
+    if (d == 2) return launch(batch_cells_tile_kernel<2, true>);
+    if (d == 3) return launch(batch_cells_tile_kernel<3, true>);
+    return cudaErrorInvalidValue;
 }
 cudaError_t batch_tile_prefix(const QueryDev* Q, const long long* off_nodes, int nq, long long nodes,
                               cudaStream_t st) {
@@ -404,6 +411,7 @@ struct Group {
     bool any_cells = false;  // some member builds its neighbours with the cell list
     bool any_tiles = false;  // some member fills its CSR by mask tiles
     int cell_words = 0;      // largest fill buffer (words per warp) of those members
+    int cell_rank = 0;       // largest ordering bitmap (words)
     bool any_halton = false; // some member samples with the Halton sequence
 };
 
@@ -661,7 +669,7 @@ gmt_status enqueue_build_back(gmt_batch* b, int32_t* parent, float* cost, cudaSt
             BCUDA(batch_fill(g.kind, g.d, Q, g.off_rows.as<long long>(), nq, g.nodes, st), "batched fill");
         }
         if (g.any_cells)
-            BCUDA(batch_cells_fill(g.d, Q, g.off_cells.as<long long>(), nq, g.cells, g.cell_words, st),
+            BCUDA(batch_cells_fill(g.d, Q, g.off_cells.as<long long>(), nq, g.cells, g.cell_words, g.cell_rank, st),
                   "batched cells");
     }
     // sampling flags of this call (appended samples are read on replays too)
@@ -880,6 +888,7 @@ gmt_status prepare(gmt_batch* b, int q, const gmt_query* queries, int32_t* paren
         g.any_cells = false;
         g.any_tiles = false;
         g.cell_words = 0;
+        g.cell_rank = 0;
         g.any_halton = false;
         for (int i = 0; i < nq; ++i) {
             const int k = g.members[i];
@@ -887,7 +896,10 @@ gmt_status prepare(gmt_batch* b, int q, const gmt_query* queries, int32_t* paren
             g.any_cells = g.any_cells || use_cells[k];
             g.any_tiles = g.any_tiles || b->qd[k].tile_cnt != nullptr;
             g.any_halton = g.any_halton || queries[k].params.sampler == GMT_SAMPLER_HALTON;
-            if (use_cells[k]) g.cell_words = std::max(g.cell_words, cell_fill_words(cgs[k], N));
+            if (use_cells[k]) {
+                g.cell_words = std::max(g.cell_words, cell_fill_words(cgs[k], N));
+                g.cell_rank = std::max(g.cell_rank, cell_rank_words(cgs[k], N));
+            }
             const long long tiles =
                 use_cells[k] ? 0
                 : g.kind == GMT_COST_DI

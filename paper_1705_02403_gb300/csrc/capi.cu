@@ -508,7 +508,8 @@ gmt_status build_impl(const gmt_space* space, const gmt_boxes* boxes, const floa
     LAUNCH(g->mark(gmt_graph::kScan, 1, st), "event");
     g->pending = false;
     const long long cap_now = edge_capacity(g);
-    if (async && !cells && extra_count == 0 && cap_now > 0) {
+    // (a cell-list graph whose longest row decides whether it fits needs the host)
+    if (async && (!cells || cell_fill_fits(cg, g->N, INT_MAX)) && extra_count == 0 && cap_now > 0) {
         // no host wait: fill into the arrays of earlier builds; the next plan
         // (or view) confirms the edge count and rebuilds if it did not fit
         const bool di_a = g->kind == GMT_COST_DI, dub_a = g->kind == GMT_COST_DUBINS;
@@ -519,7 +520,11 @@ gmt_status build_impl(const gmt_space* space, const gmt_boxes* boxes, const floa
                                                        di_a ? g->in_tau : nullptr, dub_a ? g->in_path : nullptr,
                                                        cap_now}
                                              : FillDir{nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, 0};
-        if (listed && list_cap >= cap_now) {  // the list holds every edge the arrays can
+        if (cells) {
+            LAUNCH(launch_cells_rows(sa, g->X, cg, g->cell_of, g->cell_start, g->cell_sorted, true, nullptr, nullptr,
+                                     g->out_row, g->out_col, g->out_cost, g->flags + 4, st, cap_now),
+                   "cell row kernel");
+        } else if (listed && list_cap >= cap_now) {  // the list holds every edge the arrays can
             LAUNCH(launch_fill_list(sa, g->elist, g->epath, list_cap, out_dir, in_dir, g->wpre, g->wpreT, st),
                    "fill kernel");
         } else if (tiles) {
@@ -528,7 +533,7 @@ gmt_status build_impl(const gmt_space* space, const gmt_boxes* boxes, const floa
             LAUNCH(launch_fill(sa, g->X, out_dir, in_dir, g->flags + 3, st), "fill kernel");
         }
         LAUNCH(g->mark(gmt_graph::kFill, 1, st), "event");
-        g->used_cells = false;
+        g->used_cells = cells;
         g->E = -1;
         g->pending = true;
         g->pending_cap = cap_now;

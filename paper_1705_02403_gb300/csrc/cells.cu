@@ -25,10 +25,12 @@ __global__ void __launch_bounds__(kCellWarps * 32) cells_tile_kernel(SpaceArgs s
                                                                      int* __restrict__ max_deg,
                                                                      const int* __restrict__ row,
                                                                      int* __restrict__ col, float* __restrict__ cost,
-                                                                     int* __restrict__ overflow, int words) {
-    extern __shared__ int cell_buf[];
+                                                                     int* __restrict__ overflow, int words, int rank_words,
+                                                                     long long cap) {
+    extern __shared__ __align__(16) int cell_buf[];
+    if (FILL && cap > 0 && (long long)__ldg(&row[s.N]) > cap) return;  // the caller rebuilds
     cell_tile<D, FILL>(s, X, cg, start, sorted, out_count, max_deg, row, col, cost, overflow, cell_buf, words,
-                       blockIdx.x);
+                       rank_words, blockIdx.x);
 }
 
 // ---- box grid (checks against many boxes)
@@ -207,30 +209,34 @@ bool make_cell_grid(int kind, int d, const float* lo, const float* hi, float r, 
     while ((double)r * 1.01 * (double)cg->inv_h > 1.0) cg->inv_h = std::nextafter(cg->inv_h, 0.0f);
     cg->ncells = (int)ncells;
     cg->list_only = 0;
-    // measured on one GB300 (Theorem 1 radii, cell tiles against the packed
-    // all-pairs test and the tiled fill): on one graph in 2D the cell list
-    // loses at 8192 nodes (0.055 against 0.040 ms) and wins at 16384 (0.069
-    // against 0.087); in a batch (where the cell stages' short launches
-    // overlap other queries' work) it already pays from 4096; in 3D, with 27
-    // cells of candidates to sort per tile, it loses at 16384 (0.216 against
-    // 0.113 ms) and wins at 32768 (0.280 against 0.388)
-    *pays = frac <= 0.25 && N >= (d == 2 ? (batched ? 4096 : 12000) : 32768);
+    // measured on one GB300 (Theorem 1 radii, 30 boxes; cell tiles against the
+    // packed all-pairs test and the tiled fill; pair test, scan and fill in ms):
+    // one graph, 2D: 8192 nodes 0.054 against 0.046, 12000 0.059 against 0.065;
+    // 3D: 12000 0.093 against 0.076, 16384 0.099 against 0.117.  In a batch the
+    // cell stages' short launches overlap other queries' work, and they pay
+    // sooner (builds of 400k nodes in all): 2D: 2500 nodes a query 0.58 against
+    // 0.51, 4000 0.54 against 0.68; 3D: 4000 0.93 against 0.86, 6000 1.01
+    // against 1.11.
+    *pays = frac <= 0.3 && N >= (d == 2 ? (batched ? 3200 : 10500) : (batched ? 5000 : 14000));
     return true;
 }
 
 namespace {
 template <int D>
 cudaError_t rows_t(const SpaceArgs& s, const float* X, const CellGrid& cg, const int* start, const int* sorted,
-                   bool fill, int* out_count, int* max_deg, const int* row, int* col, float* cost, int* overflow,
+                   bool fill, int* out_count, int* max_deg, const int* row, int* col, float* cost, int* overflow, long long cap,
                    cudaStream_t st) {
-    const int words = fill ? cell_fill_words(cg, s.N) : 0;
-    const size_t smem = cell_tile_smem(D, words);
-    if (fill)
-        cells_tile_kernel<D, true><<<cg.ncells, kCellWarps * 32, smem, st>>>(s, X, cg, start, sorted, out_count,
-                                                                             max_deg, row, col, cost, overflow, words);
-    else
-        cells_tile_kernel<D, false><<<cg.ncells, kCellWarps * 32, smem, st>>>(s, X, cg, start, sorted, out_count,
-                                                                              max_deg, row, col, cost, overflow, 0);
+    const int words = fill ? cell_fill_words(cg, s.N) : 0, rank = fill ? cell_rank_words(cg, s.N) : 0;
+    const size_t smem = cell_tile_smem(D, fill, words, rank);
+    auto launch = [&](auto kern) {
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        kern<<<cg.ncells, kCellWarps * 32, smem, st>>>(s, X, cg, start, sorted, out_count, max_deg, row, col, cost,
+                                                       overflow, words, rank, cap);
+        return cudaSuccess;
+    };
+    const cudaError_t e = fill ? launch(cells_tile_kernel<D, true>) : launch(cells_tile_kernel<D, false>);
+    if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }
 }  // namespace
@@ -252,10 +258,10 @@ cudaError_t launch_cells_scatter(int N, const int* cell_of, const int* cell_star
 
 cudaError_t launch_cells_rows(const SpaceArgs& s, const float* X, const CellGrid& cg, const int* cell_of,
                               const int* cell_start, const int* sorted, bool fill, int* out_count, int* max_deg,
-                              const int* row, int* col, float* cost, int* overflow, cudaStream_t st) {
+                              const int* row, int* col, float* cost, int* overflow, cudaStream_t st, long long cap) {
     (void)cell_of;
-    if (s.d == 2) return rows_t<2>(s, X, cg, cell_start, sorted, fill, out_count, max_deg, row, col, cost, overflow, st);
-    if (s.d == 3) return rows_t<3>(s, X, cg, cell_start, sorted, fill, out_count, max_deg, row, col, cost, overflow, st);
+    if (s.d == 2) return rows_t<2>(s, X, cg, cell_start, sorted, fill, out_count, max_deg, row, col, cost, overflow, cap, st);
+    if (s.d == 3) return rows_t<3>(s, X, cg, cell_start, sorted, fill, out_count, max_deg, row, col, cost, overflow, cap, st);
     return cudaErrorInvalidValue;
 }
 

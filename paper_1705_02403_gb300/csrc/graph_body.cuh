@@ -521,9 +521,12 @@ __device__ __forceinline__ void mask_tile_euclid4(const SpaceArgs& s, const floa
 // columns staged in shared memory, writes each row's columns of the tile, in
 // ascending order, from row[i] + prefix, with cost sqrt(d2) of the same
 // expression as edge_cost (so the same bits), and no gather of the samples
-// per edge.  Each lane loads its row's words; the warp then deals all its
-// rows' columns of the tile to its lanes in order, so no lane idles while
-// another walks a long row, and a row's columns go to consecutive lanes.
+// per edge.  Each lane lists its row's columns in shared memory, from the
+// prefix of the warp's rows; the warp then evaluates the listed edges, all
+// lanes busy and a row's columns on consecutive lanes.  (Finding each edge's
+// row and bit by binary search instead took three times the instructions:
+// 200 queries of 2049 nodes, 48 M edges, 0.306 ms.)
+constexpr int kTileList = 1024;
 __device__ __forceinline__ void tile_prefix_row(int* __restrict__ tile_cnt, int pitch, int nb, int i) {
     constexpr int kChunk = 16;  // loads issued together, then the chunk's prefixes stored
     int acc = 0;
@@ -547,10 +550,10 @@ __device__ __forceinline__ void fill_tile_euclid(const SpaceArgs& s, const float
     static_assert(D >= 2 && D <= 4, "float4 columns");
     constexpr int kWarps = kMaskRows / 32;
     __shared__ float4 tile[kMaskWords * 32];
-    __shared__ uint32_t swords[kWarps][32][kMaskWords];  // each row's words of the tile
-    __shared__ int sex[kWarps][33];                       // exclusive prefix of the rows' column counts
-    __shared__ int sbase[kWarps][32];                     // each row's first position for the tile
+    __shared__ uint32_t swords[kWarps][kMaskWords][32];  // each row's words of the tile
     __shared__ float4 sxi[kWarps][32];                    // each row's coordinates
+    __shared__ int soff[kWarps][32];                      // each row's position of its chunk's entries, less their prefix
+    __shared__ uint16_t list[kWarps][kTileList];          // the chunk's entries: row of the warp << 8 | column of the tile
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int i = bx * kMaskRows + threadIdx.x;
     const int w0 = by * kMaskWords;
@@ -565,57 +568,63 @@ __device__ __forceinline__ void fill_tile_euclid(const SpaceArgs& s, const float
     // each lane loads its row's words of the tile (coalesced over the rows)
     const bool row_ok = i < s.N;
     const int W = (s.N + 31) / 32;
-    int cnt = 0;
+    uint32_t wd[kMaskWords];
 #pragma unroll
     for (int ww = 0; ww < kMaskWords; ++ww) {
-        const uint32_t w = row_ok && w0 + ww < W ? mask[(size_t)(w0 + ww) * s.pitch + i] : 0u;
-        swords[warp][lane][ww] = w;
-        cnt += __popc(w);
+        wd[ww] = row_ok && w0 + ww < W ? mask[(size_t)(w0 + ww) * s.pitch + i] : 0u;
+        swords[warp][ww][lane] = wd[ww];
     }
     float c[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
     for (int a = 0; a < D; ++a) c[a] = row_ok ? X[(size_t)a * s.pitch + i] : 0.0f;
     sxi[warp][lane] = make_float4(c[0], c[1], c[2], c[3]);
-    sbase[warp][lane] = cnt > 0 ? row[i] + tile_pre[(size_t)by * s.pitch + i] : 0;
-    int incl = cnt;
+    int pos = row_ok ? row[i] + tile_pre[(size_t)by * s.pitch + i] : 0;
+    // the words per chunk: as many as leave every chunk's entries room in the
+    // list (one word of 32 rows always does)
+    int step = kMaskWords;
+    for (; step > 1; step >>= 1) {
+        bool fits = true;
+        for (int c0 = 0; c0 < kMaskWords; c0 += step) {
+            int n = 0;
 #pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, incl, off);
-        if (lane >= off) incl += y;
+            for (int ww = 0; ww < kMaskWords; ++ww) n += ww >= c0 && ww < c0 + step ? __popc(wd[ww]) : 0;
+            fits = fits && __reduce_add_sync(0xffffffffu, n) <= kTileList;
+        }
+        if (fits) break;
     }
-    sex[warp][lane] = incl - cnt;
-    if (lane == 31) sex[warp][32] = incl;
-    __syncthreads();  // the staged columns; the warp's row tables
-    // the warp's columns in (row, word, bit) order, dealt to its lanes: entry
-    // e of row r goes to position sbase[r] + (e - sex[r]), so each row's
-    // columns come out ascending and consecutive lanes write consecutive
-    // positions of a row
-    const int total = sex[warp][32];
-    for (int e = lane; e < total; e += 32) {
-        int r = 0;  // the row: the last one whose prefix is <= e
+    __syncthreads();  // the staged columns
+    for (int c0 = 0; c0 < kMaskWords; c0 += step) {
+        int cnt = 0;
+        for (int ww = c0; ww < c0 + step; ++ww) cnt += __popc(swords[warp][ww][lane]);
+        int incl = cnt;
 #pragma unroll
-        for (int step = 16; step > 0; step >>= 1)
-            if (sex[warp][r + step] <= e) r += step;
-        int m = e - sex[warp][r], k = 0;
-        uint32_t wk = swords[warp][r][0];
-        for (int ww = 0; ww < kMaskWords; ++ww) {
-            wk = swords[warp][r][ww];
-            const int cw = __popc(wk);
-            if (m < cw) { k = ww; break; }
-            m -= cw;
+        for (int off = 1; off < 32; off <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, incl, off);
+            if (lane >= off) incl += y;
         }
-        const int jt = k * 32 + select_bit(wk, m);
-        const float4 q = tile[jt], p = sxi[warp][r];
-        const float xj[4] = {q.x, q.y, q.z, q.w}, xr[4] = {p.x, p.y, p.z, p.w};
-        float d2 = 0.0f;
+        const int total = __shfl_sync(0xffffffffu, incl, 31);
+        soff[warp][lane] = pos - (incl - cnt);
+        pos += cnt;
+        int at = incl - cnt;
+        for (int ww = c0; ww < c0 + step; ++ww)
+            for (uint32_t w = swords[warp][ww][lane]; w; w &= w - 1u)
+                list[warp][at++] = (uint16_t)(lane << 8 | (ww * 32 + __ffs(w) - 1));
+        __syncwarp();
+        for (int e = lane; e < total; e += 32) {
+            const int ent = list[warp][e], r = ent >> 8, jt = ent & 255;
+            const float4 q = tile[jt], p = sxi[warp][r];
+            const float xj[4] = {q.x, q.y, q.z, q.w}, xr[4] = {p.x, p.y, p.z, p.w};
+            float d2 = 0.0f;
 #pragma unroll
-        for (int a = 0; a < D; ++a) {
-            const float tt = xj[a] - xr[a];
-            d2 = d2 + tt * tt;
+            for (int a = 0; a < D; ++a) {
+                const float tt = xj[a] - xr[a];
+                d2 = d2 + tt * tt;
+            }
+            const int at_e = soff[warp][r] + e;
+            col[at_e] = j0 + jt;
+            cost[at_e] = __fsqrt_rn(d2);
         }
-        const int pos = sbase[warp][r] + (e - sex[warp][r]);
-        col[pos] = j0 + jt;
-        cost[pos] = __fsqrt_rn(d2);
+        __syncwarp();
     }
 }
 
@@ -1109,21 +1118,36 @@ __device__ __forceinline__ void transpose_task(int N, int pitch, const uint32_t*
 }
 
 // Exclusive prefix sum: row[v] = sum_{u < v} count[u], row[N] = total (also
-// returned to every thread).  One block of 1024 threads.
-__device__ __forceinline__ int scan_rows(const int* __restrict__ count, int* __restrict__ row, int N) {
+// returned to every thread).  One block of 1024 threads, K entries per thread
+// and pass: each warp takes 32 K consecutive entries, its K loads in flight
+// together, scans them 32 at a time, and the warps' totals are scanned once
+// per pass.
+template <int K>
+__device__ __forceinline__ int scan_rows_k(const int* __restrict__ count, int* __restrict__ row, int N) {
     __shared__ int warp_sum[32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int carry = 0;
-    for (int base = 0; base < N; base += 1024) {
-        const int i = base + threadIdx.x;
-        const int v = i < N ? count[i] : 0;
-        int x = v;
+    for (int base = 0; base < N; base += 1024 * K) {
+        const int first = base + warp * 32 * K + lane;
+        int v[K], x[K], sum = 0;
 #pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, x, off);
-            if (lane >= off) x += y;
+        for (int k = 0; k < K; ++k) v[k] = first + 32 * k < N ? count[first + 32 * k] : 0;
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            x[k] = v[k];
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, x[k], off);
+                if (lane >= off) x[k] += y;
+            }
         }
-        if (lane == 31) warp_sum[warp] = x;
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            const int total = __shfl_sync(0xffffffffu, x[k], 31);
+            x[k] += sum - v[k];  // exclusive within the warp's entries
+            sum += total;
+        }
+        if (lane == 31) warp_sum[warp] = sum;
         __syncthreads();
         if (warp == 0) {
             int t = warp_sum[lane];
@@ -1135,12 +1159,21 @@ __device__ __forceinline__ int scan_rows(const int* __restrict__ count, int* __r
             warp_sum[lane] = t;
         }
         __syncthreads();
-        if (i < N) row[i] = carry + (warp > 0 ? warp_sum[warp - 1] : 0) + x - v;
+        const int before = carry + (warp > 0 ? warp_sum[warp - 1] : 0);
+#pragma unroll
+        for (int k = 0; k < K; ++k)
+            if (first + 32 * k < N) row[first + 32 * k] = before + x[k];
         carry += warp_sum[31];
         __syncthreads();
     }
     if (threadIdx.x == 0) row[N] = carry;
     return carry;
+}
+
+// Eight entries per thread from 2049 nodes (one entry per thread and pass took
+// 47 us at 65537 nodes).
+__device__ __forceinline__ int scan_rows(const int* __restrict__ count, int* __restrict__ row, int N) {
+    return N <= 2048 ? scan_rows_k<1>(count, row, N) : scan_rows_k<8>(count, row, N);
 }
 
 // Fill: the CSR columns and costs from the bit matrix.  A warp reads a row's

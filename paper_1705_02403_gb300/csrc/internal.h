@@ -200,10 +200,12 @@ cudaError_t launch_cells_scatter(int N, const int* cell_of, const int* cell_star
                                  cudaStream_t st);
 // fill = false: out_count[v] = neighbours of v, max_deg = their maximum; fill
 // = true: columns (ascending) and costs of every row at row[v]; a row longer
-// than kCellList sets *overflow and writes nothing.
+// than kCellList sets *overflow and writes nothing; an edge count above cap (>
+// 0) writes nothing at all.
 cudaError_t launch_cells_rows(const SpaceArgs& s, const float* X, const CellGrid& cg, const int* cell_of,
                               const int* cell_start, const int* sorted, bool fill, int* out_count, int* max_deg,
-                              const int* row, int* col, float* cost, int* overflow, cudaStream_t st);
+                              const int* row, int* col, float* cost, int* overflow, cudaStream_t st,
+                              long long cap = 0);
 
 // Workspace and control block of one plan (all device memory).  Counters are
 // double-buffered by iteration parity.  Open list j holds its kept entries in
