@@ -278,6 +278,9 @@ struct PlanArgs {
     // writes the final control block there once the plan is over, so the
     // caller needs no device-to-host copy (NULL: not written).
     PlanCtl* host_ctl;
+    // Optional device-mapped host word set to 1 once host_ctl is written and
+    // every output of the plan is visible (NULL: not written).
+    int* host_done;
     // Optional per-edge verdict cache (in-CSR order): 0 unknown, 1 free,
     // 2 collides.  A known verdict answers the check; an unknown one is
     // computed and stored.  Valid only while the obstacles that could change
@@ -420,6 +423,8 @@ void record_error(const char* msg);
 cudaError_t launch_plan(const PlanArgs& a, int blocks, int threads, cudaStream_t st, int cluster = 0);
 int plan_max_coresident_blocks(int kind, int dp, int threads);
 int plan_max_cluster(int kind, int dp, int threads);
+// Loads the kernels a 2D or 3D plan on a cluster (or, <= 1, one CTA) launches.
+cudaError_t load_plan_kernel(int kind, int dp, int cluster);
 // Persistent batched wavefront (one barrier per iteration) over the `nq`
 // queries queries[order[0 .. nq)] of any kinds, taken in that order from the
 // device counter `next` (zeroed by the caller); `slot` holds one int per team.

@@ -43,11 +43,16 @@
 namespace gmtk {
 
 // The first warp copies the final control block to the caller's mapped host
-// copy (src: a block whose writers have all passed a barrier since).
-__device__ __forceinline__ void publish_ctl(PlanCtl* dst, const PlanCtl* src, int rank) {
+// copy (src: a block whose writers have all passed a barrier since), then sets
+// the caller's word.
+__device__ __forceinline__ void publish_ctl(const PlanArgs& A, int rank) {
     constexpr int n = (int)(sizeof(PlanCtl) / sizeof(int));
     for (int t = rank; t < n; t += 32)
-        reinterpret_cast<int*>(dst)[t] = __ldcg(reinterpret_cast<const int*>(src) + t);
+        reinterpret_cast<int*>(A.host_ctl)[t] = __ldcg(reinterpret_cast<const int*>(A.ctl) + t);
+    if (!A.host_done) return;
+    __threadfence_system();
+    __syncwarp();
+    if (rank == 0) *(volatile int*)A.host_done = 1;
 }
 
 // Lanes per candidate pull (measured on one GB300): a single plan's team has
@@ -68,7 +73,7 @@ __global__ void __launch_bounds__(1024, 1) plan_kernel(PlanArgs A, Team team) {
     plan_body_fused<Team, KIND, DP, kPlanPullLanes>(A, team, sbox, dyn_smem);
     if (A.host_ctl) {
         team.sync(A.ctl);  // every warp's counters and rank 0's result are in
-        if (team.rank() < 32) publish_ctl(A.host_ctl, A.ctl, team.rank());
+        if (team.rank() < 32) publish_ctl(A, team.rank());
     }
 }
 
@@ -77,7 +82,7 @@ template <class Team, int KIND, int DP>
 __global__ void __launch_bounds__(1024, 1) plan_local_kernel(PlanArgs A, Team team, bool cache) {
     extern __shared__ __align__(16) unsigned char plan_smem[];
     if (plan_body_local<Team, KIND, DP, kPlanPullLanes>(A, team, plan_smem, cache) && A.host_ctl && threadIdx.x < 32)
-        publish_ctl(A.host_ctl, A.ctl, threadIdx.x);
+        publish_ctl(A, threadIdx.x);
 }
 
 // Persistent batched wavefront: every team (a CTA, or a cluster) takes the next
@@ -275,6 +280,25 @@ cudaError_t launch_plan(const PlanArgs& a, int blocks, int threads, cudaStream_t
         case 10: return plan_t<GMT_COST_EUCLID, 10>(a, blocks, threads, cluster, st);
         default: return cudaErrorInvalidValue;
     }
+}
+
+namespace {
+template <int KIND, int DP>
+cudaError_t load_plan_t(int cluster) {
+    cudaFuncAttributes a;
+    cudaError_t e = cluster > 1 ? cudaFuncGetAttributes(&a, plan_local_kernel<ClusterTeam, KIND, DP>)
+                                : cudaFuncGetAttributes(&a, plan_local_kernel<BlockTeam, KIND, DP>);
+    if (e == cudaSuccess)
+        e = cluster > 1 ? cudaFuncGetAttributes(&a, plan_kernel<ClusterTeam, KIND, DP>)
+                        : cudaFuncGetAttributes(&a, plan_kernel<BlockTeam, KIND, DP>);
+    return e;
+}
+}  // namespace
+
+cudaError_t load_plan_kernel(int kind, int dp, int cluster) {
+    if (kind == GMT_COST_DI) return load_plan_t<GMT_COST_DI, 3>(cluster);
+    if (kind == GMT_COST_DUBINS) return load_plan_t<GMT_COST_DUBINS, 3>(cluster);
+    return dp == 2 ? load_plan_t<GMT_COST_EUCLID, 2>(cluster) : load_plan_t<GMT_COST_EUCLID, 3>(cluster);
 }
 
 // Largest cluster size (16, 8, 4, 2) for which one cluster of `threads`-thread

@@ -163,7 +163,6 @@ struct Request {
 };
 
 struct Slot {
-    std::condition_variable* cv = nullptr;  // server's, notified when the slot's request finishes
     cudaStream_t stream = nullptr;
     float* ocost = nullptr;
     int* stamp = nullptr;
@@ -171,12 +170,14 @@ struct Slot {
     PlanCtl* ctl = nullptr;
     int32_t* parent = nullptr;
     float* cost = nullptr;
-    float* moved = nullptr;       // device [2 * max_boxes][2][3]
-    float* h_moved = nullptr;     // pinned staging
-    float* h_boxes = nullptr;     // pinned staging of the request's boxes
+    float* stage = nullptr;       // device: the request's boxes (lo, hi), then its moved regions
+    float* h_stage = nullptr;     // the same, pinned
+    // the plan's result and completion word, in host memory the kernel writes
     PlanCtl* h_ctl = nullptr;
+    PlanCtl* d_ctl = nullptr;
+    int* h_done = nullptr;
+    int* d_done = nullptr;
     bool busy = false;
-    std::atomic<int> finished{0};
     Request req;
     Clock::time_point t_start, t_done;
 };
@@ -207,55 +208,55 @@ gmt_status sfail(gmt_status s, const std::string& m) {
     return s;
 }
 
-void CUDART_CB on_done(void* p) {
-    Slot* s = (Slot*)p;
-    s->t_done = Clock::now();
-    s->finished.store(1);
-    s->cv->notify_all();
-}
-
-// Launches a request on a free slot (worker thread, server lock held).
-cudaError_t start_request(gmt_server* sv, Slot& sl, Session& ss, Request&& rq) {
+// Lays out a request's boxes and the regions of those that moved (their old
+// and new places) in the slot's staging, and makes them the session's.
+// Returns the moved boxes.  Worker thread, server lock held.
+int stage_request(Slot& sl, Session& ss, Request&& rq) {
     const int P = ss.dp, nb = ss.nbox;
     sl.req = std::move(rq);
     sl.t_start = Clock::now();
-    sl.finished.store(0);
-    cudaStream_t st = sl.stream;
-    // moved boxes: old and new places of every box that changed
+    __atomic_store_n(sl.h_done, 0, __ATOMIC_RELEASE);
+    std::copy(sl.req.lo.begin(), sl.req.lo.end(), sl.h_stage);
+    std::copy(sl.req.hi.begin(), sl.req.hi.end(), sl.h_stage + nb * P);
+    float* o = sl.h_stage + 2 * nb * P;
     int nm = 0;
     for (int b = 0; b < nb; ++b) {
         bool moved = false;
         for (int a = 0; a < P; ++a)
             moved = moved || sl.req.lo[b * P + a] != ss.cur_lo[b * P + a] || sl.req.hi[b * P + a] != ss.cur_hi[b * P + a];
         if (!moved) continue;
-        float* o = sl.h_moved + (size_t)nm * 4 * P;
         for (int a = 0; a < P; ++a) {
             o[a] = ss.cur_lo[b * P + a]; o[P + a] = ss.cur_hi[b * P + a];
             o[2 * P + a] = sl.req.lo[b * P + a]; o[3 * P + a] = sl.req.hi[b * P + a];
         }
+        o += 4 * P;
         ++nm;
-    }
-    std::memcpy(sl.h_boxes, sl.req.lo.data(), nb * P * sizeof(float));
-    std::memcpy(sl.h_boxes + nb * P, sl.req.hi.data(), nb * P * sizeof(float));
-    cudaError_t e = cudaSuccess;
-    if (nb > 0) {
-        e = cudaMemcpyAsync(ss.d_lo, sl.h_boxes, nb * P * sizeof(float), cudaMemcpyHostToDevice, st);
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(ss.d_hi, sl.h_boxes + nb * P, nb * P * sizeof(float), cudaMemcpyHostToDevice, st);
-    }
-    if (e == cudaSuccess && nm > 0 && ss.view.E > 0) {
-        e = cudaMemcpyAsync(sl.moved, sl.h_moved, (size_t)nm * 4 * P * sizeof(float), cudaMemcpyHostToDevice, st);
-        const long long E = ss.view.E;
-        const unsigned blocks = (unsigned)((E + 255) / 256);
-        const size_t smem = (size_t)nm * 4 * P * sizeof(float);
-        if (e == cudaSuccess) {
-            if (P == 3) invalidate_kernel<3><<<blocks, 256, smem, st>>>(E, ss.aabb, sl.moved, nm, ss.verdict);
-            else invalidate_kernel<2><<<blocks, 256, smem, st>>>(E, ss.aabb, sl.moved, nm, ss.verdict);
-            e = cudaGetLastError();
-        }
     }
     ss.cur_lo = sl.req.lo;
     ss.cur_hi = sl.req.hi;
+    return nm;
+}
+
+// Queues a staged request on its slot's stream: one upload, the verdicts to
+// clear, the plan, the result.  Worker thread, without the server lock, so
+// that submissions go on meanwhile: the session is marked busy, which keeps it
+// and its graph in place.
+cudaError_t start_request(gmt_server* sv, Slot& sl, const Session& ss, int nm) {
+    const int P = ss.dp, nb = ss.nbox;
+    cudaStream_t st = sl.stream;
+    cudaError_t e = cudaSuccess;
+    if (nb > 0)
+        e = cudaMemcpyAsync(sl.stage, sl.h_stage, (size_t)(2 * nb + 4 * nm) * P * sizeof(float), cudaMemcpyHostToDevice,
+                            st);
+    if (e == cudaSuccess && nm > 0 && ss.view.E > 0) {
+        const long long E = ss.view.E;
+        const unsigned blocks = (unsigned)((E + 255) / 256);
+        const size_t smem = (size_t)nm * 4 * P * sizeof(float);
+        const float* moved = sl.stage + 2 * nb * P;
+        if (P == 3) invalidate_kernel<3><<<blocks, 256, smem, st>>>(E, ss.aabb, moved, nm, ss.verdict);
+        else invalidate_kernel<2><<<blocks, 256, smem, st>>>(E, ss.aabb, moved, nm, ss.verdict);
+        e = cudaGetLastError();
+    }
     if (e != cudaSuccess) return e;
     const gmt_graph_view& v = ss.view;
     PlanArgs a;
@@ -265,7 +266,7 @@ cudaError_t start_request(gmt_server* sv, Slot& sl, Session& ss, Request&& rq) {
     a.in_row = v.in_row; a.in_col = v.in_col; a.in_cost = v.in_cost; a.in_tau = v.in_tau;
     a.in_path = v.in_path;
     a.rho = v.turn_radius;
-    a.boxes = BoxArgs{nb, ss.d_lo, ss.d_hi};
+    a.boxes = BoxArgs{nb, sl.stage, sl.stage + nb * P};
     for (int k = 0; k < 3 && k < v.pos_dim; ++k) { a.pos_lo[k] = ss.space.lo[k]; a.pos_hi[k] = ss.space.hi[k]; }
     a.r = v.r;
     a.delta = ss.params.lambda * v.r;
@@ -278,24 +279,41 @@ cudaError_t start_request(gmt_server* sv, Slot& sl, Session& ss, Request&& rq) {
     a.ocost = sl.ocost; a.stamp = sl.stamp;
     const size_t M = (size_t)sv->cfg.max_nodes;
     assign_plan_lists(a, sl.lists, M);
-    a.ctl = sl.ctl;
+    a.ctl = sl.ctl;  // cleared by the plan itself (a cluster or one CTA)
+    a.host_ctl = sl.d_ctl;
+    a.host_done = sl.d_done;
     a.verdict = ss.verdict;
-    e = cudaMemsetAsync(sl.ctl, 0, sizeof(PlanCtl), st);
-    if (e == cudaSuccess)
-        e = launch_plan(a, sv->cfg.cluster > 1 ? 0 : 1, sv->cfg.threads, st, sv->cfg.cluster > 1 ? sv->cfg.cluster : 0);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(sl.h_ctl, sl.ctl, sizeof(PlanCtl), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaLaunchHostFunc(st, on_done, &sl);
-    return e;
+    return launch_plan(a, sv->cfg.cluster > 1 ? 0 : 1, sv->cfg.threads, st, sv->cfg.cluster > 1 ? sv->cfg.cluster : 0);
+}
+
+// Has the slot's plan finished?  Its kernel sets the word; `query` also asks
+// the stream, so that a plan that can no longer set it (a failed kernel) ends
+// with an error status.
+bool slot_done(Slot& sl, bool query) {
+    if (!__atomic_load_n(sl.h_done, __ATOMIC_ACQUIRE)) {
+        if (!query) return false;
+        const cudaError_t e = cudaStreamQuery(sl.stream);
+        if (e == cudaErrorNotReady) return false;
+        if (!__atomic_load_n(sl.h_done, __ATOMIC_ACQUIRE)) {
+            std::memset(sl.h_ctl, 0, sizeof(PlanCtl));
+            sl.h_ctl->status = GMT_ERR_CUDA;
+            sl.h_ctl->goal_node = -1;
+        }
+    }
+    sl.t_done = Clock::now();
+    return true;
 }
 
 void worker_loop(gmt_server* sv) {
     cudaSetDevice(sv->device);
     std::unique_lock<std::mutex> lk(sv->mu);
+    Clock::time_point t_progress = Clock::now();
     while (!sv->stop) {
         bool progress = false;
+        const bool query = Clock::now() - t_progress > std::chrono::milliseconds(2);
         for (auto& up : sv->slots) {
             Slot& sl = *up;
-            if (!sl.busy || !sl.finished.load()) continue;
+            if (!sl.busy || !slot_done(sl, query)) continue;
             const PlanCtl& c = *sl.h_ctl;
             gmt_server_result r;
             std::memset(&r, 0, sizeof(r));
@@ -333,7 +351,10 @@ void worker_loop(gmt_server* sv) {
             sv->queue.erase(qit);
             ss.busy = true;
             sl.busy = true;
-            cudaError_t e = start_request(sv, sl, ss, std::move(rq));
+            const int nm = stage_request(sl, ss, std::move(rq));
+            lk.unlock();
+            const cudaError_t e = start_request(sv, sl, ss, nm);
+            lk.lock();
             if (e != cudaSuccess) {
                 sv->worker_error = std::string("request launch: ") + cudaGetErrorString(e);
                 gmt_server_result r;
@@ -348,10 +369,26 @@ void worker_loop(gmt_server* sv) {
             }
             progress = true;
         }
-        if (progress) sv->cv.notify_all();
+        if (progress) {
+            sv->cv.notify_all();
+            t_progress = Clock::now();
+            continue;
+        }
         bool any_busy = false;
         for (auto& up : sv->slots) any_busy = any_busy || up->busy;
-        if (!progress) sv->cv.wait_for(lk, any_busy ? std::chrono::microseconds(200) : std::chrono::milliseconds(2));
+        // plans in flight: look at their words again at once, with the lock free
+        // in between (a plan takes a few hundred microseconds; a sleep would
+        // end up to 50 late), and less often once nothing has happened for 2 ms;
+        // nothing in flight: wait for a submission
+        if (any_busy) {
+            lk.unlock();
+            if (query) std::this_thread::sleep_for(std::chrono::microseconds(20));
+            else std::this_thread::yield();
+            lk.lock();
+        } else {
+            sv->cv.wait_for(lk, std::chrono::milliseconds(2));
+            t_progress = Clock::now();
+        }
     }
 }
 
@@ -385,7 +422,6 @@ gmt_status gmt_server_create(const gmt_server_config* cfg, gmt_server** out) {
     cudaError_t e = cudaStreamCreateWithFlags(&sv->setup, cudaStreamNonBlocking);
     for (int k = 0; k < cfg->slots && e == cudaSuccess; ++k) {
         auto sl = std::make_unique<Slot>();
-        sl->cv = &sv->cv;
         e = cudaStreamCreateWithFlags(&sl->stream, cudaStreamNonBlocking);
         if (e == cudaSuccess) e = cudaMalloc(&sl->ocost, 2 * M * 4);  // two snapshot buffers
         if (e == cudaSuccess) e = cudaMalloc(&sl->stamp, M * 4);
@@ -393,10 +429,12 @@ gmt_status gmt_server_create(const gmt_server_config* cfg, gmt_server** out) {
         if (e == cudaSuccess) e = cudaMalloc(&sl->ctl, 256);
         if (e == cudaSuccess) e = cudaMalloc(&sl->parent, M * 4);
         if (e == cudaSuccess) e = cudaMalloc(&sl->cost, M * 4);
-        if (e == cudaSuccess) e = cudaMalloc(&sl->moved, (size_t)mb * 4 * 3 * 4);
-        if (e == cudaSuccess) e = cudaMallocHost(&sl->h_moved, (size_t)mb * 4 * 3 * 4);
-        if (e == cudaSuccess) e = cudaMallocHost(&sl->h_boxes, (size_t)mb * 2 * 3 * 4);
-        if (e == cudaSuccess) e = cudaMallocHost(&sl->h_ctl, sizeof(PlanCtl));
+        if (e == cudaSuccess) e = cudaMalloc(&sl->stage, (size_t)mb * 6 * 3 * 4);
+        if (e == cudaSuccess) e = cudaMallocHost(&sl->h_stage, (size_t)mb * 6 * 3 * 4);
+        if (e == cudaSuccess) e = cudaHostAlloc((void**)&sl->h_ctl, sizeof(PlanCtl), cudaHostAllocMapped);
+        if (e == cudaSuccess) e = cudaHostGetDevicePointer((void**)&sl->d_ctl, sl->h_ctl, 0);
+        if (e == cudaSuccess) e = cudaHostAlloc((void**)&sl->h_done, sizeof(int), cudaHostAllocMapped);
+        if (e == cudaSuccess) e = cudaHostGetDevicePointer((void**)&sl->d_done, sl->h_done, 0);
         sv->slots.push_back(std::move(sl));
     }
     if (e != cudaSuccess) {
@@ -420,12 +458,12 @@ void gmt_server_free(gmt_server* sv) {
     for (auto& up : sv->slots) {
         Slot& sl = *up;
         if (sl.stream) cudaStreamSynchronize(sl.stream);
-        void* d[] = {sl.ocost, sl.stamp, sl.lists, sl.ctl, sl.parent, sl.cost, sl.moved};
+        void* d[] = {sl.ocost, sl.stamp, sl.lists, sl.ctl, sl.parent, sl.cost, sl.stage};
         for (void* p : d)
             if (p) cudaFree(p);
-        if (sl.h_moved) cudaFreeHost(sl.h_moved);
-        if (sl.h_boxes) cudaFreeHost(sl.h_boxes);
+        if (sl.h_stage) cudaFreeHost(sl.h_stage);
         if (sl.h_ctl) cudaFreeHost(sl.h_ctl);
+        if (sl.h_done) cudaFreeHost(sl.h_done);
         if (sl.stream) cudaStreamDestroy(sl.stream);
     }
     for (auto& kv : sv->sessions) {
@@ -528,6 +566,11 @@ gmt_status gmt_server_open_session(gmt_server* sv, const gmt_space* space, const
     if (st != GMT_OK) return undo(st, std::string("session graph: ") + gmt_last_error());
     gmt_graph_get_view(s.graph, &s.view);
     e = edge_cache_setup(s.view, *space, *params, &s.aabb, &s.verdict, sv->setup);
+    // the request's kernels are loaded now rather than by the first request
+    cudaFuncAttributes fa;
+    if (e == cudaSuccess) e = load_plan_kernel(space->kind, space->pos_dim, sv->cfg.cluster);
+    if (e == cudaSuccess)
+        e = P == 3 ? cudaFuncGetAttributes(&fa, invalidate_kernel<3>) : cudaFuncGetAttributes(&fa, invalidate_kernel<2>);
     if (e == cudaSuccess) e = cudaStreamSynchronize(sv->setup);
     if (e != cudaSuccess) return undo(GMT_ERR_CUDA, std::string("session setup: ") + cudaGetErrorString(e));
     std::lock_guard<std::mutex> lk(sv->mu);
@@ -650,6 +693,14 @@ gmt_status gmt_server_move_start(gmt_server* sv, int32_t session, const float* x
     }
     // a new graph (same seed, the current boxes) in a handle of its own, so a
     // failure leaves the session as it was
+    if (bx.count) {  // the boxes of the last request are on its slot; the build wants them here
+        cudaError_t eb = cudaMemcpyAsync(const_cast<float*>(bx.lo), lo.data(), lo.size() * sizeof(float),
+                                         cudaMemcpyHostToDevice, sv->setup);
+        if (eb == cudaSuccess)
+            eb = cudaMemcpyAsync(const_cast<float*>(bx.hi), hi.data(), hi.size() * sizeof(float),
+                                 cudaMemcpyHostToDevice, sv->setup);
+        if (eb != cudaSuccess) return finish(GMT_ERR_CUDA, std::string("start move: ") + cudaGetErrorString(eb));
+    }
     gmt_graph* ng = nullptr;
     gmt_status st = gmt_build_graph(&space, &bx, x_init, &goal, &params, &ng, sv->setup);
     if (st != GMT_OK) {
