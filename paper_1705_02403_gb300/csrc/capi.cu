@@ -126,6 +126,7 @@ struct gmt_graph {
     int* grid_list = nullptr;      size_t cap_grid_list = 0;
     int* grid_big = nullptr;       size_t cap_grid_big = 0;
     float4* grid_packed = nullptr; size_t cap_grid_packed = 0;
+    float4* grid_shape = nullptr;  size_t cap_grid_shape = 0;
     int* halton = nullptr;         size_t cap_halton = 0;    // multi-block Halton sampler scratch (ints)
     // plan workspace
     float* ocost = nullptr;        size_t cap_ocost = 0;
@@ -177,7 +178,7 @@ struct gmt_graph {
         void* dev[] = {X, is_goal, out_row, in_row_own, counts, out_col, out_cost, in_col_own,
                        in_cost_own, out_tau, in_tau, in_path, mask, maskT, tile_cnt, elist, epath, wpre, wpreT,
                        cell_of, cell_sorted, cell_cnt,
-                       cell_start, grid_cnt, grid_start, grid_list, grid_big, grid_packed, halton, ocost, stamp,
+                       cell_start, grid_cnt, grid_start, grid_list, grid_big, grid_packed, grid_shape, halton, ocost, stamp,
                        lists, ctl};
         for (void* p : dev)
             if (p) cudaFree(p);
@@ -269,7 +270,8 @@ cudaError_t build_box_grid(gmt_graph* g, const BoxArgs& boxes, BoxGridArgs* gr, 
     const size_t B = (size_t)boxes.count, cells = (size_t)G * G;
     cudaError_t e;
     if ((e = grow(&g->grid_cnt, &g->cap_grid_cnt, cells + 1)) != cudaSuccess) return e;  // + the big-box count
-    if ((e = grow(&g->grid_start, &g->cap_grid_start, cells + 1)) != cudaSuccess) return e;
+    if ((e = grow(&g->grid_start, &g->cap_grid_start, std::max(cells, (size_t)kBoxGridCells) + 1)) != cudaSuccess) return e;
+    if ((e = grow(&g->grid_shape, &g->cap_grid_shape, 1)) != cudaSuccess) return e;
     if ((e = grow(&g->grid_list, &g->cap_grid_list, B * kBoxGridMaxCells)) != cudaSuccess) return e;
     if ((e = grow(&g->grid_big, &g->cap_grid_big, B)) != cudaSuccess) return e;
     const bool packed = g->dp <= 3 && boxes.count <= kBoxGridPackMax;
@@ -281,14 +283,16 @@ cudaError_t build_box_grid(gmt_graph* g, const BoxArgs& boxes, BoxGridArgs* gr, 
     for (int k = 0; k < 2; ++k) {
         gr->lo[k] = g->pos_lo[k];
         gr->inv_h[k] = (float)((double)G / ((double)g->pos_hi[k] - (double)g->pos_lo[k]));
+        gr->span[k] = g->pos_hi[k] - g->pos_lo[k];
     }
+    gr->shape = boxes.count <= kBoxGridBlockMax ? g->grid_shape : nullptr;
     gr->start = g->grid_start;
     gr->list = g->grid_list;
     gr->packed = packed ? g->grid_packed : nullptr;
     gr->big = g->grid_big;
     gr->nbig = g->grid_cnt + cells;
     return launch_box_grid(g->dp, boxes, *gr, g->grid_cnt, g->grid_start, g->grid_list,
-                           packed ? g->grid_packed : nullptr, g->grid_big, g->grid_cnt + cells, st);
+                           packed ? g->grid_packed : nullptr, g->grid_big, g->grid_cnt + cells, g->grid_shape, st);
 }
 }  // namespace
 

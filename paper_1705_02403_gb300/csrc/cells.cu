@@ -35,12 +35,12 @@ __global__ void __launch_bounds__(kCellWarps * 32) cells_tile_kernel(SpaceArgs s
 
 // ---- box grid (checks against many boxes)
 // The cell range [c0, c1] of box b on the grid's axes (empty when lo > hi).
-__device__ __forceinline__ void box_grid_range(const BoxGridArgs& g, const float* lo, const float* hi, int* c0,
-                                               int* c1) {
+__device__ __forceinline__ void box_grid_range(const BoxGridArgs& grid, const int* g, const float* inv_h,
+                                               const float* lo, const float* hi, int* c0, int* c1) {
 #pragma unroll
     for (int a = 0; a < 2; ++a) {
-        c0[a] = box_grid_cell(g, lo[a], a);
-        c1[a] = box_grid_cell(g, hi[a], a);
+        c0[a] = box_grid_cell(grid, lo[a], a, g[a], inv_h[a]);
+        c1[a] = box_grid_cell(grid, hi[a], a, g[a], inv_h[a]);
     }
 }
 
@@ -50,8 +50,9 @@ __global__ void __launch_bounds__(256) box_grid_count_kernel(BoxArgs boxes, int 
                                                              int* __restrict__ nbig) {
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= boxes.count) return;
+    const int g[2] = {grid.g, grid.g};
     int c0[2], c1[2];
-    box_grid_range(grid, boxes.lo + (size_t)b * dp, boxes.hi + (size_t)b * dp, c0, c1);
+    box_grid_range(grid, g, grid.inv_h, boxes.lo + (size_t)b * dp, boxes.hi + (size_t)b * dp, c0, c1);
     if (c0[0] > c1[0] || c0[1] > c1[1]) return;  // lo > hi: the box holds no point
     if ((c1[0] - c0[0] + 1) * (c1[1] - c0[1] + 1) > kBoxGridMaxCells) {
         big[atomicAdd(nbig, 1)] = b;
@@ -76,8 +77,9 @@ __global__ void __launch_bounds__(256) box_grid_scatter_kernel(BoxArgs boxes, in
                                                                int* __restrict__ list, float4* __restrict__ packed) {
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= boxes.count) return;
+    const int g[2] = {grid.g, grid.g};
     int c0[2], c1[2];
-    box_grid_range(grid, boxes.lo + (size_t)b * dp, boxes.hi + (size_t)b * dp, c0, c1);
+    box_grid_range(grid, g, grid.inv_h, boxes.lo + (size_t)b * dp, boxes.hi + (size_t)b * dp, c0, c1);
     if (c0[0] > c1[0] || c0[1] > c1[1]) return;
     if ((c1[0] - c0[0] + 1) * (c1[1] - c0[1] + 1) > kBoxGridMaxCells) return;
     for (int cy = c0[1]; cy <= c1[1]; ++cy)
@@ -90,62 +92,112 @@ __global__ void __launch_bounds__(256) box_grid_scatter_kernel(BoxArgs boxes, in
 // The whole grid by one block, its cell counts in shared memory: a plan with
 // many boxes builds it before the wavefront (and a build before sampling), so
 // three dependent launches and a memset cost more than the work (1500 boxes:
-// 18.5 us of kernels in a row before).
+// 18.5 us of kernels in a row before).  The block also chooses the grid's
+// shape, from the boxes' mean extents: cells of the boxes' own proportions,
+// down to about half a box on each axis (a box then lies in about nine).
+// Obstacles cut into thin slices get thin cells: 1500 strips a hundred times
+// wider than high list 5 boxes a cell instead of 30 on square cells.
 __global__ void __launch_bounds__(1024) box_grid_block_kernel(BoxArgs boxes, int dp, BoxGridArgs grid,
                                                               int* __restrict__ start, int* __restrict__ list,
                                                               float4* __restrict__ packed, int* __restrict__ big,
-                                                              int* __restrict__ nbig) {
-    __shared__ int cnt[64 * 64];
+                                                              int* __restrict__ nbig, float4* __restrict__ shape) {
+    extern __shared__ int cnt[];  // kBoxGridCells
     __shared__ int warp_sum[32];
-    __shared__ int s_big;
-    const int cells = grid.g * grid.g, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    for (int c = tid; c < 64 * 64; c += 1024) cnt[c] = 0;
-    if (tid == 0) s_big = 0;
+    __shared__ float ext[3][32];
+    __shared__ int s_big, s_g[2];
+    __shared__ float s_inv[2];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    // mean extents of the boxes that hold points
+    float w[3] = {0.0f, 0.0f, 0.0f};
+    for (int b = tid; b < boxes.count; b += 1024) {
+        const float dx = boxes.hi[(size_t)b * dp] - boxes.lo[(size_t)b * dp];
+        const float dy = boxes.hi[(size_t)b * dp + 1] - boxes.lo[(size_t)b * dp + 1];
+        if (!(dx >= 0.0f) || !(dy >= 0.0f)) continue;
+        w[0] += fminf(dx, grid.span[0]);
+        w[1] += fminf(dy, grid.span[1]);
+        w[2] += 1.0f;
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) w[k] += __shfl_xor_sync(0xffffffffu, w[k], o);
+        if (lane == 0) ext[k][warp] = w[k];
+    }
     __syncthreads();
+    if (warp == 0) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            w[k] = ext[k][lane];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) w[k] += __shfl_xor_sync(0xffffffffu, w[k], o);
+        }
+        if (lane == 0) {
+            const float n = fmaxf(w[2], 1.0f);
+            const float fx = fmaxf(w[0] / (n * grid.span[0]), 1e-4f), fy = fmaxf(w[1] / (n * grid.span[1]), 1e-4f);
+            int P = 1;
+            while (P < kBoxGridCells && 2.0f * (float)P * fx * fy <= 4.0f) P *= 2;
+            int gy = 1;
+            while (gy < P && fx * (float)(P / gy) > 2.0f * fy * (float)gy) gy *= 2;
+            s_g[0] = P / gy;
+            s_g[1] = gy;
+#pragma unroll
+            for (int a = 0; a < 2; ++a) s_inv[a] = (float)s_g[a] / grid.span[a];
+            *shape = make_float4(__int_as_float(s_g[0]), __int_as_float(s_g[1]), s_inv[0], s_inv[1]);
+            s_big = 0;
+        }
+    }
+    for (int c = tid; c < kBoxGridCells; c += 1024) cnt[c] = 0;
+    __syncthreads();
+    const int g[2] = {s_g[0], s_g[1]}, cells = g[0] * g[1];
+    const float inv[2] = {s_inv[0], s_inv[1]};
     for (int b = tid; b < boxes.count; b += 1024) {
         int c0[2], c1[2];
-        box_grid_range(grid, boxes.lo + (size_t)b * dp, boxes.hi + (size_t)b * dp, c0, c1);
+        box_grid_range(grid, g, inv, boxes.lo + (size_t)b * dp, boxes.hi + (size_t)b * dp, c0, c1);
         if (c0[0] > c1[0] || c0[1] > c1[1]) continue;  // lo > hi: the box holds no point
         if ((c1[0] - c0[0] + 1) * (c1[1] - c0[1] + 1) > kBoxGridMaxCells) {
             big[atomicAdd(&s_big, 1)] = b;
             continue;
         }
         for (int cy = c0[1]; cy <= c1[1]; ++cy)
-            for (int cx = c0[0]; cx <= c1[0]; ++cx) atomicAdd(&cnt[cy * grid.g + cx], 1);
+            for (int cx = c0[0]; cx <= c1[0]; ++cx) atomicAdd(&cnt[cy * g[0] + cx], 1);
     }
     __syncthreads();
-    // exclusive prefix of the counts, four consecutive cells per thread
-    int v[4], sum = 0;
+    // exclusive prefix of the counts: a warp's run of cells, 32 at a time (a
+    // run per thread would meet 16-way bank conflicts)
+    constexpr int kPer = kBoxGridCells / 1024;
+    const int c0w = warp * 32 * kPer + lane;
+    int v[kPer], x[kPer], sum = 0;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        v[k] = cnt[4 * tid + k];
-        sum += v[k];
-    }
-    int incl = sum;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += y;
-    }
-    if (lane == 31) warp_sum[warp] = incl;
-    __syncthreads();
-    if (warp == 0) {
-        int w = warp_sum[lane];
+    for (int k = 0; k < kPer; ++k) {
+        v[k] = cnt[c0w + 32 * k];
+        x[k] = v[k];
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, w, o);
-            if (lane >= o) w += y;
+            const int y = __shfl_up_sync(0xffffffffu, x[k], o);
+            if (lane >= o) x[k] += y;
         }
-        warp_sum[lane] = w;
+        const int total = __shfl_sync(0xffffffffu, x[k], 31);
+        x[k] += sum - v[k];
+        sum += total;
+    }
+    if (lane == 31) warp_sum[warp] = sum;
+    __syncthreads();
+    if (warp == 0) {
+        int t = warp_sum[lane];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, t, o);
+            if (lane >= o) t += y;
+        }
+        warp_sum[lane] = t;
     }
     __syncthreads();
-    int at = (warp > 0 ? warp_sum[warp - 1] : 0) + incl - sum;
+    const int before = warp > 0 ? warp_sum[warp - 1] : 0, at = warp_sum[31];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const int c = 4 * tid + k;
-        cnt[c] = at;  // from here on the cell's next free entry
-        if (c < cells) start[c] = at;
-        at += v[k];
+    for (int k = 0; k < kPer; ++k) {
+        const int c = c0w + 32 * k;
+        cnt[c] = before + x[k];  // from here on the cell's next free entry
+        if (c < cells) start[c] = before + x[k];
     }
     if (tid == 1023) {
         start[cells] = at;  // the cells past the grid's are empty
@@ -154,20 +206,23 @@ __global__ void __launch_bounds__(1024) box_grid_block_kernel(BoxArgs boxes, int
     __syncthreads();
     for (int b = tid; b < boxes.count; b += 1024) {
         int c0[2], c1[2];
-        box_grid_range(grid, boxes.lo + (size_t)b * dp, boxes.hi + (size_t)b * dp, c0, c1);
+        box_grid_range(grid, g, inv, boxes.lo + (size_t)b * dp, boxes.hi + (size_t)b * dp, c0, c1);
         if (c0[0] > c1[0] || c0[1] > c1[1]) continue;
         if ((c1[0] - c0[0] + 1) * (c1[1] - c0[1] + 1) > kBoxGridMaxCells) continue;
         for (int cy = c0[1]; cy <= c1[1]; ++cy)
             for (int cx = c0[0]; cx <= c1[0]; ++cx)
-                box_grid_put(boxes, dp, b, atomicAdd(&cnt[cy * grid.g + cx], 1), list, packed);
+                box_grid_put(boxes, dp, b, atomicAdd(&cnt[cy * g[0] + cx], 1), list, packed);
     }
 }
 
 cudaError_t launch_box_grid(int dp, BoxArgs boxes, const BoxGridArgs& grid, int* cnt, int* start, int* list,
-                            float4* packed, int* big, int* nbig, cudaStream_t st) {
+                            float4* packed, int* big, int* nbig, float4* shape, cudaStream_t st) {
     if (dp < 2 || boxes.count < 1 || grid.g > 64) return cudaErrorInvalidValue;
     if (boxes.count <= kBoxGridBlockMax) {
-        box_grid_block_kernel<<<1, 1024, 0, st>>>(boxes, dp, grid, start, list, packed, big, nbig);
+        constexpr int smem = kBoxGridCells * (int)sizeof(int);
+        cudaError_t e = cudaFuncSetAttribute(box_grid_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+        box_grid_block_kernel<<<1, 1024, smem, st>>>(boxes, dp, grid, start, list, packed, big, nbig, shape);
         return cudaGetLastError();
     }
     cudaError_t me = cudaMemsetAsync(cnt, 0, (size_t)grid.g * grid.g * sizeof(int), st);

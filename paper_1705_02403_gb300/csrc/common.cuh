@@ -164,10 +164,26 @@ __device__ __forceinline__ bool in_any_box(const float* p, const float* lo, cons
     return false;
 }
 
-// Grid cell of coordinate x on grid axis a, clamped to the grid.
-__device__ __forceinline__ int box_grid_cell(const BoxGridArgs& g, float x, int a) {
-    const int k = (int)floorf((x - g.lo[a]) * g.inv_h[a]);
-    return min(max(k, 0), g.g - 1);
+// Grid cell of coordinate x on grid axis a, clamped to the grid's g cells.
+__device__ __forceinline__ int box_grid_cell(const BoxGridArgs& grid, float x, int a, int g, float inv_h) {
+    const int k = (int)floorf((x - grid.lo[a]) * inv_h);
+    return min(max(k, 0), g - 1);
+}
+
+// The list of the cell that holds p: entries [first, end).
+__device__ __forceinline__ void box_grid_entries(const BoxGridArgs& grid, const float* p, int& first, int& end) {
+    int gx = grid.g, gy = grid.g;
+    float ix = grid.inv_h[0], iy = grid.inv_h[1];
+    if (grid.shape) {
+        const float4 s = __ldg(grid.shape);
+        gx = __float_as_int(s.x);
+        gy = __float_as_int(s.y);
+        ix = s.z;
+        iy = s.w;
+    }
+    const int c = box_grid_cell(grid, p[1], 1, gy, iy) * gx + box_grid_cell(grid, p[0], 0, gx, ix);
+    first = __ldg(&grid.start[c]);
+    end = __ldg(&grid.start[c + 1]);
 }
 
 // Box t of the grid's list holds p: through the packed copies in list order
@@ -198,9 +214,9 @@ __device__ __forceinline__ bool grid_entry_holds(const float* p, const float* bl
 template <int DP>
 __device__ __forceinline__ bool in_any_box_grid(const float* p, const float* blo, const float* bhi,
                                                 const BoxGridArgs& grid) {
-    const int c = box_grid_cell(grid, p[1], 1) * grid.g + box_grid_cell(grid, p[0], 0);
-    const int e = __ldg(&grid.start[c + 1]);
-    for (int t = __ldg(&grid.start[c]); t < e; t += 4) {
+    int t, e;
+    box_grid_entries(grid, p, t, e);
+    for (; t < e; t += 4) {
         bool h = false;
 #pragma unroll
         for (int u = 0; u < 4; ++u) h = h | grid_entry_holds<DP>(p, blo, bhi, grid, min(t + u, e - 1));

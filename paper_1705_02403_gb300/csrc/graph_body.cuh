@@ -117,9 +117,9 @@ __device__ __forceinline__ bool point_in_boxes_group(const float* p, const BoxAr
                                                      int sub, unsigned gmask) {
     bool hit = false;
     if (grid.use) {
-        const int c = box_grid_cell(grid, p[1], 1) * grid.g + box_grid_cell(grid, p[0], 0);
-        const int e = __ldg(&grid.start[c + 1]);
-        for (int t = __ldg(&grid.start[c]) + sub; t < e; t += G) hit |= grid_entry_holds<DP>(p, boxes.lo, boxes.hi, grid, t);
+        int first, e;
+        box_grid_entries(grid, p, first, e);
+        for (int t = first + sub; t < e; t += G) hit |= grid_entry_holds<DP>(p, boxes.lo, boxes.hi, grid, t);
         const int nb = __ldg(grid.nbig);
         for (int t = sub; t < nb; t += G) hit |= in_box<DP>(p, boxes.lo, boxes.hi, __ldg(&grid.big[t]));
     } else {
@@ -904,7 +904,7 @@ __device__ __forceinline__ void mask_di_tile(const SpaceArgs& s, const float* __
 // the shortest-word cost for the ~3% that pass, 32 at a time from a per-warp
 // queue (entry (row lane << 8) | column) so that every lane computes one.
 constexpr int kDubRows = 128;  // rows (threads) per block
-constexpr int kDubWords = 1;   // 32-column words per block
+constexpr int kDubWords = 4;   // 32-column words per block
 
 // maskT, in_count (may be NULL): also write the tile's words of the transposed
 // (in-neighbour) matrix and count the in-edges, as transpose_task would.
@@ -919,10 +919,9 @@ __device__ __forceinline__ void mask_dubins_tile(const SpaceArgs& s, const float
                                                  int4* __restrict__ elist = nullptr,
                                                  float4* __restrict__ epath = nullptr,
                                                  int* __restrict__ elist_n = nullptr, int elist_cap = 0) {
-    static_assert(kDubWords == 1, "the prefilter keeps a lane's columns in one 32-bit word");
-    __shared__ float tile[4][kDubWords * 32];
+    __shared__ __align__(8) float tile[4][kDubWords * 32];
     __shared__ uint32_t words[kDubRows / 32][kDubWords][32];
-    __shared__ uint16_t queue[kDubRows / 32][32 * 32];  // every pair of the warp's tile may pass the prefilter
+    __shared__ uint16_t queue[kDubRows / 32][32 * 32 + 32];  // a word's passing pairs and the ones left before it
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int i = bx * kDubRows + threadIdx.x;
     const int j0 = by * kDubWords * 32;
@@ -938,60 +937,81 @@ __device__ __forceinline__ void mask_dubins_tile(const SpaceArgs& s, const float
     float xi[4];
 #pragma unroll
     for (int a = 0; a < 4; ++a) xi[a] = row_ok ? X[(size_t)a * s.pitch + i] : 0.0f;
-    // prefilter of the lane's row against every staged column, one bit per
-    // column; the passing pairs are then queued all at once and their costs
-    // computed 32 at a time (one per lane)
-    const int jend = min(kDubWords * 32, s.N - j0);
-    uint32_t pm = 0;
-    if (row_ok) {
-        for (int jt = 0; jt < jend; ++jt) {
-            float b_[4];
+    unsigned long long xi2[3];
 #pragma unroll
-            for (int a = 0; a < 4; ++a) b_[a] = tile[a][jt];
-            pm |= (dubins_near(xi, b_, s.r) ? 1u : 0u) << jt;
+    for (int a = 0; a < 3; ++a) xi2[a] = f2_pack(xi[a], xi[a]);
+    const float near = (s.r * s.r) * 1.015625f;  // dubins_near's bound
+    // A word at a time: the prefilter of the lane's row against the word's
+    // columns, two per step in packed arithmetic (the operations of
+    // dubins_near), one bit per column; the passing pairs join the warp's queue
+    // and their costs are computed whenever 32 wait (one per lane).  About 3% of
+    // the pairs pass, 31 per word of 32 rows: a queue drained after every word
+    // left a third of the lanes idle in the words' 1400 operations (95 us at n =
+    // 5000; over four words 67 us).
+    int qn = 0;
+#pragma unroll 1
+    for (int ww = 0; ww < kDubWords; ++ww) {
+        const int jw = ww * 32, jend = min(32, s.N - j0 - jw);
+        uint32_t pm = 0;
+        if (row_ok && jend > 0) {
+#pragma unroll 8
+            for (int jt = 0; jt < 32; jt += 2) {
+                const float2 bx2 = *reinterpret_cast<const float2*>(&tile[0][jw + jt]);
+                const float2 by2 = *reinterpret_cast<const float2*>(&tile[1][jw + jt]);
+                const float2 bz2 = *reinterpret_cast<const float2*>(&tile[2][jw + jt]);
+                const unsigned long long dx = f2_sub(f2_pack(bx2.x, bx2.y), xi2[0]);
+                const unsigned long long dy = f2_sub(f2_pack(by2.x, by2.y), xi2[1]);
+                const unsigned long long dz = f2_sub(f2_pack(bz2.x, bz2.y), xi2[2]);
+                float da, db;
+                f2_unpack(f2_add(f2_add(f2_mul(dx, dx), f2_mul(dy, dy)), f2_mul(dz, dz)), da, db);
+                pm |= (da < near ? 1u : 0u) << jt;
+                pm |= (db < near ? 1u : 0u) << (jt + 1);
+            }
+            if (jend < 32) pm &= (1u << jend) - 1u;  // columns past the last node
+            if (i >= j0 + jw && i < j0 + jw + jend) pm &= ~(1u << (i - j0 - jw));  // no self pair
         }
-        if (i >= j0 && i < j0 + jend) pm &= ~(1u << (i - j0));  // no self pair
-    }
-    int qn;
-    {
-        const int np = __popc(pm);
-        int incl = np;
+        {
+            const int np = __popc(pm);
+            int incl = np;
 #pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, incl, off);
-            if (lane >= off) incl += y;
+            for (int off = 1; off < 32; off <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, incl, off);
+                if (lane >= off) incl += y;
+            }
+            int pos = qn + incl - np;
+            for (uint32_t m = pm; m; m &= m - 1) queue[warp][pos++] = (uint16_t)((lane << 8) | (jw + __ffs(m) - 1));
+            qn += __shfl_sync(0xffffffffu, incl, 31);
+            __syncwarp();
         }
-        qn = __shfl_sync(0xffffffffu, incl, 31);
-        int pos = incl - np;
-        for (uint32_t m = pm; m; m &= m - 1) queue[warp][pos++] = (uint16_t)((lane << 8) | (__ffs(m) - 1));
-        __syncwarp();
-    }
-    for (int from = 0; from < qn; from += 32) {
-        const int count = min(32, qn - from);
-        const int e = lane < count ? queue[warp][from + lane] : 0;
-        const int src = e >> 8, jt = e & 255;
-        float a_[4], b_[4];
+        while (qn >= 32 || (qn > 0 && ww == kDubWords - 1)) {  // from the queue's end
+            const int count = min(32, qn);
+            qn -= count;
+            const int e = lane < count ? queue[warp][qn + lane] : 0;
+            const int src = e >> 8, jt = e & 255;
+            float a_[4], b_[4];
 #pragma unroll
-        for (int a = 0; a < 4; ++a) {
-            a_[a] = __shfl_sync(0xffffffffu, xi[a], src);
-            b_[a] = tile[a][jt];
-        }
-        // the steps of dubins_cost
-        const DubPath P = dubins_path(a_, b_, s.rho);
-        const float c = dubins_length(P, a_, b_);
-        const bool edge = lane < count && c < s.r;
-        if (edge) atomicOr(&words[warp][jt >> 5][src], 1u << (jt & 31));
-        if (elist) {
-            const unsigned m = __ballot_sync(0xffffffffu, edge);
-            if (m) {
-                int slot = 0;
-                if (lane == 0) slot = atomicAdd(elist_n, __popc(m));
-                slot = __shfl_sync(0xffffffffu, slot, 0) + __popc(m & ((1u << lane) - 1u));
-                if (edge && slot < elist_cap) {
-                    elist[slot] = make_int4(bx * kDubRows + warp * 32 + src, j0 + jt, __float_as_int(c), 0);
-                    epath[slot] = make_float4(P.t, P.p, P.q, __int_as_float(P.word));
+            for (int a = 0; a < 4; ++a) {
+                a_[a] = __shfl_sync(0xffffffffu, xi[a], src);
+                b_[a] = tile[a][jt];
+            }
+            // the steps of dubins_cost
+            const DubPath P = dubins_path(a_, b_, s.rho);
+            const float c = dubins_length(P, a_, b_);
+            const bool edge = lane < count && c < s.r;
+            if (edge) atomicOr(&words[warp][jt >> 5][src], 1u << (jt & 31));
+            if (elist) {
+                const unsigned m = __ballot_sync(0xffffffffu, edge);
+                if (m) {
+                    int slot = 0;
+                    if (lane == 0) slot = atomicAdd(elist_n, __popc(m));
+                    slot = __shfl_sync(0xffffffffu, slot, 0) + __popc(m & ((1u << lane) - 1u));
+                    if (edge && slot < elist_cap) {
+                        elist[slot] = make_int4(bx * kDubRows + warp * 32 + src, j0 + jt, __float_as_int(c), 0);
+                        epath[slot] = make_float4(P.t, P.p, P.q, __int_as_float(P.word));
+                    }
                 }
             }
+            __syncwarp();  // the next word's pairs overwrite the queue's end
         }
     }
     __syncwarp();
@@ -1000,17 +1020,21 @@ __device__ __forceinline__ void mask_dubins_tile(const SpaceArgs& s, const float
         // transposed: for column j0 + jt, the bits of the warp's 32 rows form
         // word (row chunk, j0 + jt) of the in-neighbour matrix
         const int chunk = (bx * kDubRows) / 32 + warp;
-        const uint32_t mine = row_ok ? words[warp][0][lane] : 0u;
         if (chunk < W) {  // uniform over the warp
-            uint32_t tw = 0;  // lane jt keeps column j0 + jt's word
+#pragma unroll 1
+            for (int ww = 0; ww < kDubWords; ++ww) {
+                const int j = j0 + ww * 32 + lane;
+                const uint32_t mine = row_ok ? words[warp][ww][lane] : 0u;
+                uint32_t tw = 0;  // lane jt keeps column jt's word
 #pragma unroll
-            for (int jt = 0; jt < 32; ++jt) {
-                const uint32_t t = __ballot_sync(0xffffffffu, (mine >> jt) & 1u);
-                if (lane == jt) tw = t;
-            }
-            if (j0 + lane < s.N) {  // one coalesced store and one atomic per lane
-                maskT[(size_t)chunk * s.pitch + j0 + lane] = tw;
-                if (tw) atomicAdd(&in_count[j0 + lane], __popc(tw));
+                for (int jt = 0; jt < 32; ++jt) {
+                    const uint32_t t = __ballot_sync(0xffffffffu, (mine >> jt) & 1u);
+                    if (lane == jt) tw = t;
+                }
+                if (j < s.N) {  // one coalesced store and one atomic per lane
+                    maskT[(size_t)chunk * s.pitch + j] = tw;
+                    if (tw) atomicAdd(&in_count[j], __popc(tw));
+                }
             }
         }
     }

@@ -44,12 +44,14 @@ struct BoxArgs {
 // that holds a point p is listed in p's cell: lo <= p <= hi gives
 // cell(lo) <= cell(p) <= cell(hi), since every step of cell() is monotone in
 // IEEE arithmetic.  A query tests the boxes of p's cell and the big boxes
-// exactly, so its verdict equals testing every box.
+// exactly, so its verdict equals testing every box, whatever the cells.
 struct BoxGridArgs {
     int use;            // 0: scan every box
-    int g;              // cells per axis
+    int g;              // cells per axis, with inv_h, where shape is NULL
     float lo[2], inv_h[2];
-    const int* start;   // [g * g + 1] first list entry of each cell
+    float span[2];      // the grid's extent
+    const float4* shape;  // cells on each axis (int bits) and their inverse sizes, chosen on the device, or NULL
+    const int* start;   // [cells + 1] first list entry of each cell
     const int* list;    // box indices, grouped by cell
     const float4* packed;  // 2D/3D: the boxes of `list` in its order (lo then hi, one or two float4s), or NULL
     const int* big;     // indices of the boxes over more than kBoxGridMaxCells cells
@@ -59,7 +61,9 @@ struct BoxGridArgs {
 constexpr int kBoxGridMinBoxes = 128;
 // Cells a box may be listed in before it goes to the big-box list.
 constexpr int kBoxGridMaxCells = 32;
-// Cells per axis for `count` boxes.
+// Most cells of a grid whose shape is chosen on the device.
+constexpr int kBoxGridCells = 16384;
+// Cells per axis for `count` boxes, for a grid shaped on the host.
 inline int box_grid_cells(int count) {
     int g = 1;
     while (g < 64 && g * g < count) g *= 2;
@@ -72,11 +76,12 @@ constexpr int kBoxGridBlockMax = 8192;
 // Boxes up to which the list also keeps packed copies (2D and 3D; at most
 // kBoxGridMaxCells copies of 32 bytes per box).
 constexpr int kBoxGridPackMax = 65536;
-// Builds the grid: cnt [g*g], nbig [1], start [g*g + 1],
+// Builds the grid: cnt [g*g], nbig [1], start [max(g*g, kBoxGridCells) + 1],
 // list [count * kBoxGridMaxCells], packed [as many entries of 1 (2D) or 2 (3D)
-// float4s] or NULL, big [count].
+// float4s] or NULL, big [count], shape [1].  Up to kBoxGridBlockMax boxes the
+// shape is chosen on the device (the caller sets grid.shape then).
 cudaError_t launch_box_grid(int dp, BoxArgs boxes, const BoxGridArgs& grid, int* cnt, int* start, int* list,
-                            float4* packed, int* big, int* nbig, cudaStream_t st);
+                            float4* packed, int* big, int* nbig, float4* shape, cudaStream_t st);
 
 // Flags written by the sampling kernel.
 enum { kSampleBadInit = 1, kSampleExhausted = 2, kSampleBadAppend = 4, kSampleTimeout = 8 };
