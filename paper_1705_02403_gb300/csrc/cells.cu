@@ -96,7 +96,10 @@ __global__ void __launch_bounds__(256) box_grid_scatter_kernel(BoxArgs boxes, in
 // shape, from the boxes' mean extents: cells of the boxes' own proportions,
 // down to about half a box on each axis (a box then lies in about nine).
 // Obstacles cut into thin slices get thin cells: 1500 strips a hundred times
-// wider than high list 5 boxes a cell instead of 30 on square cells.
+// wider than high list 2.9 boxes an occupied cell (9 at most) on 16 x 1024
+// cells, 25 (59 at most) on 64 x 64.  This kernel takes 18 us for them; the
+// Dubins plan kernel at n = 5000 went from 0.251 to 0.163 ms, its Halton
+// sampler from 43 to 21 us.
 __global__ void __launch_bounds__(1024) box_grid_block_kernel(BoxArgs boxes, int dp, BoxGridArgs grid,
                                                               int* __restrict__ start, int* __restrict__ list,
                                                               float4* __restrict__ packed, int* __restrict__ big,

@@ -947,7 +947,7 @@ __device__ __forceinline__ void mask_dubins_tile(const SpaceArgs& s, const float
     // and their costs are computed whenever 32 wait (one per lane).  About 3% of
     // the pairs pass, 31 per word of 32 rows: a queue drained after every word
     // left a third of the lanes idle in the words' 1400 operations (95 us at n =
-    // 5000; over four words 67 us).
+    // 5000; over four words 91 us).
     int qn = 0;
 #pragma unroll 1
     for (int ww = 0; ww < kDubWords; ++ww) {

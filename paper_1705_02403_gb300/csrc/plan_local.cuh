@@ -41,7 +41,8 @@
 // in L2 (plan kernel, mean over four seeds): 2D n = 1024 0.157 -> 0.107 ms,
 // 2D n = 30000 0.988 -> 0.619, 3D n = 16384 0.421 -> 0.274, 6D n = 5000 (a
 // thousand neighbours a node) 0.407 -> 0.256, double integrator n = 4096
-// 0.110 -> 0.078, Dubins airplane n = 5000 with 1500 boxes 0.363 -> 0.251.
+// 0.110 -> 0.078, Dubins airplane n = 5000 with 1500 boxes 0.363 -> 0.251
+// (0.163 since the box grid's cells have the boxes' proportions).
 // The same body on a cooperative grid of 38 to 152 CTAs (lists of changes and
 // marks through L2, a polled word per CTA as the barrier) was slower on all of
 // these but the 6D graph (equal): its two barriers cost 4-5 us an iteration.
