@@ -395,11 +395,11 @@ __device__ __forceinline__ void cell_tile(const SpaceArgs& s, const float* __res
                 const float4 q = reinterpret_cast<const float4*>(xy)[w * 16 + (b >> 1)];
                 const unsigned long long t0 = f2_sub(f2_pack(q.x, q.y), xi[0]);
                 const unsigned long long t1 = f2_sub(f2_pack(q.z, q.w), xi[1]);
-                unsigned long long d2 = f2_add(f2_mul(t0, t0), f2_mul(t1, t1));
+                unsigned long long d2 = f2_add(f2_sqr(t0), f2_sqr(t1));  // the bits of sq_dist
                 if (D == 3) {
                     const float2 z = reinterpret_cast<const float2*>(zz)[w * 16 + (b >> 1)];
                     const unsigned long long t2 = f2_sub(f2_pack(z.x, z.y), xi[2]);
-                    d2 = f2_add(d2, f2_mul(t2, t2));
+                    d2 = f2_add(d2, f2_sqr(t2));
                 }
                 float da, db;
                 f2_unpack(d2, da, db);

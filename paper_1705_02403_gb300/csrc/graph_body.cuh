@@ -364,7 +364,12 @@ __device__ __forceinline__ float edge_cost(const SpaceArgs& s, const float* from
 }
 
 // Packed FP32 pairs (two IEEE round-to-nearest operations per instruction,
-// each lane of the pair rounded on its own: the same bits as two scalar ops).
+// each lane of the pair rounded on its own).  One operation gives the bits of
+// two scalar ones, but the assembler contracts a packed multiplication with
+// the addition that takes its result, in spite of .rn and -fmad=false: such a
+// sum then differs in the last bit from the scalar one (16% of t0 t0 + t1 t1,
+// 21% with a third term, on random values).  Where the sum decides something
+// without slack, squares come from f2_sqr.
 __device__ __forceinline__ unsigned long long f2_pack(float lo, float hi) {
     unsigned long long r;
     asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
@@ -389,9 +394,20 @@ __device__ __forceinline__ unsigned long long f2_add(unsigned long long a, unsig
     return r;
 }
 
+// a * a, rounded before anything is added to it: an FMA with -0, which is
+// exact there, and whose addend the assembler cannot know.  No instruction
+// more than the multiplication (none of 15.6 M sums differed from scalar ones).
+static __constant__ unsigned long long f2_neg_zero = 0x8000000080000000ull;
+__device__ __forceinline__ unsigned long long f2_sqr(unsigned long long a) {
+    unsigned long long r;
+    asm("fma.rn.f32x2 %0, %1, %1, %2;" : "=l"(r) : "l"(a), "l"(f2_neg_zero));
+    return r;
+}
+
 // di_may_connect for two pairs at once (s0a -> s1a and s0b -> s1b): the same
 // operations in the same order, the additions and multiplications packed two
-// to an instruction, so each verdict is the scalar function's.
+// to an instruction (a filter with slack: a contracted sum's last bit does not
+// decide an edge).
 __device__ __forceinline__ void di_may_connect_x2(const float* s0a, const float* s1a, const float* s0b,
                                                   const float* s1b, float r, bool& pass_a, bool& pass_b) {
     const float rr = r * 1.01f;
@@ -963,7 +979,7 @@ __device__ __forceinline__ void mask_dubins_tile(const SpaceArgs& s, const float
                 const unsigned long long dy = f2_sub(f2_pack(by2.x, by2.y), xi2[1]);
                 const unsigned long long dz = f2_sub(f2_pack(bz2.x, bz2.y), xi2[2]);
                 float da, db;
-                f2_unpack(f2_add(f2_add(f2_mul(dx, dx), f2_mul(dy, dy)), f2_mul(dz, dz)), da, db);
+                f2_unpack(f2_add(f2_add(f2_sqr(dx), f2_sqr(dy)), f2_sqr(dz)), da, db);
                 pm |= (da < near ? 1u : 0u) << jt;
                 pm |= (db < near ? 1u : 0u) << (jt + 1);
             }
