@@ -56,16 +56,6 @@ __device__ __forceinline__ Ctr4 philox4x32_10(Ctr4 c, uint32_t k0, uint32_t k1) 
     return c;
 }
 
-// Position of the m-th (from 0) set bit of x (x has more than m set bits):
-// the largest p with fewer than m + 1 set bits below it, by binary search.
-__device__ __forceinline__ int select_bit(uint32_t x, int m) {
-    int p = 0;
-#pragma unroll
-    for (int step = 16; step > 0; step >>= 1)
-        if (__popc(x & ((1u << (p + step)) - 1u)) <= m) p += step;
-    return p;
-}
-
 // Top 24 bits of a word scaled by 2^-24: exact, in [0, 1).
 __device__ __forceinline__ float unit_float(uint32_t w) { return (float)(w >> 8) * 0x1p-24f; }
 

@@ -459,7 +459,9 @@ __device__ __forceinline__ void di_may_connect_x2(const float* s0a, const float*
 // (x_j, x_j+1, y_j, y_j+1), then (z_j, z_j+1, w_j, w_j+1)), and each lane
 // tests its row against two columns per step with packed FP32 arithmetic:
 // t = x_j - x_i, then d2 = t_0^2 + t_1^2 + ... in axis order, which is the
-// expression of sq_dist (0 + t_0^2 = t_0^2 exactly), so the bits are the same.
+// expression of sq_dist (0 + t_0^2 = t_0^2 exactly) but for the rounding of a
+// square that the assembler contracts with its addition (see f2_mul): a pair
+// within one rounding of the radius can be decided otherwise than sq_dist does.
 // Columns past the last node hold +inf (an infinite distance: no edge), so
 // the inner loop tests no bounds; the diagonal pair i = j is cleared once per
 // word.  tile_cnt (or NULL): receives the row's edge count in this tile's

@@ -2,38 +2,13 @@
 //
 // A "team" of threads runs every wavefront iteration of one plan without
 // returning to the host: one CTA (block barriers), one thread-block cluster
-// (hardware cluster barriers) or a cooperative grid (bounded global
-// barriers, co-residency guaranteed by the cooperative launch).  Each
-// iteration i has two phases separated by team barriers:
+// (hardware cluster barriers) or a cooperative grid (bounded global barriers,
+// co-residency guaranteed by the cooperative launch).
 //
-//   1  the open-set snapshot `ocost` (cost if open, +inf otherwise) is
-//      brought up to date with the previous iteration (its group closed, the
-//      nodes it opened set to their costs); group selection (Alg. 1's group) splits
-//      the open list into G_i = {v open : cost(v) <= theta_i} and the nodes
-//      that stay open; the warp that selects a node of G_i at once pushes it
-//      (the frontier push): it scans the node's out-row and claims every unexplored
-//      neighbour once per iteration through one atomicMax on its stamp
-//      (INT_MAX marks tree nodes), appending it to the candidate list.
-//      Nothing reads the snapshot in this phase.
-//   2  lazy parent, check and commit: one warp per candidate x scans its in-row,
-//      gathers the snapshot and takes argmin of (ocost[y] + c(y, x), y); the
-//      warp checks that single edge (points spread over the lanes) and, if it
-//      is free, commits parent and cost and appends x to the next open list.
-//
-// Open entries carry their cost, so selection and the snapshot update need
-// no gathers.  Open entries are dealt to the team's CTAs round-robin first,
-// then to their warps, then to lanes, so that the nodes of a small group (and
-// their pushes) spread over the team.  An open list keeps the entries that
-// stay open at its front and the newly opened nodes at its back, so phase 1
-// of the next iteration finds exactly the nodes the snapshot lacks.
-//
-// After phase 2 every thread reads the same totals and decides (Alg. 1's termination test):
-// success if G_i held a goal node, failure if no node stays open, else the
-// next threshold index is the smallest i' > i with theta_{i'} >= min open cost
-// (iterations whose group would be empty are no-ops and are skipped).  Lists
-// are appended with one atomic per warp (ballot + popc prefix), the prefix-sum
-// compaction of Section IV.  Counters are double-buffered by parity so that
-// resets need no extra barrier.
+// A CTA or a cluster keeps the wavefront's state in its shared memory
+// (plan_body_local, plan_local.cuh) when it fits and the rows start on 16-byte
+// boundaries; other graphs and cooperative grids keep it in global memory
+// (plan_body_fused, plan_fused.cuh).  Both take the same decisions.
 #include <algorithm>
 
 #include "plan_core.cuh"

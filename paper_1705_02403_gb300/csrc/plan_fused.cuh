@@ -17,7 +17,7 @@
 // (iteration i uses set i % 3 and resets set (i + 1) % 3, last read two
 // barriers earlier), so no second barrier is needed for resets.
 //
-// Results, counters and the returned path are those of plan_body (the order
+// Results, counters and the returned path are those of plan_body_local (the order
 // in which candidates are handled does not change any decision: each lazy
 // parent is the minimum (cost, index) over the snapshot).
 #pragma once
