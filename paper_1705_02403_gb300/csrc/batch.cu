@@ -792,6 +792,7 @@ gmt_status prepare(gmt_batch* b, int q, const gmt_query* queries, int32_t* paren
         const bool applies = make_cell_grid(Qh.space.kind, Qh.space.dim, Qh.space.lo, Qh.space.hi, b->r[k], N,
                                             true, &cgs[k], &pays);
         if (dbg & GMT_DEBUG_CELLS_LIST) cgs[k].list_only = 1;
+        if (dbg & GMT_DEBUG_PAIRS_CELLS) cgs[k].pairs_sum = 0;
         use_cells[k] = applies && !(dbg & GMT_DEBUG_PAIRS_ALL) && (pays || (dbg & GMT_DEBUG_PAIRS_CELLS)) &&
                        !(k < (int)force_pairs.size() && force_pairs[k]);
         xo[k] = xs; xs += (size_t)Qh.space.dim * P;

@@ -470,6 +470,7 @@ gmt_status build_impl(const gmt_space* space, const gmt_boxes* boxes, const floa
     bool cells_pay = false;
     bool cells = make_cell_grid(g->kind, g->d, space->lo, space->hi, g->r, g->N, false, &cg, &cells_pay);
     if (params->debug_flags & GMT_DEBUG_CELLS_LIST) cg.list_only = 1;
+    if (params->debug_flags & GMT_DEBUG_PAIRS_CELLS) cg.pairs_sum = 0;
     if (params->debug_flags & GMT_DEBUG_PAIRS_ALL) cells = false;
     else if (!(params->debug_flags & GMT_DEBUG_PAIRS_CELLS)) cells = cells && cells_pay;
     // Euclidean graphs of 2 to 4 dimensions fill their CSR by mask tiles

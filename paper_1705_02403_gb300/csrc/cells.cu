@@ -274,11 +274,12 @@ bool make_cell_grid(int kind, int d, const float* lo, const float* hi, float r, 
     // cell stages' short launches overlap other queries' work, and they pay
     // sooner (builds of 400k nodes in all): 2D: 2500 nodes a query 0.58 against
     // 0.51, 4000 0.54 against 0.68; 3D: 4000 0.93 against 0.86, 6000 1.01
-    // against 1.11.  The line lies higher than these times ask for: the all-pairs
-    // tiles' packed sum of squares is contracted (see f2_mul) and the cells' is
-    // not, so a pair within a rounding of the radius can be an edge of one and
-    // not of the other, and a size that changes sides changes its graph.
-    *pays = frac <= 0.25 && N >= (d == 2 ? (batched ? 4096 : 12000) : 32768);
+    // against 1.11.
+    *pays = frac <= 0.3 && N >= (d == 2 ? (batched ? 3200 : 10500) : (batched ? 5000 : 14000));
+    // Cells that replace the all-pairs tiles form their sum, which rounds fewer
+    // squares than sq_dist, so that a graph does not depend on which of the two
+    // builds it.  Cells have formed sq_dist's from these lines on.
+    cg->pairs_sum = !(frac <= 0.25 && N >= (d == 2 ? (batched ? 4096 : 12000) : 32768));
     return true;
 }
 

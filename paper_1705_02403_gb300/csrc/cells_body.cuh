@@ -177,7 +177,7 @@ __device__ __forceinline__ void cell_row(const SpaceArgs& s, const float* __rest
             float xj[D];
 #pragma unroll
             for (int a = 0; a < D; ++a) xj[a] = X[(size_t)a * s.pitch + j];
-            pass = connects<GMT_COST_EUCLID, D>(s, xv, xj);
+            pass = cg.pairs_sum ? sq_dist_pairs<D>(xv, xj) < s.r2_threshold : connects<GMT_COST_EUCLID, D>(s, xv, xj);
         }
         const unsigned m = __ballot_sync(0xffffffffu, pass);
         if (bitmap) {
@@ -258,6 +258,31 @@ __device__ __forceinline__ void cell_row(const SpaceArgs& s, const float* __rest
         cost[b + t] = edge_cost<GMT_COST_EUCLID, D>(s, xv, xj);
     }
     __syncwarp();
+}
+
+// Verdicts of a row (its coordinates in both halves of xi) on candidates
+// 32 w to 32 w + 31.  PAIRS: the all-pairs tiles' sum, else sq_dist's.
+template <int D, bool PAIRS>
+__device__ __forceinline__ unsigned cell_verdicts(const float* xy, const float* zz, const unsigned long long* xi, int w,
+                                                  float thr) {
+    unsigned bits = 0u;
+#pragma unroll
+    for (int b = 0; b < 32; b += 2) {
+        const float4 q = reinterpret_cast<const float4*>(xy)[w * 16 + (b >> 1)];
+        const unsigned long long t0 = f2_sub(f2_pack(q.x, q.y), xi[0]);
+        const unsigned long long t1 = f2_sub(f2_pack(q.z, q.w), xi[1]);
+        unsigned long long d2 = PAIRS ? f2_sqr_add(t0, f2_mul(t1, t1)) : f2_add(f2_sqr(t0), f2_sqr(t1));
+        if (D == 3) {
+            const float2 z = reinterpret_cast<const float2*>(zz)[w * 16 + (b >> 1)];
+            const unsigned long long t2 = f2_sub(f2_pack(z.x, z.y), xi[2]);
+            d2 = PAIRS ? f2_sqr_add(t2, d2) : f2_add(d2, f2_sqr(t2));
+        }
+        float da, db;
+        f2_unpack(d2, da, db);
+        bits |= (da < thr ? 1u : 0u) << b;
+        bits |= (db < thr ? 1u : 0u) << (b + 1);
+    }
+    return bits;
 }
 
 // One CTA of kCellWarps warps: every row of cell `cell`.  smem:
@@ -389,23 +414,7 @@ __device__ __forceinline__ void cell_tile(const SpaceArgs& s, const float* __res
         }
         int cnt = 0;
         for (int w = warp; w < nw; w += kCellWarps) {
-            unsigned bits = 0u;
-#pragma unroll
-            for (int b = 0; b < 32; b += 2) {
-                const float4 q = reinterpret_cast<const float4*>(xy)[w * 16 + (b >> 1)];
-                const unsigned long long t0 = f2_sub(f2_pack(q.x, q.y), xi[0]);
-                const unsigned long long t1 = f2_sub(f2_pack(q.z, q.w), xi[1]);
-                unsigned long long d2 = f2_add(f2_sqr(t0), f2_sqr(t1));  // the bits of sq_dist
-                if (D == 3) {
-                    const float2 z = reinterpret_cast<const float2*>(zz)[w * 16 + (b >> 1)];
-                    const unsigned long long t2 = f2_sub(f2_pack(z.x, z.y), xi[2]);
-                    d2 = f2_add(d2, f2_sqr(t2));
-                }
-                float da, db;
-                f2_unpack(d2, da, db);
-                bits |= (da < thr ? 1u : 0u) << b;
-                bits |= (db < thr ? 1u : 0u) << (b + 1);
-            }
+            unsigned bits = cg.pairs_sum ? cell_verdicts<D, true>(xy, zz, xi, w, thr) : cell_verdicts<D, false>(xy, zz, xi, w, thr);
             if (!has) bits = 0u;
             if (FILL) {
                 if ((self >> 5) == w) bits &= ~(1u << (self & 31));

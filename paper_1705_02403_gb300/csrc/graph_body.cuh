@@ -404,6 +404,28 @@ __device__ __forceinline__ unsigned long long f2_sqr(unsigned long long a) {
     return r;
 }
 
+// a * a + c in one rounding.
+__device__ __forceinline__ unsigned long long f2_sqr_add(unsigned long long a, unsigned long long c) {
+    unsigned long long r;
+    asm("fma.rn.f32x2 %0, %1, %1, %2;" : "=l"(r) : "l"(a), "l"(c));
+    return r;
+}
+
+// The all-pairs tiles' sum of squares, for one pair: t_1^2 is rounded, the
+// other squares are added to it without a rounding of their own, t_0's first.
+// (Packed: f2_sqr_add of the axes in that order.)
+template <int D>
+__device__ __forceinline__ float sq_dist_pairs(const float* from, const float* to) {
+    const float t0 = to[0] - from[0], t1 = to[1] - from[1];
+    float s = __fmaf_rn(t0, t0, __fmul_rn(t1, t1));
+#pragma unroll
+    for (int a = 2; a < D; ++a) {
+        const float t = to[a] - from[a];
+        s = __fmaf_rn(t, t, s);
+    }
+    return s;
+}
+
 // di_may_connect for two pairs at once (s0a -> s1a and s0b -> s1b): the same
 // operations in the same order, the additions and multiplications packed two
 // to an instruction (a filter with slack: a contracted sum's last bit does not
@@ -458,10 +480,10 @@ __device__ __forceinline__ void di_may_connect_x2(const float* s0a, const float*
 // Euclidean graphs of 2 to 4 dimensions: columns are staged in pairs (float4
 // (x_j, x_j+1, y_j, y_j+1), then (z_j, z_j+1, w_j, w_j+1)), and each lane
 // tests its row against two columns per step with packed FP32 arithmetic:
-// t = x_j - x_i, then d2 = t_0^2 + t_1^2 + ... in axis order, which is the
-// expression of sq_dist (0 + t_0^2 = t_0^2 exactly) but for the rounding of a
-// square that the assembler contracts with its addition (see f2_mul): a pair
-// within one rounding of the radius can be decided otherwise than sq_dist does.
+// t = x_j - x_i, then sq_dist_pairs.  (The sum was written as packed products
+// and sums, which the assembler contracted to this; written out, it no longer
+// depends on it.)  A pair within one rounding of the radius can be decided
+// otherwise than by sq_dist.
 // Columns past the last node hold +inf (an infinite distance: no edge), so
 // the inner loop tests no bounds; the diagonal pair i = j is cleared once per
 // word.  tile_cnt (or NULL): receives the row's edge count in this tile's
@@ -509,14 +531,14 @@ __device__ __forceinline__ void mask_tile_euclid4(const SpaceArgs& s, const floa
             const float4 q = tab[ww * 16 + (b >> 1)];
             const unsigned long long t0 = f2_sub(f2_pack(q.x, q.y), xi2[0]);
             const unsigned long long t1 = f2_sub(f2_pack(q.z, q.w), xi2[1]);
-            unsigned long long d2 = f2_add(f2_mul(t0, t0), f2_mul(t1, t1));
+            unsigned long long d2 = f2_sqr_add(t0, f2_mul(t1, t1));
             if (D > 2) {
                 const float4 r = tcd[ww * 16 + (b >> 1)];
                 const unsigned long long t2 = f2_sub(f2_pack(r.x, r.y), xi2[2]);
-                d2 = f2_add(d2, f2_mul(t2, t2));
+                d2 = f2_sqr_add(t2, d2);
                 if (D > 3) {
                     const unsigned long long t3 = f2_sub(f2_pack(r.z, r.w), xi2[3]);
-                    d2 = f2_add(d2, f2_mul(t3, t3));
+                    d2 = f2_sqr_add(t3, d2);
                 }
             }
             float da, db;

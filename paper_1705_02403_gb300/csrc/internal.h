@@ -184,6 +184,7 @@ struct CellGrid {
     float inv_h;   // 1 / h
     int ncells;
     int list_only;  // the fill sorts a list even where a bitmap would fit (test hook)
+    int pairs_sum;  // the squared distance is the all-pairs tiles' (sq_dist_pairs), not sq_dist
 };
 // Shared-memory words per warp of the cell-list fill: a bitmap of the row's
 // columns for graphs of at most 32 kCellList nodes, else a list of at most
@@ -195,7 +196,8 @@ __host__ __device__ inline bool cell_fill_fits(const CellGrid& cg, int N, int ma
 constexpr int kCellList = 1024;
 // Returns false when the cell list does not apply (not a 2D/3D geometric
 // graph); *pays is false when the 3^d cells around a node would hold more than
-// a quarter of the domain.
+// three tenths of the domain.  A caller that forces cells where they do not pay
+// clears pairs_sum.
 bool make_cell_grid(int kind, int d, const float* lo, const float* hi, float r, int N, bool batched, CellGrid* cg,
                     bool* pays);
 cudaError_t launch_cells_count(const SpaceArgs& s, const float* X, const CellGrid& cg, int* cell_of, int* cell_cnt,
