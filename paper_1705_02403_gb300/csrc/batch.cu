@@ -109,13 +109,13 @@ __global__ void __launch_bounds__(kHaltonThreads) batch_halton_kernel(const Quer
 
 template <int KIND, int D>
 __global__ void __launch_bounds__(kMaskRows) batch_mask_kernel(const QueryDev* __restrict__ Q,
-                                                               const long long* __restrict__ off, int nq) {
+                                                               const long long* __restrict__ off, int nq, bool half) {
     const long long b = blockIdx.x;
     const int k = find_query(off, nq, b);
     const QueryDev& q = Q[k];
     const int rb = (q.s.N + kMaskRows - 1) / kMaskRows;
     const int t = (int)(b - off[k]);
-    mask_tile<KIND, D>(q.s, q.X, q.mask, q.out_count, t % rb, t / rb, q.tile_cnt);
+    mask_tile<KIND, D>(q.s, q.X, q.mask, q.out_count, t % rb, t / rb, q.tile_cnt, half);
 }
 
 __global__ void __launch_bounds__(kDIRows, 8) batch_mask_di_kernel(const QueryDev* __restrict__ Q,
@@ -262,7 +262,7 @@ template <int KIND, int D>
 void mask_g(const QueryDev* Q, const long long* off, int nq, long long tiles, cudaStream_t st) {
     if (KIND == GMT_COST_DI) batch_mask_di_kernel<<<(unsigned)tiles, kDIRows, 0, st>>>(Q, off, nq);
     else if (KIND == GMT_COST_DUBINS) batch_mask_dubins_kernel<<<(unsigned)tiles, kDubRows, 0, st>>>(Q, off, nq);
-    else batch_mask_kernel<KIND, D><<<(unsigned)tiles, kMaskRows, 0, st>>>(Q, off, nq);
+    else batch_mask_kernel<KIND, D><<<(unsigned)tiles, kMaskRows, 0, st>>>(Q, off, nq, half_mask(tiles));
 }
 template <int KIND, int D>
 void fill_g(const QueryDev* Q, const long long* off, int nq, long long rows, cudaStream_t st) {

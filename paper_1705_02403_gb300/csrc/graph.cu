@@ -178,8 +178,8 @@ template <int KIND, int D>
 __global__ void __launch_bounds__(kMaskRows) pair_mask_kernel(SpaceArgs s, const float* __restrict__ X,
                                                               uint32_t* __restrict__ mask,
                                                               int* __restrict__ out_count,
-                                                              int* __restrict__ tile_cnt) {
-    mask_tile<KIND, D>(s, X, mask, out_count, blockIdx.x, blockIdx.y, tile_cnt);
+                                                              int* __restrict__ tile_cnt, bool half) {
+    mask_tile<KIND, D>(s, X, mask, out_count, blockIdx.x, blockIdx.y, tile_cnt, half);
 }
 
 __global__ void __launch_bounds__(256) tile_prefix_kernel(int N, int pitch, int nb, int* __restrict__ tile_cnt) {
@@ -329,7 +329,7 @@ template <int KIND, int D>
 cudaError_t mask_t(const SpaceArgs& s, const float* X, uint32_t* mask, int* cnt, int* tile_cnt, cudaStream_t st) {
     const int W = (s.N + 31) / 32, nb = (W + kMaskWords - 1) / kMaskWords;
     dim3 grid((s.N + kMaskRows - 1) / kMaskRows, nb);
-    pair_mask_kernel<KIND, D><<<grid, kMaskRows, 0, st>>>(s, X, mask, cnt, tile_cnt);
+    pair_mask_kernel<KIND, D><<<grid, kMaskRows, 0, st>>>(s, X, mask, cnt, tile_cnt, half_mask(nb * nb));
     // the per-tile counts become prefixes here, so the fill reads them only
     // (and a fill run again on the same mask writes the same CSR)
     if (tile_cnt) tile_prefix_kernel<<<(s.N + 255) / 256, 256, 0, st>>>(s.N, s.pitch, nb, tile_cnt);

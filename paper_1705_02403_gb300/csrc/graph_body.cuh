@@ -484,6 +484,10 @@ __device__ __forceinline__ void di_may_connect_x2(const float* s0a, const float*
 // and sums, which the assembler contracted to this; written out, it no longer
 // depends on it.)  A pair within one rounding of the radius can be decided
 // otherwise than by sq_dist.
+// The sum is the same bits for (i, j) and (j, i), so with half only the tiles
+// on and above the diagonal are evaluated; each warp also writes the mirrored words of
+// an off-diagonal tile, a 32 x 32 bit transpose in its registers (30
+// instructions against the 280 that evaluating the block again would issue).
 // Columns past the last node hold +inf (an infinite distance: no edge), so
 // the inner loop tests no bounds; the diagonal pair i = j is cleared once per
 // word.  tile_cnt (or NULL): receives the row's edge count in this tile's
@@ -491,9 +495,12 @@ __device__ __forceinline__ void di_may_connect_x2(const float* s0a, const float*
 template <int D>
 __device__ __forceinline__ void mask_tile_euclid4(const SpaceArgs& s, const float* __restrict__ X,
                                                   uint32_t* __restrict__ mask, int* __restrict__ out_count, int bx,
-                                                  int by, int* __restrict__ tile_cnt) {
+                                                  int by, int* __restrict__ tile_cnt, bool half) {
     static_assert(D >= 2 && D <= 4, "two to four axes in two float4s per column pair");
+    static_assert(kMaskRows == kMaskWords * 32, "square tiles, mirrored at the diagonal");
+    if (half && by < bx) return;  // tile (by, bx) writes it
     constexpr int kPairs = kMaskWords * 16;
+    __shared__ int col_cnt[kMaskRows];              // the mirrored rows' edges
     __shared__ float4 tab[kPairs];                  // axes 0 and 1
     __shared__ float4 tcd[D > 2 ? kPairs : 1];      // axes 2 and 3
     const int i = bx * kMaskRows + threadIdx.x;
@@ -511,8 +518,11 @@ __device__ __forceinline__ void mask_tile_euclid4(const SpaceArgs& s, const floa
         tab[idx] = make_float4(c[0][0], c[1][0], c[0][1], c[1][1]);
         if (D > 2) tcd[idx] = make_float4(c[0][2], c[1][2], c[0][3], c[1][3]);
     }
+    const bool mirror = half && by > bx, row_ok = i < s.N;  // mirror: all rows of the tile are nodes
+    col_cnt[threadIdx.x] = 0;
     __syncthreads();
-    if (i >= s.N) return;
+    if (!row_ok && !mirror) return;
+    const int lane = threadIdx.x & 31;
     unsigned long long xi2[4];
 #pragma unroll
     for (int a = 0; a < D; ++a) {
@@ -549,6 +559,27 @@ __device__ __forceinline__ void mask_tile_euclid4(const SpaceArgs& s, const floa
         if ((i >> 5) == w) bits &= ~(1u << (i & 31));  // no self-loop
         mask[(size_t)w * s.pitch + i] = bits;
         cnt += __popc(bits);
+        if (mirror) {  // lane l: column 32 w + l's word of the warp's rows
+            uint32_t x = bits;
+#pragma unroll
+            for (int sh = 16; sh > 0; sh >>= 1) {
+                const uint32_t m = sh == 16 ? 0xffffu : sh == 8 ? 0xff00ffu : sh == 4 ? 0x0f0f0f0fu : sh == 2 ? 0x33333333u : 0x55555555u;
+                const uint32_t y = __shfl_xor_sync(0xffffffffu, x, sh);
+                x = (lane & sh) ? ((y >> sh) & m) | (x & ~m) : (x & m) | ((y & m) << sh);
+            }
+            const int j = w * 32 + lane;
+            if (j < s.N) mask[(size_t)(i >> 5) * s.pitch + j] = x;
+            if (x) atomicAdd(&col_cnt[ww * 32 + lane], __popc(x));
+        }
+    }
+    if (mirror) {
+        __syncthreads();
+        const int j = j0 + threadIdx.x;
+        if (j < s.N) {
+            const int c = col_cnt[threadIdx.x];
+            if (c) atomicAdd(&out_count[j], c);
+            if (tile_cnt) tile_cnt[(size_t)bx * s.pitch + j] = c;
+        }
     }
     if (cnt) atomicAdd(&out_count[i], cnt);
     if (tile_cnt) tile_cnt[(size_t)by * s.pitch + i] = cnt;
@@ -672,9 +703,9 @@ __device__ __forceinline__ void fill_tile_euclid(const SpaceArgs& s, const float
 template <int KIND, int D>
 __device__ __forceinline__ void mask_tile(const SpaceArgs& s, const float* __restrict__ X,
                                           uint32_t* __restrict__ mask, int* __restrict__ out_count, int bx,
-                                          int by, int* __restrict__ tile_cnt = nullptr) {
+                                          int by, int* __restrict__ tile_cnt, bool half) {
     if constexpr (KIND == GMT_COST_EUCLID && D >= 2 && D <= 4) {
-        mask_tile_euclid4<D>(s, X, mask, out_count, bx, by, tile_cnt);
+        mask_tile_euclid4<D>(s, X, mask, out_count, bx, by, tile_cnt, half);
         return;
     }
     __shared__ float tile[D][kMaskWords * 32];

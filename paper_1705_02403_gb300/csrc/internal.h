@@ -194,6 +194,17 @@ __host__ __device__ inline bool cell_fill_fits(const CellGrid& cg, int N, int ma
     return (!cg.list_only && (N + 31) / 32 <= 1024) || max_deg <= 1024;
 }
 constexpr int kCellList = 1024;
+// Do the all-pairs tiles of 2 to 4 dimensions evaluate one side of the diagonal
+// only?  tiles: the launch's, both sides.  The mirrored words cost an
+// evaluated tile a third more, which shows while the tiles do not fill the chip
+// (8 resident on each of 152 SMs).  Pair stage on one GB300, half against both
+// sides: one 3D graph of 2049 nodes (81 tiles) 11.9 against 9.7 us, 8193 (1089)
+// 31 against 29, 10001 (1600) 31 against 39, 24001 103 against 162; one 2D
+// graph of 13001 35 against 46.  Batched calls: 32 queries of 1001 nodes (512)
+// 293 against 285, 100 of 1001 (1600) 436 against 438, 200 of 2049 (16200)
+// 1175 against 1260.
+constexpr long long kHalfMaskTiles = 1536;
+inline bool half_mask(long long tiles) { return tiles >= kHalfMaskTiles; }
 // Returns false when the cell list does not apply (not a 2D/3D geometric
 // graph); *pays is false when the 3^d cells around a node would hold more than
 // three tenths of the domain.  A caller that forces cells where they do not pay

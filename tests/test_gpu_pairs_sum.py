@@ -82,3 +82,31 @@ def test_cells_that_replace_all_pairs_keep_their_rows(d, n, batched):
         else:
             got = csr(Planner(problem(r)).build().view())
         same(got, csr(pairs(r)))
+
+
+@pytest.mark.parametrize("d", [2, 3])
+def test_mirrored_tiles_of_a_batch(d):
+    # enough tiles for one side of the diagonal, among them ragged small queries; each alone evaluates both sides
+    sizes = [1, 30, 31, 254, 255, 256, 510, 511, 512, 767, 768, 1023] + [1300] * 48
+    pbs = [envgen.geometric(500 + k, d=d, n=n, nbox=5, r=0.3, lam=0.5) for k, n in enumerate(sizes)]
+    bp = BatchPlanner(pbs)
+    for _ in range(2):
+        bp.plan()
+        for k in list(range(14)) + [len(sizes) - 1]:
+            v = bp.view(k)
+            got = tuple(v[f].cpu().numpy() for f in ("out_row", "out_col", "out_cost"))
+            same(got, csr(Planner(pbs[k]).build(debug_flags=N.GMT_DEBUG_PAIRS_ALL).view()))
+
+
+@pytest.mark.parametrize("d, n", [(2, 9984), (3, 10017), (4, 10239), (4, 10240)])
+def test_mirrored_tiles_of_one_graph(d, n):
+    r = {2: 0.05, 3: 0.1, 4: 0.2}[d]
+    pb = envgen.geometric(31, d=d, n=n, nbox=0 if d == 4 else 5, r=r, lam=0.5)
+    v = Planner(pb).build(debug_flags=N.GMT_DEBUG_PAIRS_ALL).view()
+    X, (row, col, _) = v.X.cpu().numpy(), csr(v)
+    rows = np.r_[0:300, 5000:5200, n - 300:n + 1]
+    for a in np.array_split(rows, 16):
+        i, j = (g.ravel() for g in np.meshgrid(a, np.arange(n + 1), indexing="ij"))
+        edge = (np.sqrt(sums(X, i, j)[0]) < F(r)) & (i != j)
+        want = j[edge]
+        assert np.array_equal(np.concatenate([col[row[u]:row[u + 1]] for u in a]), want)
