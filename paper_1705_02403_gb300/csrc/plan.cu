@@ -30,11 +30,13 @@ __device__ __forceinline__ void publish_ctl(const PlanArgs& A, int rank) {
     if (rank == 0) *(volatile int*)A.host_done = 1;
 }
 
-// Lanes per candidate pull (measured on one GB300): a single plan's team has
-// hundreds of warps for a frontier of a few hundred candidates, and 16-lane
-// pulls only lengthen each candidate's chain (DI n = 4096: 0.209 against
-// 0.132 ms); a batch's 4-CTA teams see more candidates per warp, and two
-// 16-lane pulls per warp take the 256-query plan stage from 2.41 to 2.26 ms.
+// Lanes per candidate pull.  A single plan's team has hundreds of warps for a
+// frontier of a few hundred candidates, and narrower pulls only lengthen each
+// candidate's chain (32, 16, 8 lanes, plan kernel on one GB300: 2D n = 1024
+// 105, 119, 140 us; 3D n = 16384 271, 290, 329; 6D n = 5000 266, 304, 382;
+// double integrator n = 4096 85, 114, 161; Dubins n = 5000 177, 178, 201).  A
+// batch's small teams may see many candidates per warp: half a warp each then
+// (kNarrowPulls), and always in the scratch kernel (256 queries 2.41 -> 2.26 ms).
 constexpr int kPlanPullLanes = 32;
 constexpr int kBatchPullLanes = 16;
 

@@ -56,6 +56,18 @@
 namespace gmtk {
 
 constexpr int kLocalMaxCluster = 16;
+// W < 32: candidates per warp of a CTA from which its pulls take W lanes each in
+// an iteration, else 32.  Many candidates: throughput, and two pulls per warp
+// hide each other's latency; few: a candidate's own chain, which a whole warp
+// shortens.  Plan stage on one GB300, always 16 lanes, always 32, by this line:
+// 256 uneven queries 1.452, 1.458, 1.440 ms; 200 3D queries of 2049 nodes
+// 0.664, 0.616, 0.622; 8 of 16385 0.718, 0.663, 0.669; 100 double-integrator
+// queries of 2049 0.379, 0.330, 0.330.  At 8 a warp: 1.439, 0.627, 0.669, 0.354.
+constexpr int kNarrowPulls = 16;
+template <int V>
+struct PullLanes {
+    static constexpr int value = V;
+};
 
 // Byte offsets of the state in dynamic shared memory (M own nodes, MW words
 // of own bits).  cache = true also keeps the own nodes' row bounds and states
@@ -226,7 +238,6 @@ __device__ __forceinline__ bool plan_body_local(const PlanArgs& A, const Team& t
     constexpr int D = KIND == GMT_COST_DI ? 6 : (KIND == GMT_COST_DUBINS ? 4 : DP);
     constexpr bool DIRECTED = KIND != GMT_COST_EUCLID;
     constexpr bool SINGLE = Team::kSingle;
-    using LG = LaneGroup<W>;
     const int N = A.N, n = SINGLE ? 1 : team.ctas(), me = SINGLE ? 0 : team.cta();
     const int tid = threadIdx.x, lane = tid & 31, wib = tid >> 5, wpc = blockDim.x >> 5;
     const int nbs = local_staged_boxes(A, DP);
@@ -478,12 +489,14 @@ __device__ __forceinline__ bool plan_body_local(const PlanArgs& A, const Team& t
         if (!SINGLE && stamp == 255)  // the next iteration's stamp is 1 again
             for (int w = tid; w < (int)(L.claim - L.sent) / 4; w += blockDim.x) reinterpret_cast<unsigned*>(sent)[w] = 0u;
         __syncthreads();
-        {
+        const int nc = lc.ccount[p];
+        auto pull = [&](auto lanes) {
+            constexpr int V = decltype(lanes)::value;
+            using LG = LaneGroup<V>;
             const int glane = LG::lane();
             const unsigned gmask = LG::mask();
-            const int nc = lc.ccount[p];
-            const int groups = wpc * (32 / W);
-            int t = tid / W;
+            const int groups = wpc * (32 / V);
+            int t = tid / V;
             while (t < nc) {
                 const int q = clist[t];
                 const int x = q * n + me;
@@ -502,14 +515,14 @@ __device__ __forceinline__ bool plan_body_local(const PlanArgs& A, const Team& t
                 }
                 float bc;
                 int by, be;
-                replica_parent_min<W>(A.in_col, A.in_cost, rep, r0, r1, glane, &bc, &by, &be);
+                replica_parent_min<V>(A.in_col, A.in_cost, rep, r0, r1, glane, &bc, &by, &be);
                 // the least (cost, node) over the lanes, by its two words; costs
                 // are >= 0, so their bits order as they do
                 const unsigned kc = __reduce_min_sync(gmask, float_key(bc));
                 const int ky = __reduce_min_sync(gmask, float_key(bc) == kc ? by : INT_MAX);
                 const unsigned holder = LG::ballot(float_key(bc) == kc && by == ky);
                 bc = __uint_as_float(kc);
-                be = __shfl_sync(gmask, be, __ffs(holder) - 1, W);
+                be = __shfl_sync(gmask, be, __ffs(holder) - 1, V);
                 by = ky;
                 if (be < 0) {
                     // the group node that pushed x is an open in-neighbour; the
@@ -517,7 +530,7 @@ __device__ __forceinline__ bool plan_body_local(const PlanArgs& A, const Team& t
                     if (glane == 0) { ++n_checks; ++n_failed; atomicCAS(&ctl->error, 0, (int)GMT_ERR_CUDA); }
                 } else {
                     bool computed;
-                    const bool free_edge = lazy_check<KIND, DP, W>(A, by, be, sx, B, basis, computed);
+                    const bool free_edge = lazy_check<KIND, DP, V>(A, by, be, sx, B, basis, computed);
                     if (glane == 0) {
                         n_pull += (unsigned long long)(r1 - r0);
                         ++n_checks;
@@ -537,9 +550,11 @@ __device__ __forceinline__ bool plan_body_local(const PlanArgs& A, const Team& t
                     }
                 }
                 if (glane == 0) t = groups + atomicAdd(&lc.ticket[p], 1);
-                t = __shfl_sync(gmask, t, 0, W);
+                t = __shfl_sync(gmask, t, 0, V);
             }
-        }
+        };
+        if (W < 32 && nc >= kNarrowPulls * wpc) pull(PullLanes<W>{});
+        else pull(PullLanes<32>{});
         __syncwarp();
         // the CTA's last warp sends its summary to every CTA
         {
