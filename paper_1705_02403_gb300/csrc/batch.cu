@@ -315,7 +315,7 @@ cudaError_t batch_cells_fill(int d, const QueryDev* Q, const long long* off_cell
     if (cells <= 0) return cudaSuccess;
     const size_t smem = cell_tile_smem(d, true, words, rank_words);
     auto launch = [&](auto kern) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const cudaError_t e = allow_full_smem((const void*)kern);
         if (e != cudaSuccess) return e;
         kern<<<(unsigned)cells, kCellWarps * 32, smem, st>>>(Q, off_cells, nq, words);
         return cudaGetLastError();

@@ -291,7 +291,7 @@ cudaError_t rows_t(const SpaceArgs& s, const float* X, const CellGrid& cg, const
     const int words = fill ? cell_fill_words(cg, s.N) : 0, rank = fill ? cell_rank_words(cg, s.N) : 0;
     const size_t smem = cell_tile_smem(D, fill, words, rank);
     auto launch = [&](auto kern) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const cudaError_t e = allow_full_smem((const void*)kern);
         if (e != cudaSuccess) return e;
         kern<<<cg.ncells, kCellWarps * 32, smem, st>>>(s, X, cg, start, sorted, out_count, max_deg, row, col, cost,
                                                        overflow, words, rank, cap);

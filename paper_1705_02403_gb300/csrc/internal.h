@@ -441,6 +441,12 @@ void record_error(const char* msg);
 cudaError_t launch_plan(const PlanArgs& a, int blocks, int threads, cudaStream_t st, int cluster = 0);
 int plan_max_coresident_blocks(int kind, int dp, int threads);
 int plan_max_cluster(int kind, int dp, int threads);
+// Gives a kernel all the dynamic shared memory a CTA can have (the device's
+// limit less the kernel's own static part), once per kernel and device.  The
+// limit belongs to the kernel, not to a launch: set to each launch's own size,
+// another host thread's smaller one could come between and have the launch
+// refused.  Launches and occupancy queries name their size themselves.
+cudaError_t allow_full_smem(const void* kernel);
 // Loads the kernels a 2D or 3D plan on a cluster (or, <= 1, one CTA) launches.
 cudaError_t load_plan_kernel(int kind, int dp, int cluster);
 // Persistent batched wavefront (one barrier per iteration) over the `nq`

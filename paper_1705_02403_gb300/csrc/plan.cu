@@ -10,6 +10,7 @@
 // boundaries; other graphs and cooperative grids keep it in global memory
 // (plan_body_fused, plan_fused.cuh).  Both take the same decisions.
 #include <algorithm>
+#include <mutex>
 
 #include "plan_core.cuh"
 #include "plan_fused.cuh"
@@ -140,6 +141,28 @@ __global__ void __launch_bounds__(1024, 1) plan_batch_local_kernel(const PlanArg
 }
 
 // ----------------------------------------------------------------- launcher
+cudaError_t allow_full_smem(const void* kernel) {
+    static std::mutex mu;
+    static struct { int dev; const void* kernel; } done[256];
+    static int n = 0;
+    int dev = 0, optin = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    std::lock_guard<std::mutex> lock(mu);  // held until it is set: nobody launches before
+    for (int k = 0; k < n; ++k)
+        if (done[k].dev == dev && done[k].kernel == kernel) return cudaSuccess;
+    cudaFuncAttributes a;
+    e = cudaFuncGetAttributes(&a, kernel);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)a.sharedSizeBytes);
+    if (e == cudaSuccess && n < 256) {  // past the table: set again at each call, to the same value
+        done[n].dev = dev;
+        done[n++].kernel = kernel;
+    }
+    return e;
+}
+
 namespace {
 // Dynamic shared memory a CTA of the local kernels can have.
 size_t plan_local_room() {
@@ -166,7 +189,7 @@ bool plan_local_fits(int N, int n, int D, bool directed, size_t box_bytes, int t
 template <class Kern, class Team>
 cudaError_t launch_local(Kern kern, const PlanArgs& a, const Team& team, bool cache, int n, int threads, size_t smem,
                          cudaStream_t st) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_full_smem((const void*)kern);
     if (e == cudaSuccess && n > 8) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
@@ -324,8 +347,8 @@ struct BatchLaunch {
     }
 };
 template <class Kern>
-cudaError_t batch_attributes(Kern kern, int cluster, size_t smem) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+cudaError_t batch_attributes(Kern kern, int cluster) {
+    cudaError_t e = allow_full_smem((const void*)kern);
     if (e == cudaSuccess && cluster > 8)
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     return e;
@@ -351,11 +374,11 @@ cudaError_t plan_batch_t(const PlanArgs* queries, const int* order, int nq, int*
     return with_batch_kernel<ALL_KINDS>(
         cluster, local,
         [&](auto kern, auto team) {
-            cudaError_t e = batch_attributes(kern, cluster, smem);
+            cudaError_t e = batch_attributes(kern, cluster);
             return e != cudaSuccess ? e : cudaLaunchKernelEx(&L.cfg, kern, queries, order, nq, next, slot, team);
         },
         [&](auto kern, auto team) {
-            cudaError_t e = batch_attributes(kern, cluster, smem);
+            cudaError_t e = batch_attributes(kern, cluster);
             return e != cudaSuccess ? e
                                     : cudaLaunchKernelEx(&L.cfg, kern, queries, order, nq, next, slot, scratch, team);
         });
@@ -367,7 +390,7 @@ int batch_teams_t(int threads, int cluster, size_t smem, bool local) {
     BatchLaunch L(1, cluster, threads, smem, nullptr);
     auto count = [&](auto kern, auto) {
         int n = 0;
-        if (batch_attributes(kern, cluster, smem) != cudaSuccess ||
+        if (batch_attributes(kern, cluster) != cudaSuccess ||
             cudaOccupancyMaxActiveClusters(&n, kern, &L.cfg) != cudaSuccess) {
             cudaGetLastError();
             return 0;
