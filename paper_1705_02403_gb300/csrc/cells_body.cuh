@@ -426,7 +426,15 @@ __device__ __forceinline__ void cell_tile(const SpaceArgs& s, const float* __res
         if (!FILL) {
             if (has && cnt) atomicAdd(&counts[lane], cnt);
             __syncthreads();
-            if (warp == 0 && has) out_count[v] = counts[lane] - 1;  // without the node itself
+            if (warp == 0 && has) {
+                // without the node itself, which passes the test only if its
+                // coordinates are finite (a bad start or appended sample, which
+                // the build reports, may not be: a count is never negative)
+                float x[D];
+#pragma unroll
+                for (int a = 0; a < D; ++a) x[a] = X[(size_t)a * s.pitch + v];
+                out_count[v] = counts[lane] - (sq_dist_pairs<D>(x, x) < thr ? 1 : 0);
+            }
             __syncthreads();
             continue;
         }
