@@ -206,9 +206,10 @@ gmt_status gmt_build_graph_ex(const gmt_space* space, const gmt_boxes* boxes, co
  * by the next gmt_plan (or gmt_graph_get_view) on this handle, which returns
  * the errors gmt_build_graph would have returned.  If the edges do not fit
  * those arrays, that call rebuilds synchronously and the result is the same.
- * A new handle, a cell-list neighbour build of more than 32768 nodes or
- * appended samples take the synchronous path.  `boxes` (the struct's DEVICE arrays) must stay valid
- * until that plan or view. */
+ * A new handle, appended samples or a cell-list neighbour build (from 12000
+ * nodes in 2D and 32768 in 3D, where the cells around a node hold at most a
+ * quarter of the domain) take the synchronous path.  `boxes` (the struct's
+ * DEVICE arrays) must stay valid until that plan or view. */
 gmt_status gmt_build_graph_async(const gmt_space* space, const gmt_boxes* boxes, const float* x_init,
                                  const gmt_goal* goal, const gmt_params* params, gmt_graph** graph,
                                  gmt_stream stream);

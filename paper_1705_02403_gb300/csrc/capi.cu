@@ -513,8 +513,10 @@ gmt_status build_impl(const gmt_space* space, const gmt_boxes* boxes, const floa
     LAUNCH(g->mark(gmt_graph::kScan, 1, st), "event");
     g->pending = false;
     const long long cap_now = edge_capacity(g);
-    // (a cell-list graph whose longest row decides whether it fits needs the host)
-    if (async && (!cells || cell_fill_fits(cg, g->N, INT_MAX)) && extra_count == 0 && cap_now > 0) {
+    // (cell lists that replace the all-pairs test are queued as that test is;
+    // larger ones wait, and report a bad start themselves, as documented)
+    const bool queued = !cells || (cg.pairs_sum && cell_fill_fits(cg, g->N, INT_MAX));
+    if (async && queued && extra_count == 0 && cap_now > 0) {
         // no host wait: fill into the arrays of earlier builds; the next plan
         // (or view) confirms the edge count and rebuilds if it did not fit
         const bool di_a = g->kind == GMT_COST_DI, dub_a = g->kind == GMT_COST_DUBINS;
