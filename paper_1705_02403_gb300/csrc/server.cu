@@ -209,9 +209,9 @@ gmt_status sfail(gmt_status s, const std::string& m) {
 }
 
 // Lays out a request's boxes and the regions of those that moved (their old
-// and new places) in the slot's staging, and makes them the session's.
-// Returns the moved boxes.  Worker thread, server lock held.
-int stage_request(Slot& sl, Session& ss, Request&& rq) {
+// and new places) in the slot's staging.  Returns the moved boxes.  Worker
+// thread, server lock held.
+int stage_request(Slot& sl, const Session& ss, Request&& rq) {
     const int P = ss.dp, nb = ss.nbox;
     sl.req = std::move(rq);
     sl.t_start = Clock::now();
@@ -232,8 +232,6 @@ int stage_request(Slot& sl, Session& ss, Request&& rq) {
         o += 4 * P;
         ++nm;
     }
-    ss.cur_lo = sl.req.lo;
-    ss.cur_hi = sl.req.hi;
     return nm;
 }
 
@@ -354,8 +352,17 @@ void worker_loop(gmt_server* sv) {
             const int nm = stage_request(sl, ss, std::move(rq));
             lk.unlock();
             const cudaError_t e = start_request(sv, sl, ss, nm);
-            lk.lock();
             if (e != cudaSuccess) {
+                // what was queued before the refused launch reads the staging
+                // and writes the session's verdicts: over before either is free
+                cudaStreamSynchronize(sl.stream);
+                cudaGetLastError();
+            }
+            lk.lock();
+            if (e == cudaSuccess) {
+                ss.cur_lo = sl.req.lo;
+                ss.cur_hi = sl.req.hi;
+            } else {  // the verdicts stay those of the boxes before, less the ones already cleared
                 sv->worker_error = std::string("request launch: ") + cudaGetErrorString(e);
                 gmt_server_result r;
                 std::memset(&r, 0, sizeof(r));
