@@ -86,7 +86,7 @@ struct gmt_graph {
     float rho = 0.0f;   // Dubins airplane turning radius the costs were built with
     float pos_lo[3] = {0, 0, 0}, pos_hi[3] = {0, 0, 0};
     int plan_blocks = 0, plan_threads = 0, plan_cluster = 0;   // 0 = automatic
-    int auto_cluster = -1;                                     // probed once
+    int auto_cluster[2] = {-1, -1};                            // CTAs of 512 and of 1024 threads: probed once each
     float* X = nullptr;            size_t cap_X = 0;
     uint8_t* is_goal = nullptr;    size_t cap_is_goal = 0;
     int* out_row = nullptr;        size_t cap_out_row = 0;
@@ -687,9 +687,11 @@ gmt_status gmt_plan(gmt_graph* g, const gmt_boxes* boxes, const gmt_params* para
         // where idle warps cost more than they carry: 2D n = 1024 0.107 ms
         // against 0.116 with 1024 threads and 0.142 on one CTA, equal at 4096),
         // else a cooperative grid of one CTA per SM
-        if (g->auto_cluster < 0) g->auto_cluster = plan_max_cluster(g->kind, g->dp, N <= 2048 ? 512 : 1024);
-        cluster = g->auto_cluster;
-        if (threads <= 0) threads = N <= 2048 ? 512 : 1024;
+        const int t = N <= 2048 ? 512 : 1024;
+        int& fits = g->auto_cluster[t > 512];
+        if (fits < 0) fits = plan_max_cluster(g->kind, g->dp, t);
+        cluster = fits;
+        if (threads <= 0) threads = t;
         if (cluster <= 1) blocks = -1;
     }
     if (threads <= 0) threads = 512;

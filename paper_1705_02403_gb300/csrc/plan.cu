@@ -302,18 +302,21 @@ cudaError_t load_plan_kernel(int kind, int dp, int cluster) {
 }
 
 // Largest cluster size (16, 8, 4, 2) for which one cluster of `threads`-thread
-// CTAs of the plan kernel can be resident; 0 if none.
+// CTAs can be resident with all the shared memory a plan may ask for; 0 if
+// none.  (The kernel that keeps its state in global memory needs less.)
 int plan_max_cluster(int kind, int dp, int threads) {
-    auto kern = kind == GMT_COST_DI       ? plan_kernel<ClusterTeam, GMT_COST_DI, 3>
-                : kind == GMT_COST_DUBINS ? plan_kernel<ClusterTeam, GMT_COST_DUBINS, 3>
-                : dp == 2                 ? plan_kernel<ClusterTeam, GMT_COST_EUCLID, 2>
-                                          : plan_kernel<ClusterTeam, GMT_COST_EUCLID, 3>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return 0;
+    auto kern = kind == GMT_COST_DI       ? plan_local_kernel<ClusterTeam, GMT_COST_DI, 3>
+                : kind == GMT_COST_DUBINS ? plan_local_kernel<ClusterTeam, GMT_COST_DUBINS, 3>
+                : dp == 2                 ? plan_local_kernel<ClusterTeam, GMT_COST_EUCLID, 2>
+                                          : plan_local_kernel<ClusterTeam, GMT_COST_EUCLID, 3>;
+    if (allow_full_smem((const void*)kern) != cudaSuccess ||
+        cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
+        return 0;
     for (int c = 16; c >= 2; c /= 2) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(c);
         cfg.blockDim = dim3(threads);
-        cfg.dynamicSmemBytes = plan_smem_bytes(smem_box_cap(3), 3, 12 * 1024);
+        cfg.dynamicSmemBytes = plan_local_room();
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeClusterDimension;
         attr[0].val.clusterDim.x = c;
