@@ -252,7 +252,8 @@ gmt_status gmt_plan(gmt_graph* graph, const gmt_boxes* boxes, const gmt_params* 
  * (blocks ignored); otherwise blocks == 1: one CTA with block barriers;
  * blocks > 1: a cooperative grid of that many CTAs (clamped to what can be
  * co-resident) with bounded software barriers; blocks == cluster == 0:
- * automatic (the largest cluster the GPU can hold, up to 16 CTAs).  threads:
+ * automatic (one CTA for small 2D graphs in narrow cost groups, else the
+ * largest cluster the GPU can hold, up to 16 CTAs).  threads:
  * CTA size, a multiple of 32 in [64, 1024], or 0 = automatic. */
 gmt_status gmt_graph_set_launch(gmt_graph* graph, int32_t blocks, int32_t threads, int32_t cluster);
 

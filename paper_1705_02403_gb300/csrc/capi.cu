@@ -681,9 +681,13 @@ gmt_status gmt_plan(gmt_graph* g, const gmt_boxes* boxes, const gmt_params* para
     }
 
     int blocks = g->plan_blocks, threads = g->plan_threads, cluster = g->plan_cluster;
+    if (blocks <= 0 && cluster <= 0 && threads <= 0 && plan_one_cta(g->kind, g->dp, N, params->lambda)) {
+        blocks = 1;
+        threads = 1024;
+    }
     if (blocks <= 0 && cluster <= 0) {
         // automatic: the largest resident thread-block cluster (measured
-        // fastest on GB300 at every size; CTAs of 512 threads up to 2048 nodes,
+        // fastest on GB300 at every other size; CTAs of 512 threads up to 2048 nodes,
         // where idle warps cost more than they carry: 2D n = 1024 0.107 ms
         // against 0.116 with 1024 threads and 0.142 on one CTA, equal at 4096),
         // else a cooperative grid of one CTA per SM

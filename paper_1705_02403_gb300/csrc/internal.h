@@ -447,6 +447,17 @@ int plan_max_cluster(int kind, int dp, int threads);
 // another host thread's smaller one could come between and have the launch
 // refused.  Launches and occupancy queries name their size themselves.
 cudaError_t allow_full_smem(const void* kernel);
+// Does the automatic shape run a plan on one CTA of 1024 threads rather than on
+// a cluster?  Small 2D graphs in narrow cost groups do: an iteration then has
+// too few nodes for the cluster's barriers to pay.  The nodes an iteration may
+// take go with lambda N.  Whole plan on one GB300, one CTA against 16 of 512
+// threads, us: n = 200, lambda 0.2 (40) 108 and 125, 0.5 (100) 70 and 72, 1 (200)
+// 58 and 55; 900, 0.05 (45) 522 and 662, 0.2 (180) 201 and 211, 0.5 (450) 146 and
+// 108; 2048, 0.1 (205) 536 and 569, 0.2 (410) 371 and 307; lambda = 0: n = 200
+// 466 and 640, 2048 5200 and 6587.
+inline bool plan_one_cta(int kind, int dp, int N, float lambda) {
+    return kind == GMT_COST_EUCLID && dp == 2 && N <= 2049 && lambda <= 0.5f && lambda * (float)N <= 210.0f;
+}
 // Loads the kernels a 2D or 3D plan on a cluster (or, <= 1, one CTA) launches.
 cudaError_t load_plan_kernel(int kind, int dp, int cluster);
 // Persistent batched wavefront (one barrier per iteration) over the `nq`

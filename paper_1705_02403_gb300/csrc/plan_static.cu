@@ -16,8 +16,9 @@
 //    (cudaGetSymbolAddress, with that device current) and caches it, together
 //    with the largest resident cluster of the plan kernel; make that first
 //    call before any stream capture begins.
-//  - Launch: the same automatic shape as gmt_plan (the largest resident
-//    thread-block cluster, else a cooperative grid).  Obstacles are scanned linearly by
+//  - Launch: the same automatic shape as gmt_plan (one CTA for small 2D graphs
+//    in narrow groups, else the largest resident thread-block cluster, else a
+//    cooperative grid).  Obstacles are scanned linearly by
 //    every check: the box grid that gmt_plan builds for 128 or more boxes needs
 //    allocated scratch, so many boxes cost more here than in gmt_plan.
 //  - Sharing: every call on a device uses the same array and the array keeps
@@ -163,10 +164,12 @@ extern "C" gmt_status gmt_plan_static(const gmt_space* space, const gmt_graph_vi
 
     // launch shape: as gmt_plan chooses it automatically
     int blocks = 0, cluster = 0, threads = 0;
-    threads = g->N <= 2048 ? 512 : 1024;
-    s = max_cluster(g->kind, g->pos_dim, threads, &cluster);
+    const bool one = plan_one_cta(g->kind, g->pos_dim, g->N, params->lambda);
+    if (one) blocks = 1;
+    threads = one || g->N > 2048 ? 1024 : 512;
+    if (!one) s = max_cluster(g->kind, g->pos_dim, threads, &cluster);
     if (s != GMT_OK) return s;
-    if (cluster <= 1) {
+    if (!one && cluster <= 1) {
         cluster = 0;
         int dev = 0, sms = 0;
         cudaError_t e = cudaGetDevice(&dev);
