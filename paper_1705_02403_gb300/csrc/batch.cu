@@ -586,13 +586,17 @@ int batch_max_teams(const gmt_batch* b, int cluster, int threads) {
 
 // The untuned shape.  Pairs of CTAs with 1024 threads when there are more
 // queries than larger teams, else the largest team that leaves every query one
-// of its own; 256 threads for queries of at most 1025 nodes, whose iterations
-// hold too little work for more warps; more CTAs where the largest query's
+// of its own; fewer threads for queries of at most 1025 nodes, whose iterations
+// hold too little work for more warps to pay when teams take turns on an SM (256)
+// or have many CTAs (512 on four, 256 on more); more CTAs where the largest query's
 // state needs them, and teams of 4 x 512 when it fits none (the scratch kernel's
 // best).  Plan stage on one GB300, 256 uneven queries up to 16385 nodes: 2 x
 // 1024 1.44 ms, 4 x 1024 1.93, 8 x 512 2.02, 2 x 512 2.45; 200 of 2049: 0.666,
 // 0.944, 0.981, 0.731; 32 of 4097: 4 x 1024 0.268, 8 x 512 0.282, 2 x 1024
-// 0.395; 200 of 513: 2 x 256 0.203, 2 x 1024 0.281.
+// 0.395; 200 of 513: 2 x 256 0.203, 2 x 1024 0.281.  With a team each (2 x 256, 2 x
+// 1024): 40 Dubins queries of 1001 0.487, 0.178, 3D 0.238, 0.119; 70 of 301 0.184,
+// 0.137, 3D 0.102, 0.072; of 151 equal; 60 of 61 0.070, 0.076.  38 Dubins queries of
+// 1001, 4 x 256, 512, 1024: 0.301, 0.182, 0.228.
 void untuned_shape(const gmt_batch* b, int* cluster, int* threads) {
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
@@ -605,7 +609,8 @@ void untuned_shape(const gmt_batch* b, int* cluster, int* threads) {
         if (local) break;
     }
     *cluster = local ? c : 4;
-    *threads = !local ? 512 : b->max_n <= 1025 ? 256 : 1024;
+    const bool own = (long long)c * b->q <= sms && c <= 4;  // a team, and SMs, for every query
+    *threads = !local ? 512 : b->max_n > 1025 ? 1024 : b->max_n <= 129 || !own ? 256 : c == 2 ? 1024 : 512;
 }
 
 // Plan-stage launch shape of the teams scheme: (cluster, threads, teams).
