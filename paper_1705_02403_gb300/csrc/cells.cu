@@ -89,39 +89,92 @@ __global__ void __launch_bounds__(256) box_grid_scatter_kernel(BoxArgs boxes, in
         }
 }
 
+// Shapes a grid of uneven boxes is chosen among: 2^x by 2^y cells.
+constexpr int kShapeFine = 11;  // cells per axis are at most 2^kShapeFine
+__constant__ uchar2 kBoxGridShapes[32] = {
+    {10, 4}, {9, 5}, {8, 6}, {7, 7}, {6, 8}, {5, 9}, {4, 10}, {3, 11}, {9, 3}, {8, 4}, {7, 5},
+    {6, 6},  {5, 7}, {4, 8}, {3, 9}, {8, 2}, {7, 3}, {6, 4},  {5, 5},  {4, 6}, {3, 7}, {2, 8},
+    {6, 2},  {5, 3}, {4, 4}, {3, 5}, {2, 6}, {4, 2}, {3, 3},  {2, 4},  {3, 1}, {2, 2}};
+
+// The shape with the fewest boxes to test at a point: the mean list over the
+// cells, and every box over more than kBoxGridMaxCells cells; an entry to write
+// weighs as 0.15 tests.  From at most 1024 boxes, one of every `step` by a hash
+// (obstacles may alternate).  One block of 1024 threads; cost[32] and g[2] in
+// shared memory, g the exponents of the result once the block has passed its
+// next barrier.
+__device__ __forceinline__ void box_grid_choose(const BoxArgs& boxes, int dp, const BoxGridArgs& grid,
+                                                unsigned* cost, int* g) {
+    const int tid = threadIdx.x, lane = tid & 31;
+    if (tid < 32) cost[tid] = 0u;
+    const int step = (boxes.count + 1023) / 1024, of = (boxes.count + step - 1) / step;
+    const int s = tid * step + (int)(((unsigned)tid * 2654435761u >> 16) % (unsigned)step);
+    int c0[2] = {1, 1}, c1[2] = {0, 0};
+    if (s < boxes.count) {
+        const int fine[2] = {1 << kShapeFine, 1 << kShapeFine};
+        const float inv[2] = {(float)fine[0] / grid.span[0], (float)fine[1] / grid.span[1]};
+        box_grid_range(grid, fine, inv, boxes.lo + (size_t)s * dp, boxes.hi + (size_t)s * dp, c0, c1);
+    }
+    const bool ok = c0[0] <= c1[0] && c0[1] <= c1[1];  // else it holds no point
+    __syncthreads();
+    for (int k = 0; k < 32; ++k) {
+        const int sx = kShapeFine - kBoxGridShapes[k].x, sy = kShapeFine - kBoxGridShapes[k].y;
+        const int n = ((c1[0] >> sx) - (c0[0] >> sx) + 1) * ((c1[1] >> sy) - (c0[1] >> sy) + 1);
+        // entries in the low half (at most 1024 x 32), big boxes in the high
+        const unsigned v = __reduce_add_sync(0xffffffffu, !ok ? 0u : n > kBoxGridMaxCells ? 1u << 16 : (unsigned)n);
+        if (lane == 0 && v) atomicAdd(&cost[k], v);
+    }
+    __syncthreads();
+    if (tid < 32) {
+        const float n = (float)(cost[lane] & 0xffffu), scale = (float)boxes.count / (float)of;
+        const float cells = (float)(1 << (kBoxGridShapes[lane].x + kBoxGridShapes[lane].y));
+        const float tests = scale * (n / cells + (float)(cost[lane] >> 16)) + 0.15f * n / (float)of;
+        const unsigned best = __reduce_min_sync(0xffffffffu, (__float_as_uint(tests) & ~31u) | (unsigned)lane);
+        if (lane == (int)(best & 31u)) {
+            g[0] = 1 << kBoxGridShapes[lane].x;
+            g[1] = 1 << kBoxGridShapes[lane].y;
+        }
+    }
+}
+
 // The whole grid by one block, its cell counts in shared memory: a plan with
 // many boxes builds it before the wavefront (and a build before sampling), so
 // three dependent launches and a memset cost more than the work (1500 boxes:
 // 18.5 us of kernels in a row before).  The block also chooses the grid's
-// shape, from the boxes' mean extents: cells of the boxes' own proportions,
-// down to about half a box on each axis (a box then lies in about nine).
-// Obstacles cut into thin slices get thin cells: 1500 strips a hundred times
-// wider than high list 2.9 boxes an occupied cell (9 at most) on 16 x 1024
-// cells, 25 (59 at most) on 64 x 64.  This kernel takes 18 us for them; the
-// Dubins plan kernel at n = 5000 went from 0.251 to 0.163 ms, its Halton
-// sampler from 43 to 21 us.
+// shape: cells of the mean box's proportions, down to about a quarter of its
+// area (a box then lies in about nine).  Obstacles cut into thin slices get thin
+// cells: 1500 strips a hundred times wider than high list 2.9 boxes an occupied
+// cell (9 at most) on 16 x 1024 cells, 25 (59 at most) on 64 x 64; the Dubins plan
+// kernel at n = 5000 went from 0.251 to 0.163 ms, its Halton sampler from 43 to 21
+// us.  The area is the boxes' mean, not the product of their mean extents, which
+// slices along both axes make far larger.  Where the shape leaves more than
+// kBoxGridFewBig boxes over too many cells to be listed, every point would test
+// them all, and box_grid_choose picks another: 1500 squares, a tenth of them four
+// times wider, 2D n = 1000, a build and plan 1351 -> 258 us (400 on square cells).
+constexpr int kBoxGridFewBig = 4;
 __global__ void __launch_bounds__(1024) box_grid_block_kernel(BoxArgs boxes, int dp, BoxGridArgs grid,
                                                               int* __restrict__ start, int* __restrict__ list,
                                                               float4* __restrict__ packed, int* __restrict__ big,
                                                               int* __restrict__ nbig, float4* __restrict__ shape) {
     extern __shared__ int cnt[];  // kBoxGridCells
     __shared__ int warp_sum[32];
-    __shared__ float ext[3][32];
+    __shared__ float ext[4][32];
+    __shared__ unsigned cost[32];
     __shared__ int s_big, s_g[2];
-    __shared__ float s_inv[2];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    // mean extents of the boxes that hold points
-    float w[3] = {0.0f, 0.0f, 0.0f};
+    // mean extents and area of the boxes that hold points
+    float w[4] = {0.0f, 0.0f, 0.0f, 0.0f};
     for (int b = tid; b < boxes.count; b += 1024) {
         const float dx = boxes.hi[(size_t)b * dp] - boxes.lo[(size_t)b * dp];
         const float dy = boxes.hi[(size_t)b * dp + 1] - boxes.lo[(size_t)b * dp + 1];
         if (!(dx >= 0.0f) || !(dy >= 0.0f)) continue;
-        w[0] += fminf(dx, grid.span[0]);
-        w[1] += fminf(dy, grid.span[1]);
+        const float mx = fminf(dx, grid.span[0]), my = fminf(dy, grid.span[1]);
+        w[0] += mx;
+        w[1] += my;
         w[2] += 1.0f;
+        w[3] += mx * my;
     }
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
+    for (int k = 0; k < 4; ++k) {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) w[k] += __shfl_xor_sync(0xffffffffu, w[k], o);
         if (lane == 0) ext[k][warp] = w[k];
@@ -129,7 +182,7 @@ __global__ void __launch_bounds__(1024) box_grid_block_kernel(BoxArgs boxes, int
     __syncthreads();
     if (warp == 0) {
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
+        for (int k = 0; k < 4; ++k) {
             w[k] = ext[k][lane];
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) w[k] += __shfl_xor_sync(0xffffffffu, w[k], o);
@@ -137,34 +190,44 @@ __global__ void __launch_bounds__(1024) box_grid_block_kernel(BoxArgs boxes, int
         if (lane == 0) {
             const float n = fmaxf(w[2], 1.0f);
             const float fx = fmaxf(w[0] / (n * grid.span[0]), 1e-4f), fy = fmaxf(w[1] / (n * grid.span[1]), 1e-4f);
+            const float area = fmaxf(w[3] / (n * grid.span[0] * grid.span[1]), 1e-8f);
             int P = 1;
-            while (P < kBoxGridCells && 2.0f * (float)P * fx * fy <= 4.0f) P *= 2;
+            while (P < kBoxGridCells && 2.0f * (float)P * area <= 4.0f) P *= 2;
             int gy = 1;
             while (gy < P && fx * (float)(P / gy) > 2.0f * fy * (float)gy) gy *= 2;
             s_g[0] = P / gy;
             s_g[1] = gy;
-#pragma unroll
-            for (int a = 0; a < 2; ++a) s_inv[a] = (float)s_g[a] / grid.span[a];
-            *shape = make_float4(__int_as_float(s_g[0]), __int_as_float(s_g[1]), s_inv[0], s_inv[1]);
             s_big = 0;
         }
     }
-    for (int c = tid; c < kBoxGridCells; c += 1024) cnt[c] = 0;
-    __syncthreads();
-    const int g[2] = {s_g[0], s_g[1]}, cells = g[0] * g[1];
-    const float inv[2] = {s_inv[0], s_inv[1]};
-    for (int b = tid; b < boxes.count; b += 1024) {
-        int c0[2], c1[2];
-        box_grid_range(grid, g, inv, boxes.lo + (size_t)b * dp, boxes.hi + (size_t)b * dp, c0, c1);
-        if (c0[0] > c1[0] || c0[1] > c1[1]) continue;  // lo > hi: the box holds no point
-        if ((c1[0] - c0[0] + 1) * (c1[1] - c0[1] + 1) > kBoxGridMaxCells) {
-            big[atomicAdd(&s_big, 1)] = b;
-            continue;
+    int g[2], cells;
+    float inv[2];
+    for (int attempt = 0;; ++attempt) {
+        for (int c = tid; c < kBoxGridCells; c += 1024) cnt[c] = 0;
+        __syncthreads();
+#pragma unroll
+        for (int a = 0; a < 2; ++a) {
+            g[a] = s_g[a];
+            inv[a] = (float)g[a] / grid.span[a];
         }
-        for (int cy = c0[1]; cy <= c1[1]; ++cy)
-            for (int cx = c0[0]; cx <= c1[0]; ++cx) atomicAdd(&cnt[cy * g[0] + cx], 1);
+        cells = g[0] * g[1];
+        for (int b = tid; b < boxes.count; b += 1024) {
+            int c0[2], c1[2];
+            box_grid_range(grid, g, inv, boxes.lo + (size_t)b * dp, boxes.hi + (size_t)b * dp, c0, c1);
+            if (c0[0] > c1[0] || c0[1] > c1[1]) continue;  // lo > hi: the box holds no point
+            if ((c1[0] - c0[0] + 1) * (c1[1] - c0[1] + 1) > kBoxGridMaxCells) {
+                big[atomicAdd(&s_big, 1)] = b;
+                continue;
+            }
+            for (int cy = c0[1]; cy <= c1[1]; ++cy)
+                for (int cx = c0[0]; cx <= c1[0]; ++cx) atomicAdd(&cnt[cy * g[0] + cx], 1);
+        }
+        __syncthreads();
+        if (attempt || s_big <= kBoxGridFewBig) break;  // uniform: nothing writes s_big before the next barrier
+        box_grid_choose(boxes, dp, grid, cost, s_g);
+        if (tid == 0) s_big = 0;  // read by all before the barriers of the choice
     }
-    __syncthreads();
+    if (tid == 0) *shape = make_float4(__int_as_float(g[0]), __int_as_float(g[1]), inv[0], inv[1]);
     // exclusive prefix of the counts: a warp's run of cells, 32 at a time (a
     // run per thread would meet 16-way bank conflicts)
     constexpr int kPer = kBoxGridCells / 1024;
