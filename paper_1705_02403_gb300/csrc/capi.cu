@@ -267,10 +267,10 @@ cudaError_t build_box_grid(gmt_graph* g, const BoxArgs& boxes, BoxGridArgs* gr, 
     std::memset(gr, 0, sizeof(*gr));
     if (g->dp < 2 || boxes.count < kBoxGridMinBoxes) return cudaSuccess;
     const int G = box_grid_cells(boxes.count);
-    const size_t B = (size_t)boxes.count, cells = (size_t)G * G;
+    const size_t B = (size_t)boxes.count, cells = std::max((size_t)G * G, (size_t)kBoxGridCells);
     cudaError_t e;
     if ((e = grow(&g->grid_cnt, &g->cap_grid_cnt, cells + 1)) != cudaSuccess) return e;  // + the big-box count
-    if ((e = grow(&g->grid_start, &g->cap_grid_start, std::max(cells, (size_t)kBoxGridCells) + 1)) != cudaSuccess) return e;
+    if ((e = grow(&g->grid_start, &g->cap_grid_start, cells + 1)) != cudaSuccess) return e;
     if ((e = grow(&g->grid_shape, &g->cap_grid_shape, 1)) != cudaSuccess) return e;
     if ((e = grow(&g->grid_list, &g->cap_grid_list, B * kBoxGridMaxCells)) != cudaSuccess) return e;
     if ((e = grow(&g->grid_big, &g->cap_grid_big, B)) != cudaSuccess) return e;

@@ -70,23 +70,29 @@ __device__ __forceinline__ void box_grid_put(const BoxArgs& boxes, int dp, int b
     else pack_box<3>(packed, boxes.lo, boxes.hi, b, t);
 }
 
-// One thread per box: writes it into each of its cells' lists (cnt counts
-// back down to 0).
+// One warp per box, a lane per cell of its range: writes it into its cells'
+// lists (cnt counts back down to 0).
 __global__ void __launch_bounds__(256) box_grid_scatter_kernel(BoxArgs boxes, int dp, BoxGridArgs grid,
                                                                const int* __restrict__ start, int* __restrict__ cnt,
                                                                int* __restrict__ list, float4* __restrict__ packed) {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
+    const int b = (int)((blockIdx.x * (unsigned)blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
     if (b >= boxes.count) return;
-    const int g[2] = {grid.g, grid.g};
+    int g[2] = {grid.g, grid.g};
+    float inv[2] = {grid.inv_h[0], grid.inv_h[1]};
+    if (grid.shape) {
+        const float4 s = __ldg(grid.shape);
+        g[0] = __float_as_int(s.x);
+        g[1] = __float_as_int(s.y);
+        inv[0] = s.z;
+        inv[1] = s.w;
+    }
     int c0[2], c1[2];
-    box_grid_range(grid, g, grid.inv_h, boxes.lo + (size_t)b * dp, boxes.hi + (size_t)b * dp, c0, c1);
+    box_grid_range(grid, g, inv, boxes.lo + (size_t)b * dp, boxes.hi + (size_t)b * dp, c0, c1);
     if (c0[0] > c1[0] || c0[1] > c1[1]) return;
-    if ((c1[0] - c0[0] + 1) * (c1[1] - c0[1] + 1) > kBoxGridMaxCells) return;
-    for (int cy = c0[1]; cy <= c1[1]; ++cy)
-        for (int cx = c0[0]; cx <= c1[0]; ++cx) {
-            const int c = cy * grid.g + cx;
-            box_grid_put(boxes, dp, b, start[c] + atomicSub(&cnt[c], 1) - 1, list, packed);
-        }
+    const int nx = c1[0] - c0[0] + 1, n = nx * (c1[1] - c0[1] + 1);
+    if (n > kBoxGridMaxCells || lane >= n) return;
+    const int c = (c0[1] + lane / nx) * g[0] + c0[0] + lane % nx;
+    box_grid_put(boxes, dp, b, start[c] + atomicSub(&cnt[c], 1) - 1, list, packed);
 }
 
 // Shapes a grid of uneven boxes is chosen among: 2^x by 2^y cells.
@@ -136,10 +142,11 @@ __device__ __forceinline__ void box_grid_choose(const BoxArgs& boxes, int dp, co
     }
 }
 
-// The whole grid by one block, its cell counts in shared memory: a plan with
-// many boxes builds it before the wavefront (and a build before sampling), so
-// three dependent launches and a memset cost more than the work (1500 boxes:
-// 18.5 us of kernels in a row before).  The block also chooses the grid's
+// The counts, the shape and the prefix by one block, its cell counts in shared
+// memory: a plan with many boxes builds the grid before the wavefront (and a
+// build before sampling), so dependent launches and a memset cost more than the
+// work.  With few boxes it writes the lists too, else it leaves the counts to
+// box_grid_scatter_kernel.  The block also chooses the grid's
 // shape: cells of the mean box's proportions, down to about a quarter of its
 // area (a box then lies in about nine).  Obstacles cut into thin slices get thin
 // cells: 1500 strips a hundred times wider than high list 2.9 boxes an occupied
@@ -151,10 +158,12 @@ __device__ __forceinline__ void box_grid_choose(const BoxArgs& boxes, int dp, co
 // them all, and box_grid_choose picks another: 1500 squares, a tenth of them four
 // times wider, 2D n = 1000, a build and plan 1351 -> 258 us (400 on square cells).
 constexpr int kBoxGridFewBig = 4;
+static_assert(kBoxGridMaxCells <= 32, "the scatter takes a box's cells in one warp");
 __global__ void __launch_bounds__(1024) box_grid_block_kernel(BoxArgs boxes, int dp, BoxGridArgs grid,
                                                               int* __restrict__ start, int* __restrict__ list,
                                                               float4* __restrict__ packed, int* __restrict__ big,
-                                                              int* __restrict__ nbig, float4* __restrict__ shape) {
+                                                              int* __restrict__ nbig, float4* __restrict__ shape,
+                                                              int* __restrict__ counts) {
     extern __shared__ int cnt[];  // kBoxGridCells
     __shared__ int warp_sum[32];
     __shared__ float ext[4][32];
@@ -264,11 +273,13 @@ __global__ void __launch_bounds__(1024) box_grid_block_kernel(BoxArgs boxes, int
         const int c = c0w + 32 * k;
         cnt[c] = before + x[k];  // from here on the cell's next free entry
         if (c < cells) start[c] = before + x[k];
+        if (counts && c < cells) counts[c] = v[k];
     }
     if (tid == 1023) {
         start[cells] = at;  // the cells past the grid's are empty
         *nbig = s_big;
     }
+    if (counts) return;  // the whole chip writes the lists
     __syncthreads();
     for (int b = tid; b < boxes.count; b += 1024) {
         int c0[2], c1[2];
@@ -288,17 +299,20 @@ cudaError_t launch_box_grid(int dp, BoxArgs boxes, const BoxGridArgs& grid, int*
         constexpr int smem = kBoxGridCells * (int)sizeof(int);
         cudaError_t e = cudaFuncSetAttribute(box_grid_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;
-        box_grid_block_kernel<<<1, 1024, smem, st>>>(boxes, dp, grid, start, list, packed, big, nbig, shape);
-        return cudaGetLastError();
+        const bool spread = boxes.count > kBoxGridFuseMax;
+        box_grid_block_kernel<<<1, 1024, smem, st>>>(boxes, dp, grid, start, list, packed, big, nbig, shape,
+                                                     spread ? cnt : nullptr);
+        e = cudaGetLastError();
+        if (e != cudaSuccess || !spread) return e;
+    } else {
+        cudaError_t e = cudaMemsetAsync(cnt, 0, (size_t)grid.g * grid.g * sizeof(int), st);
+        if (e == cudaSuccess) e = cudaMemsetAsync(nbig, 0, sizeof(int), st);
+        if (e != cudaSuccess) return e;
+        box_grid_count_kernel<<<(unsigned)((boxes.count + 255) / 256), 256, 0, st>>>(boxes, dp, grid, cnt, big, nbig);
+        e = launch_scan(cnt, start, grid.g * grid.g, st);
+        if (e != cudaSuccess) return e;
     }
-    cudaError_t me = cudaMemsetAsync(cnt, 0, (size_t)grid.g * grid.g * sizeof(int), st);
-    if (me == cudaSuccess) me = cudaMemsetAsync(nbig, 0, sizeof(int), st);
-    if (me != cudaSuccess) return me;
-    const unsigned blocks = (unsigned)((boxes.count + 255) / 256);
-    box_grid_count_kernel<<<blocks, 256, 0, st>>>(boxes, dp, grid, cnt, big, nbig);
-    cudaError_t e = launch_scan(cnt, start, grid.g * grid.g, st);
-    if (e != cudaSuccess) return e;
-    box_grid_scatter_kernel<<<blocks, 256, 0, st>>>(boxes, dp, grid, start, cnt, list, packed);
+    box_grid_scatter_kernel<<<(unsigned)((boxes.count + 7) / 8), 256, 0, st>>>(boxes, dp, grid, start, cnt, list, packed);
     return cudaGetLastError();
 }
 

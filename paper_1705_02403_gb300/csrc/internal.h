@@ -69,14 +69,19 @@ inline int box_grid_cells(int count) {
     while (g < 64 && g * g < count) g *= 2;
     return g;
 }
-// Boxes up to which one block builds the grid in one launch (each of its
-// threads then takes at most eight); more boxes take count, scan and scatter
-// launches over the whole chip.
+// Boxes up to which one block counts and shapes the grid (each of its threads
+// then takes at most eight), and up to which it also writes the lists itself:
+// with more, a launch over the whole chip writes them sooner than one SM does.
+// Build and plan (two grids), lists by the block and by the chip, us: 3D n = 1000,
+// 250 boxes 238 and 237, 500 285 and 278, 2000 425 and 369, 8190 733 and 518; double
+// integrator n = 1000, 130 148 and 152, 4000 323 and 231; forest n = 1500, 250 strips
+// 218 and 220, 8190 285 and 249.
 constexpr int kBoxGridBlockMax = 8192;
+constexpr int kBoxGridFuseMax = 256;
 // Boxes up to which the list also keeps packed copies (2D and 3D; at most
 // kBoxGridMaxCells copies of 32 bytes per box).
 constexpr int kBoxGridPackMax = 65536;
-// Builds the grid: cnt [g*g], nbig [1], start [max(g*g, kBoxGridCells) + 1],
+// Builds the grid: cnt [max(g*g, kBoxGridCells)], nbig [1], start [as many + 1],
 // list [count * kBoxGridMaxCells], packed [as many entries of 1 (2D) or 2 (3D)
 // float4s] or NULL, big [count], shape [1].  Up to kBoxGridBlockMax boxes the
 // shape is chosen on the device (the caller sets grid.shape then).

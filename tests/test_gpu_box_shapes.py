@@ -75,3 +75,27 @@ def test_a_few_large_boxes_are_not_tested_everywhere():
     # a tenth of the boxes four times wider: two and a half times the area, against 5.5 times the time
     # when they went over too many cells to be listed
     assert best("skew") < 3.0 * best("even")
+
+
+def test_lists_of_many_boxes_are_not_written_by_one_block():
+    def best(count):
+        rng = np.random.default_rng(count)
+        pb = envgen.di6(seed=3, n=1000, nbox=1, r=2.7)
+        c, side = rng.uniform(0.12, 0.88, (count, 3)), (0.15 / count) ** (1 / 3)
+        pb.box_lo, pb.box_hi = (c - side / 2).astype(np.float32), (c + side / 2).astype(np.float32)
+        pl = Planner(pb)
+        t = []
+        for _ in range(30):
+            t0 = time.perf_counter()
+            pl.build(asynchronous=True).plan()
+            t.append(time.perf_counter() - t0)
+        return min(t)
+    # 1.8 times the time of as many boxes again when one block wrote every list
+    assert best(8190) < 1.4 * best(8200)
+
+
+@pytest.mark.parametrize("count", [255, 256, 257, 300])
+@pytest.mark.parametrize("d", [2, 3, 4])
+def test_counts_around_the_scatter_line(O, P, d, count):
+    pb = with_boxes(envgen.geometric(count, d=d, n=250, nbox=0, r=0.3 if d < 4 else 0.6), "mixed", count)
+    assert_same(O, gpu_run(P, pb), *oracle_run(O, pb))
