@@ -1,8 +1,9 @@
 // BF16 x BF16 -> FP32 GEMM on the 5th-generation tensor cores (tcgen05) for
 // sm_103a, written with inline PTX:
 //   C[M, N] = A[M, K] . B[N, K]^T   (both operands K-major, row-major in memory)
-// For M <= 128 (fewer rows than half of a CTA pair's tile); more rows take the
-// CTA-pair kernel at the end of this file.
+// For M <= 128 (fewer rows than half of a CTA pair's tile) and where one wave of
+// deep tiles or an output by rows is faster so; more rows take the CTA-pair
+// kernel at the end of this file otherwise.
 //
 // One CTA of 128 threads computes a 128 x 128 tile of C (optionally a K-slice
 // of it, for split-K):

@@ -94,6 +94,25 @@ int pair_tile_n(int M, int N, int splits, int pairs, bool b_mn) {
     return best;
 }
 
+// Does a product of more than 128 rows run on single CTAs all the same?  per:
+// the K-blocks of a slice; rowwise: the output leaves row by row (BF16, or FP32
+// rows that do not start on 16 bytes), which costs a pair's two epilogues more
+// than four of a single CTA's tiles cost theirs.  With one wave of 128 x 128
+// tiles or less and deep K both kernels wait for the same loads, and a pair's
+// tiles only split them more finely.  One GB300, single CTAs against pairs, us:
+// BF16 513 x 20000 x 64 28 and 36, 8192 x 8192 x 64 141 and 170, 4096 x 4096 x 128
+// 38 and 45, 4096 x 512 x 512 94% of the pairs', FP32 2048 x 1003 x 256 the same,
+// 2048 x 128 x 8192 43 and 46; the other way BF16 8192 x 8192 x 512 61% faster on
+// pairs, 513 x 4096 x 512 8%, 1000 x 1003 x 256 29%, FP32 256 x 4096 x 1024 10%.
+// (Bits are equal.)
+bool single_ctas(int M, int N, int splits, int per, bool rowwise) {
+    const long long tiles_n = (N + kGemmBN - 1) / kGemmBN, tiles = (M + kGemmBM - 1) / kGemmBM * tiles_n * splits;
+    const int sms = device_sms();
+    if (tiles_n > 65535) return false;  // the grid's limit
+    if (tiles <= sms && per > 2048 / kGemmBK) return true;
+    return rowwise && 2 * tiles > sms && (tiles <= sms || per < 512 / kGemmBK);
+}
+
 // Sum of split-K partials [splits][M][N] plus the epilogue.
 __global__ void splitk_reduce_kernel(const float* __restrict__ part, int splits, int M, int N, int epilogue,
                                      const float* __restrict__ bias, float* __restrict__ C,
@@ -150,7 +169,9 @@ cudaError_t gemm_bf16_tn(int M, int N, int K, const __nv_bfloat16* A, const __nv
     cudaError_t e;
     // More than half a pair's rows: CTA pairs.  (M <= 128 would leave the
     // second CTA of every pair without rows: 4096 x 4096 x 128 rows.)
-    if (M > kGemmBM || a_mn || b_mn) {
+    // FP32 outputs leave a pair by TMA where their rows start on 16 bytes
+    const bool tma = g.epilogue != kEpiBiasReluBF16 && g.ldc % 4 == 0 && ((uintptr_t)g.C & 15) == 0;
+    if (a_mn || b_mn || (M > kGemmBM && !single_ctas(M, N, splits, per, !tma))) {
         const int pairs = std::max(1, device_sms() / 2);
         p.splits = splits; p.a_mn = a_mn; p.b_mn = b_mn;
         p.tile_n = pair_tile_n(M, N, splits, pairs, b_mn);
@@ -161,11 +182,9 @@ cudaError_t gemm_bf16_tn(int M, int N, int K, const __nv_bfloat16* A, const __nv
         if (e != cudaSuccess) return e;
         const long long items = (long long)p.tiles_m * p.tiles_n * splits;
         if (items > INT_MAX) return cudaErrorInvalidValue;
-        // FP32 outputs leave by TMA where their rows start on 16 bytes
         CUtensorMap tc;
         std::memset(&tc, 0, sizeof(tc));
-        p.tma_store = g.epilogue != kEpiBiasReluBF16 && g.ldc % 4 == 0 && ((uintptr_t)g.C & 15) == 0 &&
-                      make_out_map(&tc, g.C, g.epilogue == kEpiPartialF32 ? splits : 1, M, N, g.ldc) == cudaSuccess;
+        p.tma_store = tma && make_out_map(&tc, g.C, g.epilogue == kEpiPartialF32 ? splits : 1, M, N, g.ldc) == cudaSuccess;
         gemm_pair_bf16_kernel<<<2 * (int)std::min<long long>(items, pairs), kPairThreads, kPairSmem, st>>>(ta, tb, tc, p);
     } else {
         e = make_map(&ta, A, M, K, kGemmBM);
