@@ -23,8 +23,17 @@
  *    GMT_ERR_TIMEOUT and leaves the CUDA context usable.
  *  - There is no CPU fallback: every step of the path runs in the library's
  *    CUDA kernels.  Without a usable GPU, calls return GMT_ERR_CUDA.
- *  - Arithmetic: IEEE FP32 with round-to-nearest, no FMA contraction, IEEE
- *    division and square root in every decision, so results are reproducible.
+ *  - Arithmetic: IEEE FP32 with round-to-nearest, IEEE division and square root
+ *    in every decision, and no FMA contraction, with one exception, so results
+ *    are reproducible.  The exception: the all-pairs neighbour test of geometric
+ *    graphs in 2 to 4 dimensions, and the cell lists at the sizes where they
+ *    take its place, form the squared distance as fma(t_k, t_k, ...) with only
+ *    the second axis' square rounded.  Cell lists from 12000 nodes in 2D and
+ *    32768 in 3D (in a batch from 4096 in 2D), where the cells around a node
+ *    hold at most a quarter of the domain, round every square.  A pair whose
+ *    distance is within one rounding of r may be an edge in the one and not in
+ *    the other: so may a 2D query of 4096 to 11999 nodes differ between
+ *    gmt_plan_batch and gmt_build_graph at such a pair.
  *  - Handles are not thread-safe: one handle must not be used by two calls
  *    at once (on any streams).
  */
@@ -361,7 +370,10 @@ void gmt_batch_free(gmt_batch* batch);
  * re-run (results identical to a fresh plan).  A worker thread admits queued
  * requests to free slots (CUDA streams with their own plan scratch) as soon as
  * they free up, so requests overlap on the device; a session has at most one
- * request running.  Sessions are admitted against a device-memory budget. */
+ * request running.  Sessions are admitted against a device-memory budget.
+ * While a plan is in flight the worker polls its completion word, with a yield
+ * in between and without a sleep until 2 ms have passed without an event: a
+ * busy server takes up to one host core. */
 typedef struct {
     int32_t slots;         /* concurrent requests (streams), >= 1 */
     int32_t cluster;       /* CTAs per plan: 0/1 = one CTA, 2..16 = a cluster */

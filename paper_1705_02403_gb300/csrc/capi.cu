@@ -465,7 +465,8 @@ gmt_status build_impl(const gmt_space* space, const gmt_boxes* boxes, const floa
            "append kernel");
     LAUNCH(g->mark(gmt_graph::kSample, 1, st), "event");
     // neighbour test: cell list for 2D/3D geometric graphs with a small radius
-    // (or when forced), else all pairs; both give the same CSR
+    // (or when forced), else all pairs; both give the same CSR with pairs_sum,
+    // else all but pairs within one rounding of the radius
     CellGrid cg;
     bool cells_pay = false;
     bool cells = make_cell_grid(g->kind, g->d, space->lo, space->hi, g->r, g->N, false, &cg, &cells_pay);

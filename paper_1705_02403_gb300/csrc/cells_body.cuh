@@ -3,9 +3,10 @@
 // precomputed in Section V-A), not a change of the method.  Nodes are
 // counting-sorted by grid cell; a row's candidates are the nodes of the 3^d
 // cells around its own, which lie in 3^(d-1) runs of consecutive cells along
-// axis 0.  Every candidate takes the same FP32 edge predicate as the all-pairs
-// build, and each row's columns come out in ascending order, so the CSR is the
-// same bits.
+// axis 0.  Every candidate takes an FP32 edge predicate, and each row's columns
+// come out in ascending order.  With pairs_sum the predicate is the all-pairs
+// tiles' and the CSR is the same bits as theirs; without it every square is
+// rounded (sq_dist), and a pair within one rounding of the radius may differ.
 //
 // One CTA per cell (a cell tile): the cell's candidates (the same for every
 // row of the cell) are loaded into shared memory once, with their coordinates,

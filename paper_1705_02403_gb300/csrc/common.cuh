@@ -5,7 +5,8 @@
 // library is compiled with -fmad=false -prec-div=true -prec-sqrt=true
 // -ftz=false, and every expression below is written in the evaluation order
 // the planner's specification fixes (left to right), so results are
-// reproducible bit for bit.
+// reproducible bit for bit.  (The all-pairs test of 2 to 4 dimensions writes
+// FMAs out: sq_dist_pairs.)
 #pragma once
 
 #include <cstdint>

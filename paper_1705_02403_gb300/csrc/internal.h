@@ -221,7 +221,9 @@ cudaError_t launch_cells_count(const SpaceArgs& s, const float* X, const CellGri
 // cell_cnt returns to zero.
 cudaError_t launch_cells_scatter(int N, const int* cell_of, const int* cell_start, int* cell_cnt, int* sorted,
                                  cudaStream_t st);
-// fill = false: out_count[v] = neighbours of v, max_deg = their maximum; fill
+// fill = false: out_count[v] = neighbours of v, max_deg = the longest row among
+// the cells whose candidates exceed a tile (0 if none: other rows are not
+// bounded by the fill's list); fill
 // = true: columns (ascending) and costs of every row at row[v]; a row longer
 // than kCellList sets *overflow and writes nothing; an edge count above cap (>
 // 0) writes nothing at all.

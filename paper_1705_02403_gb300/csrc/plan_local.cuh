@@ -43,9 +43,6 @@
 // thousand neighbours a node) 0.407 -> 0.256, double integrator n = 4096
 // 0.110 -> 0.078, Dubins airplane n = 5000 with 1500 boxes 0.363 -> 0.251
 // (0.163 since the box grid's cells have the boxes' proportions).
-// The same body on a cooperative grid of 38 to 152 CTAs (lists of changes and
-// marks through L2, a polled word per CTA as the barrier) was slower on all of
-// these but the 6D graph (equal): its two barriers cost 4-5 us an iteration.
 //
 // Decisions, trees, counters and paths are those of plan_body_fused (which
 // remains for graphs whose replica does not fit).
@@ -250,7 +247,7 @@ __device__ __forceinline__ bool plan_body_local(const PlanArgs& A, const Team& t
     float* const own = reinterpret_cast<float*>(smem + L.own);
     float* const xs = reinterpret_cast<float*>(smem + L.xs);
     unsigned char* const sent = smem + L.sent;
-    unsigned* const claim = reinterpret_cast<unsigned*>(smem + L.claim);  // grid: A.g_claim instead
+    unsigned* const claim = reinterpret_cast<unsigned*>(smem + L.claim);
     unsigned* const tree = reinterpret_cast<unsigned*>(smem + L.tree);
     unsigned* const goalbits = reinterpret_cast<unsigned*>(smem + L.goal);
     unsigned short* const newl = reinterpret_cast<unsigned short*>(smem + L.lists);
