@@ -369,8 +369,8 @@ def run_gpu(args, rank, world, local_rank):
         line["serving"] = bench_serving(local_rank)
         line["dubins"] = bench_dubins(dev, flush)
         line["learned"] = bench_learned()
-        line["gpu_launches_extras"] = ("batched: 7 launches per group per batch (replayed CUDA graph); serving: 3 per "
-                                       "request; dubins: 7-8 per build, 1 per plan")
+        line["gpu_launches_extras"] = ("batched: 7 launches per group per batch (replayed CUDA graph); serving: 2 per "
+                                       "request; dubins: 6-7 per build, 2-3 per plan")
     if rank == 0 and world == 1 and not args.no_cpu_baseline:
         nb = min(args.steps, 8 if args.workload == "di6" else 20)
         seeds_cpu = [seeds[args.warmup + j] for j in range(nb)]
