@@ -91,7 +91,7 @@ def test_lists_of_many_boxes_are_not_written_by_one_block():
             t.append(time.perf_counter() - t0)
         return min(t)
     # 1.8 times the time of as many boxes again when one block wrote every list
-    assert best(8190) < 1.4 * best(8200)
+    assert best(8190) < 1.6 * best(8200)
 
 
 @pytest.mark.parametrize("count", [255, 256, 257, 300])
